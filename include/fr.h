@@ -388,8 +388,9 @@ fr_status esdirk_step(fr_ctx* ctx, const fr_tableau* tab, double dt, double* q_i
  * double-float kernels, same operand size), f32][kernel trace,
  * volume residual, volume JVP][P = p+1]: for P >= 2 the elements per CTA
  * of the one-launch-per-bucket kernels, 0 = default (as many whole elements
- * as fit 256 threads; a value whose elements exceed 256 threads also falls
- * back to it; the multi-bucket launch always fills its 256-thread blocks);
+ * as fit 256 threads, or on small meshes as few whole warps as give every SM
+ * four CTAs; a value whose elements exceed 256 threads also falls back to it;
+ * the multi-bucket launch always uses the default);
  * the slot P = 0 holds the multi-bucket choice of that precision and kernel
  * (0 undecided: one launch over all buckets while the mesh's solution points
  * fit in 8 full-occupancy waves of the GPU, else one per bucket; 1 one launch

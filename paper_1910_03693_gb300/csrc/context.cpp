@@ -184,7 +184,7 @@ fr_status rebuild_work_table(fr_ctx* c) {
   std::vector<std::pair<double, WorkItem>> items;
   for (size_t bi = 0; bi < c->buckets.size(); ++bi) {
     const Bucket& b = c->buckets[bi];
-    const int P = b.p + 1, e = epb_multi(c->nd, P);
+    const int P = b.p + 1, e = epb_multi(c->nd, P, mesh_threads(c));
     for (int f = 0; f < b.count; f += e) {
       const int ne = std::min(e, b.count - f);
       items.push_back({ne * element_weight(c->epb_tab[0][0][1], ipow(P, c->nd), P), WorkItem{(int32_t)bi, (int32_t)f}});
@@ -464,6 +464,10 @@ static fr_status create_impl(const fr_mesh_desc* m, const fr_physics* ph, const 
     }
   }
   FR_CUDA(cudaGetDevice(&c->device));
+  if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess || c->sms <= 0) {
+    cudaGetLastError();
+    c->sms = 152;
+  }
   c->nvt = c->visc ? (1 + nd) * c->nv : c->nv;
 
   // basis and mortar tables

@@ -86,22 +86,15 @@ static inline unsigned nblocks(int64_t n, int bs) { return (unsigned)((n + bs - 
 // ---------------------------------------------------------------------------
 static inline int nsp_of(int nd, int P) { return nd == 2 ? P * P : P * P * P; }
 
-// elements per CTA: tuned value, else as many whole elements as fit 256 threads
+static inline unsigned sm_count(const fr_ctx* c) { return (unsigned)c->sms; }
+
+// elements per CTA: tuned value, else as many whole elements as fit the
+// threads a CTA of this mesh should use
 static inline int epb_for(fr_ctx* c, int prec, int kind, int P) {
   const int t = c->epb_tab[prec][kind][P];
   const int nsp = nsp_of(c->nd, P);
-  const int dflt = nsp >= 256 ? 1 : 256 / nsp;
-  return (t > 0 && t * nsp <= 256) ? t : dflt;
-}
-
-// Elements per tile of the multi-bucket launch: as many whole elements as fill
-// its 256-thread blocks (the tuned per-bucket values size separate launches,
-// whose block is e * n_sp threads; a small one here would leave most of the
-// block idle).
-static inline unsigned sm_count(fr_ctx* c) {
-  static int n = 0;   // one device per process here; queried once
-  if (n <= 0) cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, c->device);
-  return n > 0 ? (unsigned)n : 152u;
+  if (t > 0 && t * nsp <= 256) return t;
+  return std::max(1, mesh_threads(c) / nsp);
 }
 
 // One launch over all buckets for this precision and kernel kind: the master
@@ -181,9 +174,11 @@ static void launch_traces(fr_ctx* c, const T* q, T* trace, cudaStream_t s) {
   if (items) {
     TraceMulti<T> m;
     size_t smem = 0;
+    int block = 32;
     for (size_t i = 0; i < c->buckets.size(); ++i) {
       const Bucket& b = c->buckets[i];
-      const int P = b.p + 1, e = epb_multi(ND, P);
+      const int P = b.p + 1, e = epb_multi(ND, P, mesh_threads(c));
+      block = std::max(block, (e * nsp_of(ND, P) + 31) / 32 * 32);
       m.b[i] = trace_args<T, ND, VISC>(c, b, q, trace);
       m.P[i] = P;
       m.epb[i] = e;
@@ -195,9 +190,9 @@ static void launch_traces(fr_ctx* c, const T* q, T* trace, cudaStream_t s) {
     static size_t configured = 0;
     ensure_smem(kern, smem, configured);
     int per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, smem);
     const unsigned grid = (unsigned)std::max(1, std::min(m.n_items, (int)(std::max(per_sm, 1) * sm_count(c))));
-    FR_LAUNCH_BF(c, name, s, nb, nfl, kern<<<grid, 256, smem, s>>>(m));
+    FR_LAUNCH_BF(c, name, s, nb, nfl, kern<<<grid, block, smem, s>>>(m));
     return;
   }
   for (const auto& b : c->buckets) {
@@ -272,9 +267,11 @@ static void launch_vols(fr_ctx* c, const T* q, const T* v, T* out, cudaStream_t 
   if (items) {
     VolMulti<T> m;
     size_t smem = 0;
+    int block = 32;
     for (size_t i = 0; i < c->buckets.size(); ++i) {
       const Bucket& b = c->buckets[i];
-      const int P = b.p + 1, e = epb_multi(ND, P);
+      const int P = b.p + 1, e = epb_multi(ND, P, mesh_threads(c));
+      block = std::max(block, (e * nsp_of(ND, P) + 31) / 32 * 32);
       m.b[i] = vol_args<T>(c, b, q, v, out, out_neg64, out64);
       m.P[i] = P;
       m.epb[i] = e;
@@ -286,9 +283,9 @@ static void launch_vols(fr_ctx* c, const T* q, const T* v, T* out, cudaStream_t 
     static size_t configured = 0;
     ensure_smem(kern, smem, configured);
     int per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, smem);
     const unsigned grid = (unsigned)std::max(1, std::min(m.n_items, (int)(std::max(per_sm, 1) * sm_count(c))));
-    FR_LAUNCH_BF(c, name, s, nb, nfl, kern<<<grid, 256, smem, s>>>(m));
+    FR_LAUNCH_BF(c, name, s, nb, nfl, kern<<<grid, block, smem, s>>>(m));
     return;
   }
   for (const auto& b : c->buckets) {
@@ -308,61 +305,76 @@ static void launch_vols(fr_ctx* c, const T* q, const T* v, T* out, cudaStream_t 
   }
 }
 
+// The face groups of the mesh as one launch's group table: mixed-degree groups
+// first (their CTAs run longest), then conforming ones, then boundaries; faces
+// a CTA as many as its threads hold, fewer (whole warps idle) on meshes whose
+// face points would otherwise leave SMs without a CTA (see spread_threads).
+// Returns the number of blocks.
+template <typename T, int ND>
+static int face_groups(fr_ctx* c, FaceMulti<T>& m) {
+  int64_t points = 0;
+  for (const auto& g : c->fgroups) points += (int64_t)g.n * ipow(g.pm + 1, ND - 1);
+  for (const auto& g : c->bgroups) points += (int64_t)g.n * ipow(g.p + 1, ND - 1);
+  const int threads = spread_threads(points, kFaceThreads, c->sms);
+  int blocks = 0;
+  m.ng = 0;
+  auto add = [&](const FaceRec* recs, const BndRec* brecs, int n, int Pm, int Ps, int kind) {
+    FaceGroupRef& r = m.g[m.ng++];
+    const int nfp = ipow(Pm, ND - 1);
+    r.recs = recs;
+    r.brecs = brecs;
+    r.n = n;
+    r.Pm = Pm;
+    r.Ps = Ps;
+    r.kind = kind;
+    r.fb = std::max(1, threads / nfp);
+    r.block0 = blocks;
+    blocks += (int)nblocks(n, r.fb);
+  };
+  for (const auto& g : c->fgroups)
+    if (g.pm != g.ps) add(g.d_recs, nullptr, g.n, g.pm + 1, g.ps + 1, 0);
+  for (const auto& g : c->fgroups)
+    if (g.pm == g.ps) add(g.d_recs, nullptr, g.n, g.pm + 1, g.ps + 1, 0);
+  for (const auto& g : c->bgroups) add(nullptr, g.d_recs, g.n, g.p + 1, g.p + 1, g.kind);
+  return blocks;
+}
+
 template <typename T, int ND, bool VISC, int MODE, bool DIAG = false>
 static void launch_faces(fr_ctx* c, const T* trq, const T* trv, cudaStream_t s) {
+  FaceMulti<T> m;
+  const int blocks = face_groups<T, ND>(c, m);
+  if (blocks == 0) return;
+  for (const auto& b : c->buckets) m.geo[b.p + 1] = geo_view<T>(c, b.p);
+  m.trq = trq;
+  m.trv = trv;
+  m.fout = (T*)c->d_fout;
+  m.basis = basis_ptr<T>(c);
+  m.mortar = mortar_ptr<T>(c, 0, 0);
+  m.gamma = (T)c->phys.gamma;
+  m.mu = (T)c->phys.mu;
+  m.kappa = (T)c->phys.kappa;
+  for (int v = 0; v < 5; ++v) m.qinf[v] = (T)c->phys.q_inf[v];
+  m.nvt = c->nvt;
+  m.flux = c->phys.flux;
+  m.gate = c->gate;
+  double nb = 0.0, nfl = 0.0;
   for (const auto& g : c->fgroups) {
-    FaceArgs<T> a;
-    a.gate = c->gate;
-    a.recs = g.d_recs;
-    a.trq = trq;
-    a.trv = trv;
-    a.fout = (T*)c->d_fout;
-    a.scratch = (T*)c->d_scratch;
-    a.basis = basis_ptr<T>(c);
-    a.mortar = g.pm != g.ps ? mortar_ptr<T>(c, g.pm + 1, g.ps + 1) : nullptr;
-    a.geo_m = geo_view<T>(c, g.pm);
-    a.geo_s = geo_view<T>(c, g.ps);
-    a.gamma = (T)c->phys.gamma;
-    a.mu = (T)c->phys.mu;
-    a.kappa = (T)c->phys.kappa;
-    a.flux = c->phys.flux;
-    a.n = g.n;
-    a.Pm = g.pm + 1;
-    a.Ps = g.ps + 1;
-    a.nvt = c->nvt;
-    a.scratch_base = g.scratch_base;
-    const int64_t nm = (int64_t)g.n * ipow(a.Pm, ND - 1);
-    FR_LAUNCH_BF(c, MODE == 1 ? kname<T>("face_jvp_f64", "face_jvp_f32", "face_jvp_df")
-                              : kname<T>("face_res_f64", "face_res_f32", "face_res_df"),
-                 s, (double)nm * values_face(ND, VISC, MODE == 1) * sizeof(T),
-                 MODE == 1 ? 0.0 : (double)nm * flops_face(ND, VISC, DIAG),
-                 face_kernel<T, ND, VISC, MODE, DIAG><<<nblocks(nm, 128), 128, 0, s>>>(a));
-    if (g.pm != g.ps) {
-      const int64_t ns = (int64_t)g.n * ipow(a.Ps, ND - 1);
-      FR_LAUNCH(c, "mortar_project", s,
-                mortar_project_kernel<T, ND, VISC, MODE><<<nblocks(ns, 128), 128, 0, s>>>(a));
-    }
+    const int64_t nm = (int64_t)g.n * ipow(g.pm + 1, ND - 1);
+    nb += (double)nm * values_face(ND, VISC, MODE == 1) * sizeof(T);
+    if (MODE == 0) nfl += (double)nm * flops_face(ND, VISC, DIAG);
   }
-  for (const auto& g : c->bgroups) {
-    BndArgs<T> a;
-    a.gate = c->gate;
-    a.recs = g.d_recs;
-    a.trq = trq;
-    a.trv = trv;
-    a.fout = (T*)c->d_fout;
-    a.basis = basis_ptr<T>(c);
-    a.geo = geo_view<T>(c, g.p);
-    a.gamma = (T)c->phys.gamma;
-    a.mu = (T)c->phys.mu;
-    a.kappa = (T)c->phys.kappa;
-    a.flux = c->phys.flux;
-    for (int v = 0; v < 5; ++v) a.qinf[v] = (T)c->phys.q_inf[v];
-    a.n = g.n;
-    a.P = g.p + 1;
-    a.kind = g.kind;
-    const int64_t nm = (int64_t)g.n * ipow(a.P, ND - 1);
-    FR_LAUNCH(c, "boundary", s, bnd_kernel<T, ND, VISC, MODE><<<nblocks(nm, 128), 128, 0, s>>>(a));
+  size_t smem = 0;
+  for (int i = 0; i < m.ng; ++i) {
+    const FaceGroupRef& g = m.g[i];
+    if (g.Pm != g.Ps)
+      smem = std::max(smem, (size_t)g.fb * MixedFace<ND, VISC, MODE>::stride(ipow(g.Pm, ND - 1), ipow(g.Ps, ND - 1)) * sizeof(T));
   }
+  auto kern = face_kernel<T, ND, VISC, MODE, DIAG>;
+  static size_t configured = 46 * 1024;   // static shared memory besides: 2 KB
+  ensure_smem(kern, smem, configured);
+  FR_LAUNCH_BF(c, MODE == 1 ? kname<T>("face_jvp_f64", "face_jvp_f32", "face_jvp_df")
+                            : kname<T>("face_res_f64", "face_res_f32", "face_res_df"),
+               s, nb, nfl, kern<<<blocks, kFaceThreads, smem, s>>>(m));
 }
 
 template <typename T, int ND, bool VISC, bool DIAG = false>
@@ -442,7 +454,7 @@ template <typename T, int ND, bool VISC>
 static void launch_ctraces(fr_ctx* c, const T* q, T* out, cudaStream_t s) {
   constexpr int NV = ND + 2, NF = 2 * ND, CT = VISC ? 2 * NV : NV;
   for (const auto& b : c->buckets) {
-    const int P = b.p + 1, e = epb_multi(ND, P);
+    const int P = b.p + 1, e = epb_multi(ND, P, mesh_threads(c));
     CTraceArgs<T> a;
     a.gate = c->gate;
     a.q = q;

@@ -108,10 +108,25 @@ struct FusedNbr {
   int32_t code;    // bits 0-7: orientation code (this side's point -> the neighbour's); bit 8: this side is the master
 };
 
-// Elements per tile of the multi-bucket launch: as many as fill a 256-thread block.
-inline int epb_multi(int nd, int P) {
+// Threads a CTA should use when a pass over the mesh has `points` points (one
+// thread each) and a CTA holds at most `full`: `full` once that gives every SM
+// four CTAs, below that as few whole warps as keep four CTAs an SM.  On a small
+// mesh full CTAs occupy a few SMs and leave the rest idle, and an SM's FP64
+// pipe (2 FMAs a clock: 16 clocks a warp instruction) is shared by the warps on
+// it, so the pass takes as long as the fullest SM (256 quadrilaterals, p = 2:
+// 10 CTAs of 252 threads, the FP64 volume pass 11.9 us; 86 CTAs of 27: 9.0 us).
+constexpr int kSpreadPerSm = 4;
+inline int spread_threads(int64_t points, int full, int sms) {
+  const int64_t per = (points + (int64_t)kSpreadPerSm * sms - 1) / ((int64_t)kSpreadPerSm * sms);
+  const int64_t warps = (per + 31) / 32 * 32;
+  return (int)(warps < full ? warps : full);
+}
+
+// Elements per tile of the multi-bucket launch (the tuned per-bucket values
+// size separate launches): as many as the CTA's threads hold.
+inline int epb_multi(int nd, int P, int threads = 256) {
   const int nsp = nd == 2 ? P * P : P * P * P;
-  return nsp >= 256 ? 1 : 256 / nsp;
+  return nsp >= threads ? 1 : threads / nsp;
 }
 
 // Element weight of the multi-bucket work table (tuning slot [0][0][P = 1]):
@@ -142,6 +157,7 @@ struct fr_ctx {
   bool diag = false;        // diag_mesh and the diagonal-metric kernels enabled
   frgb::PhysParams phys{};
   int device = 0;
+  int sms = 152;            // the device's SM count (queried at creation)
   // host mesh
   std::vector<double> nodes;
   std::vector<int32_t> nbr;
@@ -272,6 +288,8 @@ struct fr_ctx {
 };
 
 namespace frgb {
+// threads a CTA of the element kernels should use on this mesh
+inline int mesh_threads(const fr_ctx* c) { return spread_threads(c->n_dof / c->nv, 256, c->sms); }
 void clear_work_cache(fr_ctx* c);
 fr_status rebuild_work_table(fr_ctx* c);
 void clear_graphs(fr_ctx* c);

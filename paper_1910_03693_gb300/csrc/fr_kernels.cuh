@@ -316,24 +316,64 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) trace_multi_kerne
 }
 
 // ---------------------------------------------------------------------------
-// Interior face kernel: common flux on the mortar (Pm points per direction).
-// One thread per (face, mortar point).  MODE 0: residual; 1: JVP.
+// Face kernel: every face of the mesh in one launch.  Faces come in groups:
+// interior ones of one degree pair (Pm >= Ps: the master's mortar has Pm
+// points per direction), boundary ones of one degree and kind.  A CTA takes
+// `fb` whole faces of one group, one thread per mortar (or boundary) point.
+//
+// Mixed-degree groups (Pm > Ps): the slave's traces and lifting coefficients
+// of the CTA's faces are staged in shared memory, every thread interpolates
+// them to its mortar point, and after the flux the mortar values go back
+// through the same shared memory to the L2 projection onto the slave's points.
+// One launch a face pass: with a launch per group (and one more for the
+// projection of each mixed group) a mesh of degrees 1..4 took 10 face and 6
+// projection launches one after the other, each a fraction of a wave: at 1600
+// quadrilaterals 24 us a group for the FP64 JVP, bound by a few SMs' FP64
+// pipes, against one launch that spreads all faces over the chip (measured: 300
+// us of face launches a product -> 37 us; curved O-grid of 12,288 elements,
+// degrees 1..4: FP32 JVP faces 323 -> 68 us, FP64 Roe residual faces 815 -> 442
+// us).  Staging the slave replaces one dependent global load per slave point
+// and component of every mortar thread.
+// MODE 0: residual; 1: JVP.
 // ---------------------------------------------------------------------------
+constexpr int kMaxFaceGroups = kMaxDeg * kMaxDeg + 2 * kMaxDeg;   // degree pairs, boundary kinds by degree
+constexpr int kFaceThreads = 128;
+
+struct FaceGroupRef {
+  const FaceRec* recs;     // interior groups
+  const BndRec* brecs;     // boundary groups
+  int n, block0;           // faces; the group's first block
+  int Pm, Ps, kind, fb;    // kind: 0 interior, else the boundary kind; faces a CTA
+};
+
 template <typename T>
-struct FaceArgs {
-  const FaceRec* recs;
-  const T* trq;        // traces of q
-  const T* trv;        // traces of the tangent (JVP)
+struct FaceMulti {
+  FaceGroupRef g[kMaxFaceGroups];
+  GeoView<T> geo[kPM + 1];          // by P
+  const T* trq;                     // traces of q
+  const T* trv;                     // traces of the tangent (JVP)
   T* fout;
-  T* scratch;          // mixed-degree groups: [face][comp][NFPm]
   const BasisTab<T>* basis;
-  const MortarTab<T>* mortar;   // Pm -> Ps tables (nullptr when Pm == Ps)
-  GeoView<T> geo_m, geo_s;
+  const MortarTab<T>* mortar;       // table of (Pm, Ps) at Pm (kPM + 1) + Ps
   T gamma, mu, kappa;
-  int n, Pm, Ps, nvt;
-  int flux;            // common inviscid flux: 0 Rusanov, 1 Roe
-  int64_t scratch_base;
-  const int* gate = nullptr;   // see gate_closed
+  T qinf[5];
+  int ng, nvt;
+  int flux;                         // common inviscid flux: 0 Rusanov, 1 Roe
+  const int* gate = nullptr;        // see gate_closed
+};
+
+// Shared memory of one face of a mixed group, in values: the slave's staged
+// traces (of q, then of the tangent) and lifting coefficients, reused for the
+// mortar values of the projection.
+template <int ND, bool VISC, int MODE>
+struct MixedFace {
+  static constexpr int NV = ND + 2;
+  static constexpr int NT = VISC ? NV * (1 + ND) : NV;                     // trace components
+  static constexpr int NO = VISC ? (MODE == 1 ? 3 * NV : 2 * NV) : NV;     // face-output components
+  __host__ __device__ static int stride(int NFPm, int NFPs) {
+    const int in = ((MODE == 1 ? 2 : 1) * NT + (VISC ? ND : 0)) * NFPs, out = NO * NFPm;
+    return in > out ? in : out;
+  }
 };
 
 template <int ND, typename S, typename T>
@@ -346,57 +386,94 @@ __device__ __forceinline__ void load_trace_pt(const T* trq, const T* trv, int64_
   }
 }
 
-// value of the slave's trace component at mortar point u (slave axes, Pm grid)
-template <int ND, typename S, typename T>
-__device__ __forceinline__ void slave_at_mortar(const FaceArgs<T>& a, int64_t base, int comp0,
-                                                int ncomp, int u, S* out) {
-  const int Ps = a.Ps, Pm = a.Pm;
-  const int NFPs = ND == 2 ? Ps : Ps * Ps;
-  if (Pm == Ps) {
-    load_trace_pt<ND>(a.trq, a.trv, base, comp0, ncomp, NFPs, u, out);
-    return;
-  }
-  const int ua = u % Pm, ub = ND == 2 ? 0 : u / Pm;
-  for (int c = 0; c < ncomp; ++c) set_scalar(out[c], T(0), T(0));
+// Interpolation to mortar point (ua, ub) of NC components staged at sq (and
+// their tangents at sv, JVP) as [component][NFPs].
+template <int ND, int NC, int MODE, typename S, typename T>
+__device__ __forceinline__ void staged_at_mortar(const T* sq, const T* sv, const MortarTab<T>& mt, int Ps, int NFPs,
+                                                 int ua, int ub, S* out) {
+#pragma unroll
+  for (int c = 0; c < NC; ++c) set_scalar(out[c], T(0), T(0));
   for (int bb = 0; bb < (ND == 2 ? 1 : Ps); ++bb) {
-    const T wb = ND == 2 ? T(1) : a.mortar->I[ub][bb];
+    const T wb = ND == 2 ? T(1) : mt.I[ub][bb];
     for (int aa = 0; aa < Ps; ++aa) {
-      const T w = a.mortar->I[ua][aa] * wb;
+      const T w = mt.I[ua][aa] * wb;
       const int pt = aa + Ps * bb;
-      for (int c = 0; c < ncomp; ++c) {
-        T v = a.trq[base + (int64_t)(comp0 + c) * NFPs + pt];
-        T dv = a.trv ? a.trv[base + (int64_t)(comp0 + c) * NFPs + pt] : T(0);
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
         S x;
-        set_scalar(x, v, dv);
+        set_scalar(x, sq[c * NFPs + pt], MODE == 1 ? sv[c * NFPs + pt] : T(0));
         out[c] = out[c] + w * x;
       }
     }
   }
 }
 
-template <int ND, typename T>
-__device__ __forceinline__ void slave_coef_at_mortar(const FaceArgs<T>& a, const FaceRec& r, int u,
-                                                     T* cS) {
-  // c = g_s'(face) S_d[j] / |J| at the slave's own points, interpolated to the mortar
-  const int Ps = a.Ps, Pm = a.Pm;
-  const int ds = r.sf >> 1, ss = r.sf & 1;
-  const T g = a.basis[Ps].dgf[ss];
-  for (int j = 0; j < ND; ++j) cS[j] = T(0);
-  if (Pm == Ps) {
-    const T gJ = g * geo_face(a.geo_s, r.se, r.sf, ND * ND + 1, u);
-    for (int j = 0; j < ND; ++j) cS[j] = gJ * geo_face(a.geo_s, r.se, r.sf, ds * ND + j, u);
-    return;
-  }
-  const int ua = u % Pm, ub = ND == 2 ? 0 : u / Pm;
-  for (int bb = 0; bb < (ND == 2 ? 1 : Ps); ++bb) {
-    const T wb = ND == 2 ? T(1) : a.mortar->I[ub][bb];
-    for (int aa = 0; aa < Ps; ++aa) {
-      const T w = a.mortar->I[ua][aa] * wb;
-      const int pt = aa + Ps * bb;
-      const T gJ = g * geo_face(a.geo_s, r.se, r.sf, ND * ND + 1, pt);
-      for (int j = 0; j < ND; ++j) cS[j] += w * (gJ * geo_face(a.geo_s, r.se, r.sf, ds * ND + j, pt));
+// Outputs of one side of a face at its point t: the transformed common flux,
+// and (NS) the jump q^com - q.
+template <int ND, bool VISC, int MODE, typename S, typename T>
+__device__ __forceinline__ void store_face_side(T* o, int NFP, int t, T sg, const S* Fn, const S* qc, const S* q) {
+  constexpr int NV = ND + 2;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    S x = sg * Fn[v];
+    o[v * NFP + t] = MODE == 1 ? tangent(x) : value(x);
+    if (VISC) {
+      S dq = qc[v] - q[v];
+      o[(NV + v) * NFP + t] = value(dq);
+      if (MODE == 1) o[(2 * NV + v) * NFP + t] = tangent(dq);
     }
   }
+}
+
+// Boundary point: ghost state (wall / far field), common flux against it.
+template <typename T, int ND, bool VISC, int MODE>
+__device__ __forceinline__ void boundary_point(const FaceMulti<T>& m, const FaceGroupRef& g, const BndRec& r, int t) {
+  constexpr int NV = ND + 2;
+  using S = typename std::conditional<MODE == 1, Dual<T>, T>::type;
+  const int NFP = ND == 2 ? g.Pm : g.Pm * g.Pm;
+  const GeoView<T>& geo = m.geo[g.Pm];
+  const int d = r.mf >> 1, s = r.mf & 1;
+  const T* trv = MODE == 1 ? m.trv : nullptr;
+  S qM[NV], qG[NV];
+  load_trace_pt<ND>(m.trq, trv, r.mt, 0, NV, NFP, t, qM);
+  ghost_state<ND>(qM, g.kind, m.qinf, qG);
+  T A[ND], n[ND];
+  const T sg = s ? T(1) : T(-1);
+  const T absA = geo_face(geo, r.me, r.mf, ND * ND + 2 + d, t);
+  const T inv_absA = geo_face(geo, r.me, r.mf, ND * ND + 2 + ND + d, t);
+#pragma unroll
+  for (int j = 0; j < ND; ++j) {
+    A[j] = sg * geo_face(geo, r.me, r.mf, d * ND + j, t);
+    n[j] = A[j] * inv_absA;
+  }
+  S Fn[NV];
+  common_flux<ND>(m.flux, qM, qG, n, absA, m.gamma, Fn);
+  S qc[NV];
+  if (VISC) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) qc[v] = T(0.5) * (qM[v] + qG[v]);
+    T cM[ND];
+    const T gJ = m.basis[g.Pm].dgf[s] * geo_face(geo, r.me, r.mf, ND * ND + 1, t);
+#pragma unroll
+    for (int j = 0; j < ND; ++j) cM[j] = gJ * geo_face(geo, r.me, r.mf, d * ND + j, t);
+    S GM[ND][NV], Gc[ND][NV];
+    load_trace_pt<ND>(m.trq, trv, r.mt, NV, ND * NV, NFP, t, &GM[0][0]);
+#pragma unroll
+    for (int j = 0; j < ND; ++j)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) Gc[j][v] = GM[j][v] + cM[j] * (qc[v] - qM[v]);
+    S fv[ND][NV];
+    flux_viscous<ND>(qc, Gc, m.gamma, m.mu, m.kappa, fv);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      S acc = szero<S>();
+#pragma unroll
+      for (int j = 0; j < ND; ++j) acc = acc + fv[j][v] * A[j];
+      if (g.kind == -1 && v == NV - 1) acc = szero<S>();   // adiabatic wall
+      Fn[v] = Fn[v] - acc;
+    }
+  }
+  store_face_side<ND, VISC, MODE>(m.fout + r.mo, NFP, t, sg, Fn, qc, qM);
 }
 
 // DIAG: both sides have diagonal metrics (axis-aligned affine elements), so the
@@ -408,252 +485,187 @@ __device__ __forceinline__ void slave_coef_at_mortar(const FaceArgs<T>& a, const
 // double-float viscous instance spills 160 bytes at the cap and still streams
 // its traces faster than at three CTAs (252 -> 234 us at 32^3).
 template <typename T, int ND, bool VISC, int MODE, bool DIAG = false>
-__global__ void __launch_bounds__(128, (is_dfloat<T>::value || sizeof(T) == 4) ? 4 : 1) face_kernel(FaceArgs<T> a) {
+__global__ void __launch_bounds__(kFaceThreads, (is_dfloat<T>::value || sizeof(T) == 4) ? 4 : 1)
+    face_kernel(const __grid_constant__ FaceMulti<T> m) {
   constexpr int NV = ND + 2;
-  if (gate_closed(a.gate)) return;
+  using MF = MixedFace<ND, VISC, MODE>;
   using S = typename std::conditional<MODE == 1, Dual<T>, T>::type;
-  const int Pm = a.Pm;
-  const int NFPm = ND == 2 ? Pm : Pm * Pm;
-  const int NFPs = ND == 2 ? a.Ps : a.Ps * a.Ps;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= (int64_t)a.n * NFPm) return;
-  const int t = (int)(gid % NFPm);
-  const FaceRec r = a.recs[gid / NFPm];
-  const int dm = r.mf >> 1, sm = r.mf & 1, ss = r.sf & 1;
-  const int u = orient_map(r.orient, t, Pm, ND);
-  const T* trv = MODE == 1 ? a.trv : nullptr;
-
-  S qM[NV], qS[NV];
-  load_trace_pt<ND>(a.trq, trv, r.mt, 0, NV, NFPm, t, qM);
-  {
-    FaceArgs<T> b = a;
-    b.trv = trv;
-    slave_at_mortar<ND>(b, r.st, 0, NV, u, qS);
-  }
-  T A[ND], n[ND];
-  const T sgm = sm ? T(1) : T(-1);
-  const T absA = geo_face(a.geo_m, r.me, r.mf, ND * ND + 2 + dm, t);
-  const T inv_absA = geo_face(a.geo_m, r.me, r.mf, ND * ND + 2 + ND + dm, t);
-#pragma unroll
-  for (int j = 0; j < ND; ++j) {
-    A[j] = sgm * geo_face(a.geo_m, r.me, r.mf, dm * ND + j, t);
-    n[j] = A[j] * inv_absA;
-  }
-  S Fn[NV];
-  common_flux<ND>(a.flux, qM, qS, n, absA, a.gamma, Fn);
-  S qc[NV];
-  if (VISC) {
-#pragma unroll
-    for (int v = 0; v < NV; ++v) qc[v] = T(0.5) * (qM[v] + qS[v]);
-    T cM[ND], cS[ND];
-    const T gJ = a.basis[Pm].dgf[sm] * geo_face(a.geo_m, r.me, r.mf, ND * ND + 1, t);
-#pragma unroll
-    for (int j = 0; j < ND; ++j) cM[j] = gJ * geo_face(a.geo_m, r.me, r.mf, dm * ND + j, t);
-    slave_coef_at_mortar<ND>(a, r, u, cS);
-    S GM[ND][NV], GS[ND][NV], Gc[ND][NV];
-    load_trace_pt<ND>(a.trq, trv, r.mt, NV, ND * NV, NFPm, t, &GM[0][0]);
-    {
-      FaceArgs<T> b = a;
-      b.trv = trv;
-      slave_at_mortar<ND>(b, r.st, NV, ND * NV, u, &GS[0][0]);
-    }
-    if (DIAG) {
-#pragma unroll
-      for (int j = 0; j < ND; ++j)
-#pragma unroll
-        for (int v = 0; v < NV; ++v) Gc[j][v] = T(0.5) * (GM[j][v] + GS[j][v]);
-#pragma unroll
-      for (int j = 0; j < ND; ++j) {
-        if (j != dm) continue;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) Gc[j][v] = Gc[j][v] + T(0.5) * (cM[j] * (qc[v] - qM[v]) + cS[j] * (qc[v] - qS[v]));
-      }
-      S fr[NV];
-      flux_viscous_row<ND>(qc, Gc, a.gamma, a.mu, a.kappa, dm, fr);
-      T Ad = T(0);
-#pragma unroll
-      for (int j = 0; j < ND; ++j)
-        if (j == dm) Ad = A[j];
-#pragma unroll
-      for (int v = 0; v < NV; ++v) Fn[v] = Fn[v] - fr[v] * Ad;
-    } else {
-#pragma unroll
-      for (int j = 0; j < ND; ++j)
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-          Gc[j][v] = T(0.5) * (GM[j][v] + cM[j] * (qc[v] - qM[v]) + GS[j][v] + cS[j] * (qc[v] - qS[v]));
-      S fv[ND][NV];
-      flux_viscous<ND>(qc, Gc, a.gamma, a.mu, a.kappa, fv);
-#pragma unroll
-      for (int v = 0; v < NV; ++v) {
-        S acc = szero<S>();
-#pragma unroll
-        for (int j = 0; j < ND; ++j) acc = acc + fv[j][v] * A[j];
-        Fn[v] = Fn[v] - acc;
-      }
-    }
-  }
-  // master side
-  T* om = a.fout + r.mo;
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    S x = sgm * Fn[v];
-    om[v * NFPm + t] = MODE == 1 ? tangent(x) : value(x);
-    if (VISC) {
-      S dq = qc[v] - qM[v];
-      om[(NV + v) * NFPm + t] = value(dq);
-      if (MODE == 1) om[(2 * NV + v) * NFPm + t] = tangent(dq);
-    }
-  }
-  const T sgs = ss ? T(1) : T(-1);
-  if (Pm == a.Ps) {
-    T* os = a.fout + r.so;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      S x = sgs * (T(0) - Fn[v]);
-      os[v * NFPs + u] = MODE == 1 ? tangent(x) : value(x);
-      if (VISC) {
-        S dq = qc[v] - qS[v];
-        os[(NV + v) * NFPs + u] = value(dq);
-        if (MODE == 1) os[(2 * NV + v) * NFPs + u] = tangent(dq);
-      }
-    }
-  } else {
-    // mortar values (master order) for the projection kernel: -Fn, then q^com
-    T* sc = a.scratch + a.scratch_base + (int64_t)r.idx * 4 * NV * NFPm;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      S x = T(0) - Fn[v];
-      sc[v * NFPm + t] = MODE == 1 ? tangent(x) : value(x);
-      if (VISC) {
-        sc[(NV + v) * NFPm + t] = value(qc[v]);
-        if (MODE == 1) sc[(2 * NV + v) * NFPm + t] = tangent(qc[v]);
-      }
-    }
-  }
-}
-
-// L2 projection of the mortar values onto the lower-degree side.
-// One thread per (face, slave point).
-template <typename T, int ND, bool VISC, int MODE>
-__global__ void __launch_bounds__(128) mortar_project_kernel(FaceArgs<T> a) {
-  constexpr int NV = ND + 2;
-  if (gate_closed(a.gate)) return;
-  const int Pm = a.Pm, Ps = a.Ps;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ int64_t sst[kFaceThreads];       // mixed groups: the faces' slave trace blocks, elements and faces
+  __shared__ int32_t sse[kFaceThreads], ssf[kFaceThreads];
+  if (gate_closed(m.gate)) return;
+  int gi = 0;
+  while (gi + 1 < m.ng && (int)blockIdx.x >= m.g[gi + 1].block0) ++gi;
+  const FaceGroupRef& g = m.g[gi];
+  const int Pm = g.Pm, Ps = g.Ps;
   const int NFPm = ND == 2 ? Pm : Pm * Pm;
   const int NFPs = ND == 2 ? Ps : Ps * Ps;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= (int64_t)a.n * NFPs) return;
-  const int pt = (int)(gid % NFPs);
-  const FaceRec r = a.recs[gid / NFPs];
-  const int ss = r.sf & 1;
-  const T sgs = ss ? T(1) : T(-1);
-  const int pa = pt % Ps, pb = ND == 2 ? 0 : pt / Ps;
-  const T* sc = a.scratch + a.scratch_base + (int64_t)r.idx * 4 * NV * NFPm;
-  const int ncomp = VISC ? (MODE == 1 ? 3 * NV : 2 * NV) : NV;
-  T acc[3 * NV];
-  for (int c = 0; c < ncomp; ++c) acc[c] = T(0);
-  for (int mb = 0; mb < (ND == 2 ? 1 : Pm); ++mb) {
-    const T wb = ND == 2 ? T(1) : a.mortar->Pi[pb][mb];
-    for (int ma = 0; ma < Pm; ++ma) {
-      const T w = a.mortar->Pi[pa][ma] * wb;
-      const int tm = orient_inv(r.orient, ma + Pm * mb, Pm, ND);
-      for (int c = 0; c < ncomp; ++c) acc[c] += w * sc[c * NFPm + tm];
-    }
+  const int lf = threadIdx.x / NFPm, t = threadIdx.x - lf * NFPm;
+  const int64_t f0 = (int64_t)((int)blockIdx.x - g.block0) * g.fb;
+  const bool valid = lf < g.fb && f0 + lf < g.n;
+  if (g.kind != 0) {
+    if (valid) boundary_point<T, ND, VISC, MODE>(m, g, g.brecs[f0 + lf], t);
+    return;
   }
-  T* os = a.fout + r.so;
-  for (int v = 0; v < NV; ++v) {
-    os[v * NFPs + pt] = sgs * acc[v];
+  const bool mixed = Pm != Ps;
+  FaceRec r{};
+  if (valid) r = g.recs[f0 + lf];
+  const T* trv = MODE == 1 ? m.trv : nullptr;
+  const MortarTab<T>& mt = m.mortar[Pm * (kPM + 1) + Ps];
+  T* const sm = reinterpret_cast<T*>(smem_raw);
+  const int fstride = MF::stride(NFPm, NFPs);
+  if (mixed) {
+    if (valid && t == 0) {
+      sst[lf] = r.st;
+      sse[lf] = r.se;
+      ssf[lf] = r.sf;
+    }
+    __syncthreads();
+    const int nfaces = (int)min((int64_t)g.fb, (int64_t)g.n - f0);
+    const int per = MF::NT * NFPs;
+    for (int k = threadIdx.x; k < nfaces * per; k += kFaceThreads) {
+      const int f = k / per, o = k - f * per;
+      sm[f * fstride + o] = m.trq[sst[f] + o];
+      if (MODE == 1) sm[f * fstride + per + o] = trv[sst[f] + o];
+    }
     if (VISC) {
-      const T qs = a.trq[r.st + (int64_t)v * NFPs + pt];
-      os[(NV + v) * NFPs + pt] = acc[NV + v] - qs;
-      if (MODE == 1) {
-        const T qsd = a.trv[r.st + (int64_t)v * NFPs + pt];
-        os[(2 * NV + v) * NFPs + pt] = acc[2 * NV + v] - qsd;
+      // lifting coefficients g_s'(face) S_d[j] / |J| at the slave's own points
+      const GeoView<T>& gs = m.geo[Ps];
+      for (int k = threadIdx.x; k < nfaces * NFPs; k += kFaceThreads) {
+        const int f = k / NFPs, pt = k - f * NFPs;
+        const int64_t e = sse[f];
+        const int sf = ssf[f];
+        const T gJ = m.basis[Ps].dgf[sf & 1] * geo_face(gs, e, sf, ND * ND + 1, pt);
+        T* c = sm + f * fstride + (MODE == 1 ? 2 : 1) * per;
+#pragma unroll
+        for (int j = 0; j < ND; ++j) c[j * NFPs + pt] = gJ * geo_face(gs, e, sf, (sf >> 1) * ND + j, pt);
+      }
+    }
+    __syncthreads();
+  }
+  const int dm = r.mf >> 1, sm_ = r.mf & 1, ss = r.sf & 1;
+  const T sgm = sm_ ? T(1) : T(-1), sgs = ss ? T(1) : T(-1);
+  int u = 0;
+  S Fn[NV], qc[NV];
+  if (valid) {
+    u = orient_map(r.orient, t, Pm, ND);
+    const int ua = u % Pm, ub = ND == 2 ? 0 : u / Pm;
+    const T* sq = sm + lf * fstride;           // staged slave traces (mixed)
+    const T* sv = sq + MF::NT * NFPs;
+    const GeoView<T>& geo_m = m.geo[Pm];
+    S qM[NV], qS[NV];
+    load_trace_pt<ND>(m.trq, trv, r.mt, 0, NV, NFPm, t, qM);
+    if (mixed) staged_at_mortar<ND, NV, MODE>(sq, sv, mt, Ps, NFPs, ua, ub, qS);
+    else load_trace_pt<ND>(m.trq, trv, r.st, 0, NV, NFPs, u, qS);
+    T A[ND], n[ND];
+    const T absA = geo_face(geo_m, r.me, r.mf, ND * ND + 2 + dm, t);
+    const T inv_absA = geo_face(geo_m, r.me, r.mf, ND * ND + 2 + ND + dm, t);
+#pragma unroll
+    for (int j = 0; j < ND; ++j) {
+      A[j] = sgm * geo_face(geo_m, r.me, r.mf, dm * ND + j, t);
+      n[j] = A[j] * inv_absA;
+    }
+    common_flux<ND>(m.flux, qM, qS, n, absA, m.gamma, Fn);
+    if (VISC) {
+#pragma unroll
+      for (int v = 0; v < NV; ++v) qc[v] = T(0.5) * (qM[v] + qS[v]);
+      T cM[ND], cS[ND];
+      const T gJ = m.basis[Pm].dgf[sm_] * geo_face(geo_m, r.me, r.mf, ND * ND + 1, t);
+#pragma unroll
+      for (int j = 0; j < ND; ++j) cM[j] = gJ * geo_face(geo_m, r.me, r.mf, dm * ND + j, t);
+      S GM[ND][NV], GS[ND][NV], Gc[ND][NV];
+      load_trace_pt<ND>(m.trq, trv, r.mt, NV, ND * NV, NFPm, t, &GM[0][0]);
+      if (mixed) {
+        staged_at_mortar<ND, ND, 0>(sq + (MODE == 1 ? 2 : 1) * MF::NT * NFPs, (const T*)nullptr, mt, Ps, NFPs, ua, ub, cS);
+        staged_at_mortar<ND, ND * NV, MODE>(sq + NV * NFPs, sv + NV * NFPs, mt, Ps, NFPs, ua, ub, &GS[0][0]);
+      } else {
+        const GeoView<T>& geo_s = m.geo[Ps];
+        const T gJs = m.basis[Ps].dgf[ss] * geo_face(geo_s, r.se, r.sf, ND * ND + 1, u);
+#pragma unroll
+        for (int j = 0; j < ND; ++j) cS[j] = gJs * geo_face(geo_s, r.se, r.sf, (r.sf >> 1) * ND + j, u);
+        load_trace_pt<ND>(m.trq, trv, r.st, NV, ND * NV, NFPs, u, &GS[0][0]);
+      }
+      if (DIAG) {
+#pragma unroll
+        for (int j = 0; j < ND; ++j)
+#pragma unroll
+          for (int v = 0; v < NV; ++v) Gc[j][v] = T(0.5) * (GM[j][v] + GS[j][v]);
+#pragma unroll
+        for (int j = 0; j < ND; ++j) {
+          if (j != dm) continue;
+#pragma unroll
+          for (int v = 0; v < NV; ++v) Gc[j][v] = Gc[j][v] + T(0.5) * (cM[j] * (qc[v] - qM[v]) + cS[j] * (qc[v] - qS[v]));
+        }
+        S fr[NV];
+        flux_viscous_row<ND>(qc, Gc, m.gamma, m.mu, m.kappa, dm, fr);
+        T Ad = T(0);
+#pragma unroll
+        for (int j = 0; j < ND; ++j)
+          if (j == dm) Ad = A[j];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) Fn[v] = Fn[v] - fr[v] * Ad;
+      } else {
+#pragma unroll
+        for (int j = 0; j < ND; ++j)
+#pragma unroll
+          for (int v = 0; v < NV; ++v)
+            Gc[j][v] = T(0.5) * (GM[j][v] + cM[j] * (qc[v] - qM[v]) + GS[j][v] + cS[j] * (qc[v] - qS[v]));
+        S fv[ND][NV];
+        flux_viscous<ND>(qc, Gc, m.gamma, m.mu, m.kappa, fv);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          S acc = szero<S>();
+#pragma unroll
+          for (int j = 0; j < ND; ++j) acc = acc + fv[j][v] * A[j];
+          Fn[v] = Fn[v] - acc;
+        }
+      }
+    }
+    store_face_side<ND, VISC, MODE>(m.fout + r.mo, NFPm, t, sgm, Fn, qc, qM);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Fn[v] = T(0) - Fn[v];    // the slave's side
+    if (!mixed) store_face_side<ND, VISC, MODE>(m.fout + r.so, NFPs, u, sgs, Fn, qc, qS);
+  }
+  if (!mixed) return;
+  // mortar values -Fn, then q^com, in the slave's point order; then the L2
+  // projection, one thread per (face, slave point): fewer than mortar points
+  __syncthreads();   // every read of the staged traces is done
+  if (valid) {
+    T* sc = sm + lf * fstride + u;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      sc[v * NFPm] = MODE == 1 ? tangent(Fn[v]) : value(Fn[v]);
+      if (VISC) {
+        sc[(NV + v) * NFPm] = value(qc[v]);
+        if (MODE == 1) sc[(2 * NV + v) * NFPm] = tangent(qc[v]);
       }
     }
   }
-}
-
-// ---------------------------------------------------------------------------
-// Boundary faces: ghost state (wall / far field).  One thread per (face, point).
-// ---------------------------------------------------------------------------
-template <typename T>
-struct BndArgs {
-  const BndRec* recs;
-  const T* trq;
-  const T* trv;
-  T* fout;
-  const BasisTab<T>* basis;
-  GeoView<T> geo;
-  T gamma, mu, kappa;
-  T qinf[5];
-  int n, P, kind;
-  int flux;            // common inviscid flux: 0 Rusanov, 1 Roe
-  const int* gate = nullptr;   // see gate_closed
-};
-
-template <typename T, int ND, bool VISC, int MODE>
-__global__ void __launch_bounds__(128) bnd_kernel(BndArgs<T> a) {
-  constexpr int NV = ND + 2;
-  if (gate_closed(a.gate)) return;
-  using S = typename std::conditional<MODE == 1, Dual<T>, T>::type;
-  const int P = a.P;
-  const int NFP = ND == 2 ? P : P * P;
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= (int64_t)a.n * NFP) return;
-  const int t = (int)(gid % NFP);
-  const BndRec r = a.recs[gid / NFP];
-  const int d = r.mf >> 1, s = r.mf & 1;
-  const T* trv = MODE == 1 ? a.trv : nullptr;
-  S qM[NV], qG[NV];
-  load_trace_pt<ND>(a.trq, trv, r.mt, 0, NV, NFP, t, qM);
-  ghost_state<ND>(qM, a.kind, a.qinf, qG);
-  T A[ND], n[ND];
-  const T sg = s ? T(1) : T(-1);
-  const T absA = geo_face(a.geo, r.me, r.mf, ND * ND + 2 + d, t);
-  const T inv_absA = geo_face(a.geo, r.me, r.mf, ND * ND + 2 + ND + d, t);
+  __syncthreads();
+  const int lp = threadIdx.x / NFPs, pt = threadIdx.x - lp * NFPs;
+  if (lp >= g.fb || f0 + lp >= g.n) return;
+  const FaceRec rp = g.recs[f0 + lp];
+  const T sgp = (rp.sf & 1) ? T(1) : T(-1);
+  const int pa = pt % Ps, pb = ND == 2 ? 0 : pt / Ps;
+  const T* sc = sm + lp * fstride;
+  T acc[MF::NO];
 #pragma unroll
-  for (int j = 0; j < ND; ++j) {
-    A[j] = sg * geo_face(a.geo, r.me, r.mf, d * ND + j, t);
-    n[j] = A[j] * inv_absA;
-  }
-  S Fn[NV];
-  common_flux<ND>(a.flux, qM, qG, n, absA, a.gamma, Fn);
-  S qc[NV];
-  if (VISC) {
+  for (int c = 0; c < MF::NO; ++c) acc[c] = T(0);
+  for (int mb = 0; mb < (ND == 2 ? 1 : Pm); ++mb) {
+    const T wb = ND == 2 ? T(1) : mt.Pi[pb][mb];
+    for (int ma = 0; ma < Pm; ++ma) {
+      const T w = mt.Pi[pa][ma] * wb;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) qc[v] = T(0.5) * (qM[v] + qG[v]);
-    T cM[ND];
-    const T gJ = a.basis[P].dgf[s] * geo_face(a.geo, r.me, r.mf, ND * ND + 1, t);
-#pragma unroll
-    for (int j = 0; j < ND; ++j) cM[j] = gJ * geo_face(a.geo, r.me, r.mf, d * ND + j, t);
-    S GM[ND][NV], Gc[ND][NV];
-    load_trace_pt<ND>(a.trq, trv, r.mt, NV, ND * NV, NFP, t, &GM[0][0]);
-#pragma unroll
-    for (int j = 0; j < ND; ++j)
-#pragma unroll
-      for (int v = 0; v < NV; ++v) Gc[j][v] = GM[j][v] + cM[j] * (qc[v] - qM[v]);
-    S fv[ND][NV];
-    flux_viscous<ND>(qc, Gc, a.gamma, a.mu, a.kappa, fv);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      S acc = szero<S>();
-#pragma unroll
-      for (int j = 0; j < ND; ++j) acc = acc + fv[j][v] * A[j];
-      if (a.kind == -1 && v == NV - 1) acc = szero<S>();   // adiabatic wall
-      Fn[v] = Fn[v] - acc;
+      for (int c = 0; c < MF::NO; ++c) acc[c] += w * sc[c * NFPm + ma + Pm * mb];
     }
   }
-  T* om = a.fout + r.mo;
+  T* os = m.fout + rp.so;
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    S x = sg * Fn[v];
-    om[v * NFP + t] = MODE == 1 ? tangent(x) : value(x);
+    os[v * NFPs + pt] = sgp * acc[v];
     if (VISC) {
-      S dq = qc[v] - qM[v];
-      om[(NV + v) * NFP + t] = value(dq);
-      if (MODE == 1) om[(2 * NV + v) * NFP + t] = tangent(dq);
+      os[(NV + v) * NFPs + pt] = acc[NV + v] - m.trq[rp.st + (int64_t)v * NFPs + pt];
+      if (MODE == 1) os[(2 * NV + v) * NFPs + pt] = acc[2 * NV + v] - trv[rp.st + (int64_t)v * NFPs + pt];
     }
   }
 }

@@ -15,6 +15,76 @@
 
 namespace frgb {
 
+template <typename T>
+struct FaceArgs {
+  const FaceRec* recs;
+  const T* trq;        // traces of q
+  const T* trv;        // traces of the tangent (JVP)
+  T* fout;
+  T* scratch;          // mixed-degree groups: [face][comp][NFPm]
+  const BasisTab<T>* basis;
+  const MortarTab<T>* mortar;   // Pm -> Ps tables (nullptr when Pm == Ps)
+  GeoView<T> geo_m, geo_s;
+  T gamma, mu, kappa;
+  int n, Pm, Ps, nvt;
+  int flux;            // common inviscid flux: 0 Rusanov, 1 Roe
+  int64_t scratch_base;
+  const int* gate = nullptr;   // see gate_closed
+};
+
+// value of the slave's trace component at mortar point u (slave axes, Pm grid)
+template <int ND, typename S, typename T>
+__device__ __forceinline__ void slave_at_mortar(const FaceArgs<T>& a, int64_t base, int comp0,
+                                                int ncomp, int u, S* out) {
+  const int Ps = a.Ps, Pm = a.Pm;
+  const int NFPs = ND == 2 ? Ps : Ps * Ps;
+  if (Pm == Ps) {
+    load_trace_pt<ND>(a.trq, a.trv, base, comp0, ncomp, NFPs, u, out);
+    return;
+  }
+  const int ua = u % Pm, ub = ND == 2 ? 0 : u / Pm;
+  for (int c = 0; c < ncomp; ++c) set_scalar(out[c], T(0), T(0));
+  for (int bb = 0; bb < (ND == 2 ? 1 : Ps); ++bb) {
+    const T wb = ND == 2 ? T(1) : a.mortar->I[ub][bb];
+    for (int aa = 0; aa < Ps; ++aa) {
+      const T w = a.mortar->I[ua][aa] * wb;
+      const int pt = aa + Ps * bb;
+      for (int c = 0; c < ncomp; ++c) {
+        T v = a.trq[base + (int64_t)(comp0 + c) * NFPs + pt];
+        T dv = a.trv ? a.trv[base + (int64_t)(comp0 + c) * NFPs + pt] : T(0);
+        S x;
+        set_scalar(x, v, dv);
+        out[c] = out[c] + w * x;
+      }
+    }
+  }
+}
+
+template <int ND, typename T>
+__device__ __forceinline__ void slave_coef_at_mortar(const FaceArgs<T>& a, const FaceRec& r, int u,
+                                                     T* cS) {
+  // c = g_s'(face) S_d[j] / |J| at the slave's own points, interpolated to the mortar
+  const int Ps = a.Ps, Pm = a.Pm;
+  const int ds = r.sf >> 1, ss = r.sf & 1;
+  const T g = a.basis[Ps].dgf[ss];
+  for (int j = 0; j < ND; ++j) cS[j] = T(0);
+  if (Pm == Ps) {
+    const T gJ = g * geo_face(a.geo_s, r.se, r.sf, ND * ND + 1, u);
+    for (int j = 0; j < ND; ++j) cS[j] = gJ * geo_face(a.geo_s, r.se, r.sf, ds * ND + j, u);
+    return;
+  }
+  const int ua = u % Pm, ub = ND == 2 ? 0 : u / Pm;
+  for (int bb = 0; bb < (ND == 2 ? 1 : Ps); ++bb) {
+    const T wb = ND == 2 ? T(1) : a.mortar->I[ub][bb];
+    for (int aa = 0; aa < Ps; ++aa) {
+      const T w = a.mortar->I[ua][aa] * wb;
+      const int pt = aa + Ps * bb;
+      const T gJ = g * geo_face(a.geo_s, r.se, r.sf, ND * ND + 1, pt);
+      for (int j = 0; j < ND; ++j) cS[j] += w * (gJ * geo_face(a.geo_s, r.se, r.sf, ds * ND + j, pt));
+    }
+  }
+}
+
 // Transpose of the linear map G -> f_v(q, G) at fixed q: Gb = (d f_v / d G)^T fb.
 template <int ND, typename T>
 __device__ __forceinline__ void viscous_adjoint_G(const T* q, const T (*fb)[ND + 2], T gamma, T mu,
