@@ -354,7 +354,6 @@ fr_status build_layout(fr_ctx* c) {
       v.push_back(r);
     }
   }
-  int64_t sc = 0;
   for (auto& kv : inter) {
     // master-face direction as the major key (element order kept within a
     // direction): warps then see one normal axis, which the diagonal-metric
@@ -365,10 +364,6 @@ fr_status build_layout(fr_ctx* c) {
     g.pm = kv.first.first;
     g.ps = kv.first.second;
     g.n = (int)kv.second.size();
-    if (g.pm != g.ps) {
-      g.scratch_base = sc;
-      sc += (int64_t)g.n * 4 * nv * ipow(g.pm + 1, nd - 1);
-    }
     FR_CUDA(cudaMalloc(&g.d_recs, sizeof(FaceRec) * g.n));
     FR_CUDA(cudaMemcpy(g.d_recs, kv.second.data(), sizeof(FaceRec) * g.n, cudaMemcpyHostToDevice));
     c->fgroups.push_back(g);
@@ -381,10 +376,6 @@ fr_status build_layout(fr_ctx* c) {
     FR_CUDA(cudaMalloc(&g.d_recs, sizeof(BndRec) * g.n));
     FR_CUDA(cudaMemcpy(g.d_recs, kv.second.data(), sizeof(BndRec) * g.n, cudaMemcpyHostToDevice));
     c->bgroups.push_back(g);
-  }
-  if (sc > c->scratch_cap) {
-    set_error("mortar scratch exceeds its capacity");
-    return FR_ERR_INVALID;
   }
   FR_TRY(build_fused_table(c, elem_slot));
   rebuild_work_table(c);   // a failure leaves no table: launches go per bucket
@@ -596,12 +587,10 @@ static fr_status create_impl(const fr_mesh_desc* m, const fr_physics* ph, const 
     c->n_dof_cap = (int64_t)E * c->nv * NSP;
     c->trace_cap = (int64_t)E * nf * c->nvt * NFP;
     c->fout_cap = (int64_t)E * nf * 3 * c->nv * NFP;
-    c->scratch_cap = (int64_t)E * nf * 4 * c->nv * NFP;   // bound on all mortar groups
   }
   FR_CUDA(cudaMalloc(&c->d_trace_q, sizeof(double) * c->trace_cap));
   FR_CUDA(cudaMalloc(&c->d_trace_v, sizeof(double) * c->trace_cap));
   FR_CUDA(cudaMalloc(&c->d_fout, sizeof(double) * c->fout_cap));
-  FR_CUDA(cudaMalloc(&c->d_scratch, sizeof(double) * std::max<int64_t>(c->scratch_cap, 1)));
   FR_CUDA(cudaMalloc(&c->d_slot_elem, sizeof(int32_t) * E));
   FR_CUDA(cudaMalloc(&c->d_elem_slot, sizeof(int32_t) * E));
   FR_CUDA(cudaMalloc(&c->d_canon_off, sizeof(int64_t) * E));
@@ -637,7 +626,6 @@ static void destroy_impl(fr_ctx* c) {
   cudaFree(c->d_trace_q);
   cudaFree(c->d_trace_v);
   cudaFree(c->d_fout);
-  cudaFree(c->d_scratch);
   cudaFree(c->d_fbar);
   cudaFree(c->d_trbar);
   cudaFree(c->d_slot_elem);

@@ -339,11 +339,9 @@ static int face_groups(fr_ctx* c, FaceMulti<T>& m) {
   return blocks;
 }
 
-template <typename T, int ND, bool VISC, int MODE, bool DIAG = false>
-static void launch_faces(fr_ctx* c, const T* trq, const T* trv, cudaStream_t s) {
-  FaceMulti<T> m;
+template <typename T, int ND>
+static int face_multi(fr_ctx* c, const T* trq, const T* trv, FaceMulti<T>& m) {
   const int blocks = face_groups<T, ND>(c, m);
-  if (blocks == 0) return;
   for (const auto& b : c->buckets) m.geo[b.p + 1] = geo_view<T>(c, b.p);
   m.trq = trq;
   m.trv = trv;
@@ -357,6 +355,14 @@ static void launch_faces(fr_ctx* c, const T* trq, const T* trv, cudaStream_t s) 
   m.nvt = c->nvt;
   m.flux = c->phys.flux;
   m.gate = c->gate;
+  return blocks;
+}
+
+template <typename T, int ND, bool VISC, int MODE, bool DIAG = false>
+static void launch_faces(fr_ctx* c, const T* trq, const T* trv, cudaStream_t s) {
+  FaceMulti<T> m;
+  const int blocks = face_multi<T, ND>(c, trq, trv, m);
+  if (blocks == 0) return;
   double nb = 0.0, nfl = 0.0;
   for (const auto& g : c->fgroups) {
     const int64_t nm = (int64_t)g.n * ipow(g.pm + 1, ND - 1);
@@ -686,37 +692,49 @@ static void jvp_impl(fr_ctx* c, const T* q, const T* v, T* Jv, cudaStream_t s, b
 
 
 // ---------------------------------------------------------------------------
-// VJP: forward traces and face outputs, then volume^T -> face^T -> trace^T
+// VJP: forward traces and (NS) primal jumps, then volume^T -> face^T -> trace^T
 // ---------------------------------------------------------------------------
-template <typename T, int ND, int P, bool VISC>
-static void launch_vol_adj_p(fr_ctx* c, const VolAdjArgs<T>& a, cudaStream_t s) {
-  using Cfg = VolCfg<ND, P>;
-  const size_t smem = (size_t)Cfg::EPB * (2 * (ND + 2) + 2 * ND * (ND + 2)) * Cfg::NSP * sizeof(T);
-  auto kern = vol_adj_kernel<T, ND, P, VISC>;
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    configured = true;
-  }
-  FR_LAUNCH_B(c, sizeof(T) == 8 ? "vol_adj_f64" : "vol_adj_f32", s,
-              (double)a.count * (ND + 2) * Cfg::NSP * sizeof(T) * 2,
-              kern<<<nblocks(a.count, Cfg::EPB), Cfg::THREADS, smem, s>>>(a));
+template <typename T, int ND, int P, bool VISC, bool DIAG>
+static void launch_vol_adj_p(const VolAdjArgs<T>& a, int epb, cudaStream_t s) {
+  const size_t smem = (size_t)epb * (VISC ? 2 + ND : 1) * (ND + 2) * Shape<ND, P>::NSP * sizeof(T);
+  auto kern = vol_adj_kernel<T, ND, P, VISC, DIAG>;
+  static size_t configured = 48 * 1024;
+  ensure_smem(kern, smem, configured);
+  kern<<<nblocks(a.count, epb), epb * Shape<ND, P>::NSP, smem, s>>>(a, epb);
 }
 
-template <typename T, int ND, bool VISC>
+template <typename T, int ND, bool VISC, bool DIAG>
 static void vjp_impl(fr_ctx* c, const T* q, const T* w, T* out, cudaStream_t s) {
+  constexpr int NV = ND + 2;
   T* trq = (T*)c->d_trace_q;
-  T* fbar = (T*)c->d_fbar;
-  T* trbar = (T*)c->d_trbar;
-  launch_traces<T, ND, VISC>(c, q, trq, s);
-  launch_faces<T, ND, VISC, 0>(c, trq, nullptr, s);
+  FaceAdjMulti<T> am;
+  FaceMulti<T>& m = am.f;
+  const int blocks = face_multi<T, ND>(c, trq, nullptr, m);
+  am.fbar = (const T*)c->d_fbar;
+  am.trbar = (T*)c->d_trbar;
+  size_t jsmem = 0, fsmem = 0;
+  double npts = 0.0;
+  for (int i = 0; i < m.ng; ++i) {
+    const FaceGroupRef& g = m.g[i];
+    const int nm = ipow(g.Pm, ND - 1), ns = ipow(g.Ps, ND - 1);
+    npts += (double)g.n * nm;
+    if (nm != ns) jsmem = std::max(jsmem, (size_t)g.fb * NV * nm * sizeof(T));
+    fsmem = std::max(fsmem, (size_t)g.fb * AdjFace<ND, VISC>::stride(nm, ns) * sizeof(T));
+  }
+  launch_traces<T, ND, VISC, DIAG>(c, q, trq, s);
+  if (VISC && blocks > 0) {
+    auto kern = jump_kernel<T, ND>;
+    static size_t configured = 48 * 1024;
+    ensure_smem(kern, jsmem, configured);
+    FR_LAUNCH_B(c, "jump", s, npts * 4 * NV * sizeof(T), kern<<<blocks, kFaceThreads, jsmem, s>>>(m));
+  }
   for (const auto& b : c->buckets) {
     VolAdjArgs<T> a;
     a.q = q;
     a.w = w;
     a.out = out;
     a.fout = (const T*)c->d_fout;
-    a.fbar = fbar;
+    a.fbar = (T*)c->d_fbar;
     a.slot_elem = c->d_slot_elem;
     a.basis = basis_ptr<T>(c);
     a.geo = geo_view<T>(c, b.p);
@@ -727,63 +745,27 @@ static void vjp_impl(fr_ctx* c, const T* q, const T* w, T* out, cudaStream_t s) 
     a.out_base = b.out_base;
     a.count = b.count;
     a.slot_begin = b.slot_begin;
-    switch (b.p + 1) {
-      case 2: launch_vol_adj_p<T, ND, 2, VISC>(c, a, s); break;
-      case 3: launch_vol_adj_p<T, ND, 3, VISC>(c, a, s); break;
-      case 4: launch_vol_adj_p<T, ND, 4, VISC>(c, a, s); break;
-      case 5: launch_vol_adj_p<T, ND, 5, VISC>(c, a, s); break;
-      case 6: launch_vol_adj_p<T, ND, 6, VISC>(c, a, s); break;
-    }
+    const int P = b.p + 1, e = epb_multi(ND, P, mesh_threads(c));
+    FR_LAUNCH_B(c, sizeof(T) == 8 ? "vol_adj_f64" : "vol_adj_f32", s,
+                (double)b.count * NV * nsp_of(ND, P) * sizeof(T) * 2, {
+      switch (P) {
+        case 2: launch_vol_adj_p<T, ND, 2, VISC, DIAG>(a, e, s); break;
+        case 3: launch_vol_adj_p<T, ND, 3, VISC, DIAG>(a, e, s); break;
+        case 4: launch_vol_adj_p<T, ND, 4, VISC, DIAG>(a, e, s); break;
+        case 5: launch_vol_adj_p<T, ND, 5, VISC, DIAG>(a, e, s); break;
+        case 6: launch_vol_adj_p<T, ND, 6, VISC, DIAG>(a, e, s); break;
+      }
+    });
   }
-  for (const auto& g : c->fgroups) {
-    FaceAdjArgs<T> a;
-    a.recs = g.d_recs;
-    a.trq = trq;
-    a.fbar = fbar;
-    a.trbar = trbar;
-    a.scratch = (T*)c->d_scratch;
-    a.basis = basis_ptr<T>(c);
-    a.mortar = g.pm != g.ps ? mortar_ptr<T>(c, g.pm + 1, g.ps + 1) : nullptr;
-    a.geo_m = geo_view<T>(c, g.pm);
-    a.geo_s = geo_view<T>(c, g.ps);
-    a.gamma = (T)c->phys.gamma;
-    a.mu = (T)c->phys.mu;
-    a.kappa = (T)c->phys.kappa;
-    a.flux = c->phys.flux;
-    a.n = g.n;
-    a.Pm = g.pm + 1;
-    a.Ps = g.ps + 1;
-    a.scratch_base = g.scratch_base;
-    const int64_t nm = (int64_t)g.n * ipow(a.Pm, ND - 1);
-    FR_LAUNCH(c, "face_adj", s, face_adj_kernel<T, ND, VISC><<<nblocks(nm, 128), 128, 0, s>>>(a));
-    if (g.pm != g.ps) {
-      const int64_t ns = (int64_t)g.n * ipow(a.Ps, ND - 1);
-      FR_LAUNCH(c, "mortar_gather_adj", s,
-                mortar_gather_adj_kernel<T, ND, VISC><<<nblocks(ns, 128), 128, 0, s>>>(a));
-    }
-  }
-  for (const auto& g : c->bgroups) {
-    BndAdjArgs<T> a;
-    a.recs = g.d_recs;
-    a.trq = trq;
-    a.fbar = fbar;
-    a.trbar = trbar;
-    a.basis = basis_ptr<T>(c);
-    a.geo = geo_view<T>(c, g.p);
-    a.gamma = (T)c->phys.gamma;
-    a.mu = (T)c->phys.mu;
-    a.kappa = (T)c->phys.kappa;
-    a.flux = c->phys.flux;
-    for (int v = 0; v < 5; ++v) a.qinf[v] = (T)c->phys.q_inf[v];
-    a.n = g.n;
-    a.P = g.p + 1;
-    a.kind = g.kind;
-    const int64_t nm = (int64_t)g.n * ipow(a.P, ND - 1);
-    FR_LAUNCH(c, "boundary_adj", s, bnd_adj_kernel<T, ND, VISC><<<nblocks(nm, 128), 128, 0, s>>>(a));
+  if (blocks > 0) {
+    auto kern = face_adj_kernel<T, ND, VISC, DIAG>;
+    static size_t configured = 48 * 1024;
+    ensure_smem(kern, fsmem, configured);
+    FR_LAUNCH(c, "face_adj", s, kern<<<blocks, kFaceThreads, fsmem, s>>>(am));
   }
   for (const auto& b : c->buckets) {
     TraceAdjArgs<T> a;
-    a.trbar = trbar;
+    a.trbar = (const T*)c->d_trbar;
     a.out = out;
     a.basis = basis_ptr<T>(c);
     a.state_base = b.state_base;
@@ -792,14 +774,15 @@ static void vjp_impl(fr_ctx* c, const T* q, const T* w, T* out, cudaStream_t s) 
     a.nvt = c->nvt;
     const int P = b.p + 1;
     const int64_t n = (int64_t)b.count * ipow(P, ND);
-    const unsigned g = nblocks(n, 256);
-    FR_LAUNCH_B(c, "trace_adj", s, (double)n * (ND + 2) * sizeof(T), {
+    const int threads = mesh_threads(c);
+    const unsigned g = nblocks(n, threads);
+    FR_LAUNCH_B(c, "trace_adj", s, (double)n * NV * sizeof(T), {
       switch (P) {
-        case 2: trace_adj_kernel<T, ND, 2, VISC><<<g, 256, 0, s>>>(a); break;
-        case 3: trace_adj_kernel<T, ND, 3, VISC><<<g, 256, 0, s>>>(a); break;
-        case 4: trace_adj_kernel<T, ND, 4, VISC><<<g, 256, 0, s>>>(a); break;
-        case 5: trace_adj_kernel<T, ND, 5, VISC><<<g, 256, 0, s>>>(a); break;
-        case 6: trace_adj_kernel<T, ND, 6, VISC><<<g, 256, 0, s>>>(a); break;
+        case 2: trace_adj_kernel<T, ND, 2, VISC><<<g, threads, 0, s>>>(a); break;
+        case 3: trace_adj_kernel<T, ND, 3, VISC><<<g, threads, 0, s>>>(a); break;
+        case 4: trace_adj_kernel<T, ND, 4, VISC><<<g, threads, 0, s>>>(a); break;
+        case 5: trace_adj_kernel<T, ND, 5, VISC><<<g, threads, 0, s>>>(a); break;
+        case 6: trace_adj_kernel<T, ND, 6, VISC><<<g, threads, 0, s>>>(a); break;
       }
     });
   }
@@ -965,7 +948,7 @@ static void run_op_cfg(fr_ctx* c, int op, const void* q, const void* v, void* ou
   T* oo = (T*)out;
   if (op == 0) residual_impl<T, ND, VISC, DIAG>(c, qq, oo, s);
   else if (op == 1) jvp_impl<T, ND, VISC, DIAG>(c, qq, vv, oo, s);
-  else if (op == 2) vjp_impl<T, ND, VISC>(c, qq, vv, oo, s);
+  else if (op == 2) vjp_impl<T, ND, VISC, DIAG>(c, qq, vv, oo, s);
   else if (op == 3) {
     if (fused_jvp_on<T>(c) || compact_jvp_on<T>(c)) launch_ctraces<T, ND, VISC>(c, qq, (T*)c->d_trace_q, s);
     else launch_traces<T, ND, VISC, DIAG>(c, qq, (T*)c->d_trace_q, s);

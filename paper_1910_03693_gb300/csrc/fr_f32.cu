@@ -15,7 +15,7 @@ fr_status run_op_f32(fr_ctx* c, int op, const void* q, const void* v, void* out,
     }
   }
   if (c->nd == 2) run_f32_2d(c, op, q, v, out, s);
-  else if (c->diag && op != 2) run_f32_3d_diag(c, op, q, v, out, s);   // the VJP has no diagonal variant
+  else if (c->diag) run_f32_3d_diag(c, op, q, v, out, s);
   else run_f32_3d(c, op, q, v, out, s);
   return cuda_check(cudaGetLastError(), "FR kernel launch");
 }

@@ -87,7 +87,6 @@ struct Bucket {
 struct FaceGroup {
   int pm = 0, ps = 0, n = 0;
   FaceRec* d_recs = nullptr;
-  int64_t scratch_base = 0; // values, mixed-degree groups only
 };
 struct BndGroup {
   int p = 0, kind = 0, n = 0;
@@ -196,11 +195,10 @@ struct fr_ctx {
   int32_t* d_elem_slot = nullptr;        // [E] slot of each element
   // workspaces (bytes sized for FP64 at capacity)
   int nvt = 0;                           // trace components per face point
-  int64_t trace_cap = 0, fout_cap = 0, scratch_cap = 0;
+  int64_t trace_cap = 0, fout_cap = 0;
   void* d_trace_q = nullptr;
   void* d_trace_v = nullptr;
   void* d_fout = nullptr;
-  void* d_scratch = nullptr;
   void* d_fbar = nullptr;                // VJP: adjoints of the face outputs
   void* d_trbar = nullptr;               // VJP: adjoints of the traces
   // faces
