@@ -373,7 +373,7 @@ fr_status esdirk_step(fr_ctx* ctx, const fr_tableau* tab, double dt, double* q_i
 /* Launch configuration (the paper has no counterpart: it is the GPU work
  * decomposition).  The trace and volume kernels process `epb` elements per
  * CTA (one thread per solution point); with several degree buckets they run
- * as one persistent launch over a table of (bucket, tile) items ordered by
+ * as one launch over a table of (bucket, tile) items ordered by
  * decreasing cost n_sp (p+1) per tile, the paper's element-weight estimate
  * (Sec. 3.2).  In GMRES with the exact JVP, each Arnoldi product -J V[j]
  * (column gather, JVP kernels, sign) is replayed from a CUDA graph captured
@@ -392,9 +392,8 @@ fr_status esdirk_step(fr_ctx* ctx, const fr_tableau* tab, double dt, double* q_i
  * four CTAs; a value whose elements exceed 256 threads also falls back to it;
  * the multi-bucket launch always uses the default);
  * the slot P = 0 holds the multi-bucket choice of that precision and kernel
- * (0 undecided: one launch over all buckets while the mesh's solution points
- * fit in 8 full-occupancy waves of the GPU, else one per bucket; 1 one launch
- * over all buckets; 2 one launch per bucket), which FR_TUNE_MULTI_LAUNCH
+ * (0 undecided: one launch over all buckets, but for the double-float
+ * kernels on meshes of more than 512 points per SM; 1 one launch over all buckets; 2 one launch per bucket), which FR_TUNE_MULTI_LAUNCH
  * enables; slot [0][0][P = 1] holds the element weight
  * that orders the multi-bucket work table (0 n_sp (p+1), 1 n_sp, 2 n_sp^2,
  * 3 n_sp^3: the paper's candidate weights, Sec. 3.2); slot [prec][2][P = 1]
@@ -410,7 +409,7 @@ fr_status esdirk_step(fr_ctx* ctx, const fr_tableau* tab, double dt, double* q_i
  * flags; elements per CTA outside [0, 256], multi-bucket choices outside
  * [0, 2], weight models outside [0, 3], the exact JVP's choice outside [0, 4]
  * or unknown flag bits give FR_ERR_INVALID. */
-#define FR_TUNE_MULTI_LAUNCH 1  /* one persistent launch over all degree buckets */
+#define FR_TUNE_MULTI_LAUNCH 1  /* one launch over all degree buckets */
 #define FR_TUNE_GRAPHS 2        /* host-driven GMRES: the Arnoldi products
                                    replayed from a CUDA graph               */
 #define FR_TUNE_DIAG_METRICS 4  /* 3D meshes of axis-aligned affine elements:

@@ -99,18 +99,21 @@ static inline int epb_for(fr_ctx* c, int prec, int kind, int P) {
 
 // One launch over all buckets for this precision and kernel kind: the master
 // switch, more than one bucket, and the per-kind choice (the autotuner writes
-// it into the unused P = 0 slot of the table: 1 yes, 2 no).  Undecided (0):
-// one launch while the mesh's solution points fit in 8 full-occupancy waves
-// (2048 threads per SM), where launches and tails dominate; beyond that each
-// bucket runs alone at its own degree's register footprint (measured: the
-// 4M-DOF vortex batch is faster in one launch, the 18M-DOF cylinder and the
-// 16M-DOF adapted C-grid per bucket).
-static inline bool use_multi(fr_ctx* c, int prec, int kind) {
+// it into the unused P = 0 slot of the table: 1 yes, 2 no).  Undecided (0): one
+// launch, but for the double-float kernels beyond 512 points per SM: their
+// unrolled code is large, and CTAs of several degrees on an SM share its
+// instruction cache.  Measured, all in one
+// launch against one per bucket: O-grid of degrees 1..4, 3.4M DOF, FP32 JVP 226
+// against 275 us, FP64 residual 1186 / 1301, double-float 589 / 540; 17M DOF
+// 923 / 948, 5563 / 5686, 2089 / 1978; double-float alone: 8,400 points 65 / 100,
+// 84,000 130 / 130, 203,000 269 / 235; batch of degrees 1..5, 2.8M DOF, FP32
+// JVP 69 / 85, 18M DOF 652 / 662.
+static inline bool use_multi(fr_ctx* c, int prec, int kind, bool df = false) {
   if (!c->multi_launch || c->buckets.size() <= 1) return false;
   const int choice = c->epb_tab[prec][kind][0];
   if (choice == 1) return true;
   if (choice == 2) return false;
-  return c->n_dof / c->nv <= (int64_t)8 * 2048 * sm_count(c);
+  return !df || c->n_dof / c->nv <= (int64_t)512 * sm_count(c);
 }
 
 // Work table of the multi-bucket launch, built when the layout or the tuning
@@ -170,7 +173,7 @@ static void launch_traces(fr_ctx* c, const T* q, T* trace, cudaStream_t s) {
   }
   const char* name = kname<T>("trace_f64", "trace_f32", "trace_df");
   int n_items = 0;
-  const WorkItem* items = use_multi(c, prec, 0) ? work_items(c, prec, 0, &n_items) : nullptr;
+  const WorkItem* items = use_multi(c, prec, 0, is_dfloat<T>::value) ? work_items(c, prec, 0, &n_items) : nullptr;
   if (items) {
     TraceMulti<T> m;
     size_t smem = 0;
@@ -185,14 +188,10 @@ static void launch_traces(fr_ctx* c, const T* q, T* trace, cudaStream_t s) {
       smem = std::max(smem, (size_t)e * ((ND + 2) * nsp_of(ND, P) + 2 * ND * (ND + 2) * ipow(P, ND - 1)) * sizeof(T));
     }
     m.items = items;
-    m.n_items = n_items;
     auto kern = trace_multi_kernel<T, ND, VISC, DIAG>;
     static size_t configured = 0;
     ensure_smem(kern, smem, configured);
-    int per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, smem);
-    const unsigned grid = (unsigned)std::max(1, std::min(m.n_items, (int)(std::max(per_sm, 1) * sm_count(c))));
-    FR_LAUNCH_BF(c, name, s, nb, nfl, kern<<<grid, block, smem, s>>>(m));
+    FR_LAUNCH_BF(c, name, s, nb, nfl, kern<<<n_items, block, smem, s>>>(m));
     return;
   }
   for (const auto& b : c->buckets) {
@@ -263,7 +262,7 @@ static void launch_vols(fr_ctx* c, const T* q, const T* v, T* out, cudaStream_t 
     nfl += MODE == 1 ? 0.0 : (double)b.count * nsp_of(ND, P) * flops_volume(ND, P, VISC, DIAG);
   }
   int n_items = 0;
-  const WorkItem* items = use_multi(c, prec, kind) ? work_items(c, prec, kind, &n_items) : nullptr;
+  const WorkItem* items = use_multi(c, prec, kind, is_dfloat<T>::value) ? work_items(c, prec, kind, &n_items) : nullptr;
   if (items) {
     VolMulti<T> m;
     size_t smem = 0;
@@ -278,14 +277,10 @@ static void launch_vols(fr_ctx* c, const T* q, const T* v, T* out, cudaStream_t 
       smem = std::max(smem, (size_t)e * (ND + 2) * (1 + ND) * nsp_of(ND, P) * sizeof(S));
     }
     m.items = items;
-    m.n_items = n_items;
     auto kern = vol_multi_kernel<T, ND, VISC, MODE, DIAG>;
     static size_t configured = 0;
     ensure_smem(kern, smem, configured);
-    int per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, block, smem);
-    const unsigned grid = (unsigned)std::max(1, std::min(m.n_items, (int)(std::max(per_sm, 1) * sm_count(c))));
-    FR_LAUNCH_BF(c, name, s, nb, nfl, kern<<<grid, block, smem, s>>>(m));
+    FR_LAUNCH_BF(c, name, s, nb, nfl, kern<<<n_items, block, smem, s>>>(m));
     return;
   }
   for (const auto& b : c->buckets) {
@@ -450,36 +445,38 @@ static bool cface_vt_usable(const fr_ctx* c, const T* v) {
   }
 }
 
-template <typename T, int ND, int P, bool VISC>
-static void launch_ctrace_p(const CTraceArgs<T>& a, int epb, cudaStream_t s) {
-  const size_t smem = (size_t)epb * (ND + 2) * Shape<ND, P>::NSP * sizeof(T);
-  ctrace_kernel<T, ND, P, VISC><<<nblocks(a.count, epb), epb * Shape<ND, P>::NSP, smem, s>>>(a, epb);
-}
-
+// compact traces of q, every bucket in one launch
 template <typename T, int ND, bool VISC>
 static void launch_ctraces(fr_ctx* c, const T* q, T* out, cudaStream_t s) {
   constexpr int NV = ND + 2, NF = 2 * ND, CT = VISC ? 2 * NV : NV;
-  for (const auto& b : c->buckets) {
-    const int P = b.p + 1, e = epb_multi(ND, P, mesh_threads(c));
-    CTraceArgs<T> a;
-    a.gate = c->gate;
-    a.q = q;
-    a.out = out;
-    a.basis = basis_ptr<T>(c);
-    a.state_base = b.state_base;
-    a.ctrace_base = b.ctrace_base;
-    a.count = b.count;
-    const double nb = (double)b.count * (NV * nsp_of(ND, P) + NF * CT * ipow(P, ND - 1)) * sizeof(T);
-    FR_LAUNCH_B(c, kname<T>("ctrace_f64", "ctrace_f32", "ctrace_df"), s, nb, {
-      switch (P) {
-        case 2: launch_ctrace_p<T, ND, 2, VISC>(a, e, s); break;
-        case 3: launch_ctrace_p<T, ND, 3, VISC>(a, e, s); break;
-        case 4: launch_ctrace_p<T, ND, 4, VISC>(a, e, s); break;
-        case 5: launch_ctrace_p<T, ND, 5, VISC>(a, e, s); break;
-        case 6: launch_ctrace_p<T, ND, 6, VISC>(a, e, s); break;
-      }
-    });
+  CTraceArgs<T> a;
+  a.gate = c->gate;
+  a.q = q;
+  a.out = out;
+  a.basis = basis_ptr<T>(c);
+  a.nb = (int)c->buckets.size();
+  int blocks = 0, threads = 32;
+  size_t smem = 0;
+  double nb = 0.0;
+  for (int i = 0; i < a.nb; ++i) {
+    const Bucket& b = c->buckets[i];
+    const int P = b.p + 1, nsp = nsp_of(ND, P), e = epb_multi(ND, P, mesh_threads(c));
+    a.b[i] = CTraceBucket{b.state_base, b.ctrace_base, b.count, P, e, blocks};
+    blocks += (int)nblocks(b.count, e);
+    threads = std::max(threads, (e * nsp + 31) / 32 * 32);
+    smem = std::max(smem, (size_t)e * NV * nsp * sizeof(T));
+    nb += (double)b.count * (NV * nsp + NF * CT * ipow(P, ND - 1)) * sizeof(T);
   }
+  FR_LAUNCH_B(c, kname<T>("ctrace_f64", "ctrace_f32", "ctrace_df"), s, nb, {
+    switch (a.nb == 1 ? a.b[0].P : 0) {
+      case 2: ctrace_kernel<T, ND, 2, VISC><<<blocks, threads, smem, s>>>(a); break;
+      case 3: ctrace_kernel<T, ND, 3, VISC><<<blocks, threads, smem, s>>>(a); break;
+      case 4: ctrace_kernel<T, ND, 4, VISC><<<blocks, threads, smem, s>>>(a); break;
+      case 5: ctrace_kernel<T, ND, 5, VISC><<<blocks, threads, smem, s>>>(a); break;
+      case 6: ctrace_kernel<T, ND, 6, VISC><<<blocks, threads, smem, s>>>(a); break;
+      default: ctrace_kernel<T, ND, 0, VISC><<<blocks, threads, smem, s>>>(a); break;
+    }
+  });
 }
 
 // Elements per CTA of the fused kernel: as many as fill 256 threads, at most as
@@ -636,7 +633,7 @@ static void jvp_compact_impl(fr_ctx* c, const T* q, const T* v, T* Jv, cudaStrea
     return;
   }
   launch_ctraces<T, ND, VISC>(c, v, trv, s);
-  for (const auto& g : c->fgroups) {
+  auto face_args = [&](const FaceGroup& g) {
     CFaceArgs<T> a;
     a.gate = c->gate;
     a.recs = g.d_recs;
@@ -651,11 +648,43 @@ static void jvp_compact_impl(fr_ctx* c, const T* q, const T* v, T* Jv, cudaStrea
     a.flux = c->phys.flux;
     a.n = g.n;
     a.nvt = c->nvt;
-    const int P = g.pm + 1, NFP = ipow(P, ND - 1);
-    // both sides' compact traces of q and v in; both sides' face outputs out
-    const double nb = (double)g.n * NFP * (4.0 * CT + 2.0 * (VISC ? 3 : 1) * NV) * sizeof(T);
-    FR_LAUNCH_B(c, kname<T>("cface_jvp_f64", "cface_jvp_f32", "cface_jvp_df"), s, nb, {
-      switch (P) {
+    return a;
+  };
+  // both sides' compact traces of q and v in; both sides' face outputs out
+  auto face_bytes = [&](const FaceGroup& g) {
+    return (double)g.n * ipow(g.pm + 1, ND - 1) * (4.0 * CT + 2.0 * (VISC ? 3 : 1) * NV) * sizeof(T);
+  };
+  const char* name = kname<T>("cface_jvp_f64", "cface_jvp_f32", "cface_jvp_df");
+  // several degrees: one launch for all, but for 3D beyond 8 full-occupancy
+  // waves of points, where the bulk-copy kernel of some degrees (111 against
+  // 145 us at 32^3) is worth a launch per group
+  const bool one = c->fgroups.size() > 1 && (ND == 2 || c->n_dof / c->nv <= (int64_t)8 * 2048 * sm_count(c));
+  if (one) {
+    CFaceMulti<T> m;
+    m.ng = 0;
+    int blocks = 0;
+    size_t smem = 0;
+    double nb = 0.0;
+    for (const auto& g : c->fgroups) {
+      const int nfp = ipow(g.pm + 1, ND - 1), fb = nfp >= 128 ? 1 : 128 / nfp;
+      m.g[m.ng] = face_args(g);
+      m.P[m.ng] = g.pm + 1;
+      m.block0[m.ng] = blocks;
+      blocks += (int)nblocks(g.n, fb);
+      smem = std::max(smem, (size_t)fb * 4 * CT * nfp * sizeof(T));
+      nb += face_bytes(g);
+      m.ng += 1;
+    }
+    auto kern = cface_multi_kernel<T, ND, VISC, DIAG>;
+    static size_t configured = 48 * 1024;
+    ensure_smem(kern, smem, configured);
+    FR_LAUNCH_B(c, name, s, nb, kern<<<blocks, 128, smem, s>>>(m));
+  }
+  for (const auto& g : c->fgroups) {
+    if (one) break;
+    const CFaceArgs<T> a = face_args(g);
+    FR_LAUNCH_B(c, name, s, face_bytes(g), {
+      switch (g.pm + 1) {
         case 2: launch_cface_p<T, ND, 2, VISC, DIAG>(c, a, s); break;
         case 3: launch_cface_p<T, ND, 3, VISC, DIAG>(c, a, s); break;
         case 4: launch_cface_p<T, ND, 4, VISC, DIAG>(c, a, s); break;

@@ -292,26 +292,27 @@ struct TraceMulti {
   int P[kMaxBuckets];
   int epb[kMaxBuckets];
   const WorkItem* items;
-  int n_items;
 };
 
-// Every bucket in one persistent launch: CTAs walk the cost-ordered work
-// table with a grid stride and dispatch on the tile's degree.
+// Every bucket in one launch: CTA w takes tile w of the cost-ordered work
+// table and dispatches on its degree.  One tile a CTA and the register caps of
+// the one-degree kernels: walking the table with a grid stride instead made the
+// compiler hold 128 (FP32) to 255 (FP64) registers across the loop, two or one
+// CTAs an SM, against 36-80 of the same code at one degree (O-grid of degrees 1..4, 3.4M
+// DOF: FP32 trace 69 -> 50 us, volume JVP 79 -> 65; FP64 trace 367 -> 302, volume
+// 582 -> 531).
 template <typename T, int ND, bool VISC, bool DIAG>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 1) trace_multi_kernel(const __grid_constant__ TraceMulti<T> m) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) trace_multi_kernel(const __grid_constant__ TraceMulti<T> m) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (gate_closed(m.b[0].gate)) return;
-  for (int w = blockIdx.x; w < m.n_items; w += gridDim.x) {
-    const WorkItem it = m.items[w];
-    const int b = it.bucket;
-    switch (m.P[b]) {
-      case 2: trace_body<T, ND, 2, VISC, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
-      case 3: trace_body<T, ND, 3, VISC, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
-      case 4: trace_body<T, ND, 4, VISC, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
-      case 5: trace_body<T, ND, 5, VISC, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
-      case 6: trace_body<T, ND, 6, VISC, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
-    }
-    __syncthreads();
+  const WorkItem it = m.items[blockIdx.x];
+  const int b = it.bucket;
+  switch (m.P[b]) {
+    case 2: trace_body<T, ND, 2, VISC, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
+    case 3: trace_body<T, ND, 3, VISC, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
+    case 4: trace_body<T, ND, 4, VISC, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
+    case 5: trace_body<T, ND, 5, VISC, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
+    case 6: trace_body<T, ND, 6, VISC, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
   }
 }
 
@@ -864,24 +865,22 @@ struct VolMulti {
   int P[kMaxBuckets];
   int epb[kMaxBuckets];
   const WorkItem* items;
-  int n_items;
 };
 
+// as trace_multi_kernel; FP64 holds two CTAs an SM but for the 3D viscous JVP
 template <typename T, int ND, bool VISC, int MODE, bool DIAG>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 || is_dfloat<T>::value) ? 2 : 1) vol_multi_kernel(const __grid_constant__ VolMulti<T> m) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : (ND == 3 && VISC && MODE == 1 ? 1 : 2))
+    vol_multi_kernel(const __grid_constant__ VolMulti<T> m) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (gate_closed(m.b[0].gate)) return;
-  for (int w = blockIdx.x; w < m.n_items; w += gridDim.x) {
-    const WorkItem it = m.items[w];
-    const int b = it.bucket;
-    switch (m.P[b]) {
-      case 2: vol_body<T, ND, 2, VISC, MODE, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
-      case 3: vol_body<T, ND, 3, VISC, MODE, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
-      case 4: vol_body<T, ND, 4, VISC, MODE, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
-      case 5: vol_body<T, ND, 5, VISC, MODE, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
-      case 6: vol_body<T, ND, 6, VISC, MODE, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
-    }
-    __syncthreads();
+  const WorkItem it = m.items[blockIdx.x];
+  const int b = it.bucket;
+  switch (m.P[b]) {
+    case 2: vol_body<T, ND, 2, VISC, MODE, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
+    case 3: vol_body<T, ND, 3, VISC, MODE, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
+    case 4: vol_body<T, ND, 4, VISC, MODE, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
+    case 5: vol_body<T, ND, 5, VISC, MODE, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
+    case 6: vol_body<T, ND, 6, VISC, MODE, DIAG>(m.b[b], it.first, m.epb[b], smem_raw); break;
   }
 }
 

@@ -90,38 +90,42 @@ __device__ __forceinline__ void trace_point(const T* sq, const BasisTab<T>& B, i
 
 // ---------------------------------------------------------------------------
 // Pass 1: compact traces.  One thread per solution point for the load, then
-// per face point.
+// per face point.  One launch covers every degree bucket (a bucket is a range
+// of blocks).
 // ---------------------------------------------------------------------------
+struct CTraceBucket {
+  int64_t state_base, ctrace_base;
+  int count, P, epb, block0;
+};
+
 template <typename T>
 struct CTraceArgs {
+  CTraceBucket b[kMaxBuckets];
   const T* q;
   T* out;
   const BasisTab<T>* basis;
-  int64_t state_base, ctrace_base;
-  int count;
+  int nb;
   const int* gate = nullptr;   // see gate_closed
 };
 
 template <typename T, int ND, int P, bool VISC>
-__global__ void __launch_bounds__(256) ctrace_kernel(CTraceArgs<T> a, int epb) {
+__device__ __forceinline__ void ctrace_body(const CTraceArgs<T>& a, const CTraceBucket& bk, unsigned char* smem_raw) {
   using Sh = Shape<ND, P>;
   constexpr int NV = Sh::NV, NF = Sh::NF, NSP = Sh::NSP, NFP = Sh::NFP;
   constexpr int CT = CompactWidth<VISC, NV>::value;
   constexpr int NFPT = NF * NFP, ITERS = (NFPT + NSP - 1) / NSP;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  if (gate_closed(a.gate)) return;
   const int le = threadIdx.x / NSP, lt = threadIdx.x % NSP;
-  const int64_t i = (int64_t)blockIdx.x * epb + le;
-  const bool valid = le < epb && i < a.count;
+  const int64_t i = (int64_t)((int)blockIdx.x - bk.block0) * bk.epb + le;
+  const bool valid = le < bk.epb && i < bk.count;
   T* sq = reinterpret_cast<T*>(smem_raw) + le * NV * NSP;
   if (valid) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) sq[v * NSP + lt] = a.q[a.state_base + (i * NV + v) * NSP + lt];
+    for (int v = 0; v < NV; ++v) sq[v * NSP + lt] = a.q[bk.state_base + (i * NV + v) * NSP + lt];
   }
   __syncthreads();
   if (!valid) return;
   const BasisTab<T>& B = a.basis[P];
-  T* out = a.out + a.ctrace_base + i * NF * CT * NFP;
+  T* out = a.out + bk.ctrace_base + i * NF * CT * NFP;
 #pragma unroll
   for (int it = 0; it < ITERS; ++it) {
     const int fp = lt + it * NSP;
@@ -133,6 +137,30 @@ __global__ void __launch_bounds__(256) ctrace_kernel(CTraceArgs<T> a, int epb) {
     for (int v = 0; v < NV; ++v) {
       out[(f * CT + v) * NFP + t] = qf[v];
       if (VISC) out[(f * CT + NV + v) * NFP + t] = dn[v];
+    }
+  }
+}
+
+// PF: the degree's P when the mesh has one bucket, else 0 (at 32^3, p = 3 the
+// instance that switches on the degree holds 4 CTAs an SM and takes 41 us, the
+// instance of one degree 36 us; 32 vortices of five degrees: 10 launches a
+// product of 7 us each -> 2 of 13 us)
+template <typename T, int ND, int PF, bool VISC>
+__global__ void __launch_bounds__(256, PF == 0 ? 4 : 1) ctrace_kernel(const __grid_constant__ CTraceArgs<T> a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (gate_closed(a.gate)) return;
+  if constexpr (PF != 0) {
+    ctrace_body<T, ND, PF, VISC>(a, a.b[0], smem_raw);
+  } else {
+    int bi = 0;
+    while (bi + 1 < a.nb && (int)blockIdx.x >= a.b[bi + 1].block0) ++bi;
+    const CTraceBucket& bk = a.b[bi];
+    switch (bk.P) {
+      case 2: ctrace_body<T, ND, 2, VISC>(a, bk, smem_raw); break;
+      case 3: ctrace_body<T, ND, 3, VISC>(a, bk, smem_raw); break;
+      case 4: ctrace_body<T, ND, 4, VISC>(a, bk, smem_raw); break;
+      case 5: ctrace_body<T, ND, 5, VISC>(a, bk, smem_raw); break;
+      case 6: ctrace_body<T, ND, 6, VISC>(a, bk, smem_raw); break;
     }
   }
 }
@@ -684,17 +712,16 @@ __device__ __forceinline__ void cface_point(const CFaceArgs<T>& a, const FaceRec
 }
 
 template <typename T, int ND, int P, bool VISC, bool DIAG>
-__global__ void __launch_bounds__(128, 4) cface_kernel(CFaceArgs<T> a) {
+__device__ __forceinline__ void cface_body(const CFaceArgs<T>& a, int block, T* sh) {
   constexpr int NV = ND + 2;
   constexpr int NFP = ND == 2 ? P : P * P;
   constexpr int CT = CompactWidth<VISC, NV>::value;
   constexpr int FB = NFP >= 128 ? 1 : 128 / NFP;    // faces a CTA
-  constexpr int BLK = CT * NFP;
-  __shared__ T sh[FB][4][BLK];                        // master q, master v, slave q, slave v
-  if (gate_closed(a.gate)) return;
+  constexpr int BLK = CT * NFP;                      // sh: [FB][4][BLK]: master q, master v, slave q, slave v
   const int lf = threadIdx.x / NFP, t = threadIdx.x % NFP;
-  const int64_t fidx = (int64_t)blockIdx.x * FB + lf;
+  const int64_t fidx = (int64_t)block * FB + lf;
   const bool valid = lf < FB && fidx < a.n;
+  T* mine = sh + lf * 4 * BLK;
   FaceRec r{};
   CFaceGeo<T, ND> g{};
   if (valid) {
@@ -714,11 +741,47 @@ __global__ void __launch_bounds__(128, 4) cface_kernel(CFaceArgs<T> a) {
 #pragma unroll
     for (int w = 0; w < 4; ++w)
 #pragma unroll
-      for (int c = 0; c < CT; ++c) sh[lf][w][c * NFP + t] = buf[w][c];
+      for (int c = 0; c < CT; ++c) mine[w * BLK + c * NFP + t] = buf[w][c];
   }
   __syncthreads();
   if (!valid) return;
-  cface_point<T, ND, P, VISC, DIAG>(a, r, t, g, sh[lf][0], sh[lf][1], sh[lf][2], sh[lf][3]);
+  cface_point<T, ND, P, VISC, DIAG>(a, r, t, g, mine, mine + BLK, mine + 2 * BLK, mine + 3 * BLK);
+}
+
+// FP64 (viscous, 3D) keeps 255 registers: at four CTAs an SM it spilled 1.4 KB a thread
+template <typename T, int ND, int P, bool VISC, bool DIAG>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2) cface_kernel(CFaceArgs<T> a) {
+  constexpr int NFP = ND == 2 ? P : P * P;
+  constexpr int FB = NFP >= 128 ? 1 : 128 / NFP;
+  __shared__ T sh[FB * 4 * CompactWidth<VISC, ND + 2>::value * NFP];
+  if (gate_closed(a.gate)) return;   // before any barrier
+  cface_body<T, ND, P, VISC, DIAG>(a, blockIdx.x, sh);
+}
+
+// The face groups of a mesh of several degrees (a batch of conforming meshes)
+// in one launch: a group is a range of blocks.
+template <typename T>
+struct CFaceMulti {
+  CFaceArgs<T> g[kMaxBuckets];
+  int P[kMaxBuckets], block0[kMaxBuckets];
+  int ng;
+};
+
+template <typename T, int ND, bool VISC, bool DIAG>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2) cface_multi_kernel(const __grid_constant__ CFaceMulti<T> m) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T* sh = reinterpret_cast<T*>(smem_raw);
+  if (gate_closed(m.g[0].gate)) return;
+  int gi = 0;
+  while (gi + 1 < m.ng && (int)blockIdx.x >= m.block0[gi + 1]) ++gi;
+  const int block = (int)blockIdx.x - m.block0[gi];
+  switch (m.P[gi]) {
+    case 2: cface_body<T, ND, 2, VISC, DIAG>(m.g[gi], block, sh); break;
+    case 3: cface_body<T, ND, 3, VISC, DIAG>(m.g[gi], block, sh); break;
+    case 4: cface_body<T, ND, 4, VISC, DIAG>(m.g[gi], block, sh); break;
+    case 5: cface_body<T, ND, 5, VISC, DIAG>(m.g[gi], block, sh); break;
+    case 6: cface_body<T, ND, 6, VISC, DIAG>(m.g[gi], block, sh); break;
+  }
 }
 
 // ---------------------------------------------------------------------------
