@@ -393,8 +393,8 @@ fr_status esdirk_step(fr_ctx* ctx, const fr_tableau* tab, double dt, double* q_i
  * the multi-bucket launch always uses the default);
  * the slot P = 0 holds the multi-bucket choice of that precision and kernel
  * (0 undecided: one launch over all buckets, but for the double-float
- * kernels on meshes of more than 512 points per SM; 1 one launch over all buckets; 2 one launch per bucket), which FR_TUNE_MULTI_LAUNCH
- * enables; slot [0][0][P = 1] holds the element weight
+ * kernels on meshes of more than 512 points per SM; 1 one launch over all
+ * buckets; 2 one launch per bucket), which FR_TUNE_MULTI_LAUNCH enables; slot [0][0][P = 1] holds the element weight
  * that orders the multi-bucket work table (0 n_sp (p+1), 1 n_sp, 2 n_sp^2,
  * 3 n_sp^3: the paper's candidate weights, Sec. 3.2); slot [prec][2][P = 1]
  * chooses the exact JVP's kernels where FR_TUNE_FUSED_JVP allows the

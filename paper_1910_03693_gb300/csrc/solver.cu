@@ -60,26 +60,69 @@ static unsigned red_blocks(int64_t n) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (n + 2 * kRedThreads - 1) / (2 * kRedThreads)));
 }
 
+// Sums of M values (a power of two up to 32) over a warp, all at once: lane l < M
+// returns with the sum of value l.  Each step adds the half of the values a
+// lane gives up to the half it keeps, so M values take M - 1 additions (and one
+// for each lane bit beyond M) instead of five each.  The FP64 pipe issues a warp
+// addition every 16 clocks: with five additions a value, the reduction of 27
+// dot products alone kept an SM's eight warps busy for 8 us (86,400 DOF, up to 26
+// columns, with the short vectors' walk below: dots 28.3 -> 21.0 us, updates 22.9
+// -> 19.4 us a launch).
+template <int M>
+__device__ __forceinline__ double warp_sums(double (&v)[M]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int s = M / 2; s > 0; s >>= 1) {
+    const bool up = (lane & s) != 0;
+#pragma unroll
+    for (int i = 0; i < s; ++i) {
+      const double give = up ? v[i] : v[i + s], keep = up ? v[i + s] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, s);
+    }
+  }
+  double r = v[0];
+#pragma unroll
+  for (int s = M; s < 32; s <<= 1) r += __shfl_xor_sync(0xffffffffu, r, s);
+  return r;
+}
+
+// Warp sums of vals[0..k) into red[warp][0..k), 32 values at a time.
+template <int KC>
+__device__ __forceinline__ void warp_sums_to(const double (&vals)[KC], int k, double (*red)[KC]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int c0 = 0; c0 < KC; c0 += 32) {
+    constexpr int kFull = 32;
+    if (c0 < k) {
+      if (KC - c0 >= kFull) {
+        double v[kFull];
+#pragma unroll
+        for (int i = 0; i < kFull; ++i) v[i] = c0 + i < KC ? vals[c0 + i < KC ? c0 + i : 0] : 0.0;
+        const double r = warp_sums<kFull>(v);
+        if (c0 + lane < k) red[warp][c0 + lane] = r;
+      } else {
+        constexpr int R = KC % 32, M = R <= 1 ? 1 : R <= 2 ? 2 : R <= 4 ? 4 : R <= 8 ? 8 : R <= 16 ? 16 : 32;
+        double v[M];
+#pragma unroll
+        for (int i = 0; i < M; ++i) v[i] = c0 + i < KC ? vals[c0 + i < KC ? c0 + i : 0] : 0.0;
+        const double r = warp_sums<M>(v);
+        if (lane < M && c0 + lane < k) red[warp][c0 + lane] = r;
+      }
+    }
+  }
+}
+
 // Sum vals[0..k) over the grid into out[0..k), deterministically: every block
-// writes its sums (warp-shuffle then shared-memory tree, fixed order) to its
-// own slot of `partial`; the last block to arrive (arrival counter) adds the
-// slots in a fixed order, writes out[] and re-arms the counter.
+// writes its sums (warp sums, then the warps in order) to its own slot of
+// `partial`; the last block to arrive (arrival counter) adds the slots in a
+// fixed order, writes out[] and re-arms the counter.
 // Returns true in the block that wrote out[] (after its threads < k stored it).
 template <int KC>
 __device__ __forceinline__ bool grid_sum(const double (&vals)[KC], int k, double* __restrict__ partial,
                                          double* __restrict__ out, unsigned* __restrict__ ticket) {
   __shared__ double red[kRedThreads / 32][KC];
   __shared__ bool last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int kk = 0; kk < KC; ++kk) {
-    if (kk < k) {
-      double v = vals[kk];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) red[warp][kk] = v;
-    }
-  }
+  warp_sums_to<KC>(vals, k, red);
   __syncthreads();
   if (threadIdx.x < k) {
     double t = 0.0;
@@ -94,7 +137,7 @@ __device__ __forceinline__ bool grid_sum(const double (&vals)[KC], int k, double
   if (!last) return false;
   __threadfence();
   // the last block: thread t adds the slots t, t + blockDim, ... (all loads of
-  // a thread issued together), then the same warp/shared-memory tree as above
+  // a thread issued together), then the same warp and block sums as above
   constexpr int kSlots = (kRedBlocks + kRedThreads - 1) / kRedThreads;
   double tot[KC];
 #pragma unroll
@@ -109,15 +152,7 @@ __device__ __forceinline__ bool grid_sum(const double (&vals)[KC], int k, double
     }
   }
   __syncthreads();
-#pragma unroll
-  for (int kk = 0; kk < KC; ++kk) {
-    if (kk < k) {
-      double v = tot[kk];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) red[warp][kk] = v;
-    }
-  }
+  warp_sums_to<KC>(tot, k, red);
   __syncthreads();
   if (threadIdx.x < k) {
     double t = 0.0;
@@ -258,7 +293,9 @@ struct Unroll {
   // at 32^3 (30 Arnoldi iterations): dots 2.9 -> 4.2 TB/s, updates 4.0 -> 4.4
   // TB/s; reading many columns at once, DRAM serves long runs of each column
   // better than single 512-byte segments spread over the whole vector
-  static constexpr int U = MAP == 1 ? 4 : (KC <= 2 ? 4 : (KC <= 8 ? 2 : 1));
+  // MAP 2 (short vectors): one slot a thread and step, so that the warps of
+  // every SM get work (86,400 values: runs of four slots fill 42 of 169 blocks)
+  static constexpr int U = MAP == 2 ? 1 : MAP == 1 ? 4 : (KC <= 2 ? 4 : (KC <= 8 ? 2 : 1));
   static constexpr int CH = MAP == 1 ? (KC < 4 ? KC : 4) : (KC < 8 ? KC : 8);   // columns per load batch
   // accumulators per column: more than one breaks the FMA dependence chain
   // but costs registers and occupancy, and measured slower in the solver
@@ -658,7 +695,8 @@ __device__ __forceinline__ float dot4(float4 a, float4 b, float s) {
 // out[kk] = s_w V[kk]^T w for kk < k (s_w = -1 with NEG: w holds J v and the
 // Arnoldi vector is -J v), and with with_norm out[k] = ||w||^2; FP32 columns
 // and w, walked as warp runs of U x 32 float4 slots.
-template <int KC, bool NEG>
+// U: float4 slots a thread and loop step (1 for short vectors, see Unroll).
+template <int KC, bool NEG, int U>
 __global__ void __launch_bounds__(kRedThreads) k_multidot32(const float* __restrict__ V, int64_t ldv, int k,
                                                              const float* __restrict__ w, int64_t n,
                                                              double* __restrict__ partial, double* __restrict__ out,
@@ -667,7 +705,7 @@ __global__ void __launch_bounds__(kRedThreads) k_multidot32(const float* __restr
   if (gate && *gate) return;
   // two columns a load batch: 32 registers of column values in flight, so
   // that two CTAs of 256 threads fit on an SM up to KC = 8
-  constexpr int U = 4, CH = KC < 2 ? KC : 2;
+  constexpr int CH = KC < 2 ? KC : 2;
   double acc[KC + 1];
 #pragma unroll
   for (int kk = 0; kk <= KC; ++kk) acc[kk] = 0.0;
@@ -715,7 +753,7 @@ __global__ void __launch_bounds__(kRedThreads) k_multidot32(const float* __restr
 // w_out = s_w w_in - sum_kk s_kk^2 raw[kk] V[kk] in FP32 (s_w = -1 with NEG),
 // out[0] = ||w_out||^2; w_out may be w_in.  With next_scale, the block that
 // finishes the norm stores 1/||w_out|| and next_j as k_orth_update does.
-template <int KC, bool NEG>
+template <int KC, bool NEG, int U>
 __global__ void __launch_bounds__(kRedThreads) k_orth_update32(const float* __restrict__ V, int64_t ldv, int k,
                                                                 const double* __restrict__ raw,
                                                                 const double* __restrict__ scale, const float* w_in,
@@ -724,7 +762,7 @@ __global__ void __launch_bounds__(kRedThreads) k_orth_update32(const float* __re
                                                                 double* __restrict__ next_scale, int* __restrict__ jidx,
                                                                 int next_j, const int* __restrict__ gate, StepArgs step) {
   if (gate && *gate) return;
-  constexpr int U = 4, CH = KC < 4 ? KC : 4;
+  constexpr int CH = KC < 4 ? KC : 4;
   __shared__ float hs[KC];
   if (threadIdx.x < KC)
     hs[threadIdx.x] = threadIdx.x < k ? (float)(scale[threadIdx.x] * scale[threadIdx.x] * raw[threadIdx.x]) : 0.f;
@@ -802,11 +840,19 @@ __global__ void k_scale32(const double* __restrict__ x, double a, float* __restr
     y[i] = (float)(a * x[i]);
 }
 
+// Whether n values in slots of w leave SMs without a block when every thread
+// takes a run of four slots: then one slot a thread.
+static bool short_vector(const fr_ctx* c, int64_t n, int w) {
+  return n < (int64_t)4 * w * kRedThreads * 2 * c->sms;
+}
+
 // launch KERNEL<KC, VEC, WT, NEG> with the smallest KC >= k; VEC when every
 // vector starts on a 16-byte boundary and the column stride is even
 #define FR_KC_LAUNCH(KC_, V_, grid, KERNEL, WT, NEG, ...)                                                \
   do {                                                                                                  \
-    if (c->arnoldi_map == 1)                                                                            \
+    if (c->arnoldi_map == 1 && short_vector(c, n, (V_) ? 2 : 1))                                        \
+      KERNEL<KC_, V_, WT, NEG, 2><<<wave_grid<KERNEL<KC_, V_, WT, NEG, 2>>(grid), kRedThreads, 0, s>>>(__VA_ARGS__); \
+    else if (c->arnoldi_map == 1)                                                                       \
       KERNEL<KC_, V_, WT, NEG, 1><<<wave_grid<KERNEL<KC_, V_, WT, NEG, 1>>(grid), kRedThreads, 0, s>>>(__VA_ARGS__); \
     else                                                                                                \
       KERNEL<KC_, V_, WT, NEG, 0><<<wave_grid<KERNEL<KC_, V_, WT, NEG, 0>>(grid), kRedThreads, 0, s>>>(__VA_ARGS__); \
@@ -828,8 +874,13 @@ __global__ void k_scale32(const double* __restrict__ x, double a, float* __restr
   } while (0)
 
 // the FP32-basis kernels KERNEL<KC, NEG> with the smallest KC >= k
-#define FR_KC32_LAUNCH(KC_, NEG_, grid, KERNEL, ...) \
-  KERNEL<KC_, NEG_><<<wave_grid<KERNEL<KC_, NEG_>>(grid), kRedThreads, 0, s>>>(__VA_ARGS__)
+#define FR_KC32_LAUNCH(KC_, NEG_, grid, KERNEL, ...)                                                       \
+  do {                                                                                                   \
+    if (short_vector(c, n, 4))                                                                           \
+      KERNEL<KC_, NEG_, 1><<<wave_grid<KERNEL<KC_, NEG_, 1>>(grid), kRedThreads, 0, s>>>(__VA_ARGS__);     \
+    else                                                                                                 \
+      KERNEL<KC_, NEG_, 4><<<wave_grid<KERNEL<KC_, NEG_, 4>>(grid), kRedThreads, 0, s>>>(__VA_ARGS__);     \
+  } while (0)
 #define FR_KC32_CASES(k, NEG_, grid, KERNEL, ...)                        \
   do {                                                                  \
     if ((k) <= 1) FR_KC32_LAUNCH(1, NEG_, grid, KERNEL, __VA_ARGS__);   \
