@@ -12,8 +12,6 @@
 
 namespace frgb {
 
-fr_status build_layout(fr_ctx* c);
-
 // ---------------------------------------------------------------------------
 // indicator: eta = sum w|J| (s - s_{p-1})^2 / sum w|J| s^2 with s_{p-1} the
 // Legendre truncation that drops every mode with an index equal to p.  One
@@ -85,12 +83,11 @@ __global__ void k_max_partial(const double* __restrict__ x, int n, double* __res
   if (threadIdx.x == 0) part[blockIdx.x] = sm[0];
 }
 
-__global__ void k_max_final(const double* __restrict__ part, int nb, double* __restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double m = 0.0;
-    for (int b = 0; b < nb; ++b) m = fmax(m, part[b]);
-    out[0] = m;
-  }
+__global__ void k_max_final(const double* __restrict__ part, int nb, double* __restrict__ out) {   // one warp
+  double m = 0.0;
+  for (int b = threadIdx.x; b < nb; b += 32) m = fmax(m, part[b]);
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (threadIdx.x == 0) out[0] = m;
 }
 
 template <typename T, int ND>
@@ -181,9 +178,9 @@ __global__ void k_decide(const double* __restrict__ eta, const double* __restric
   p_new[e] = (int8_t)p;
 }
 
-// one Jacobi sweep of p_e <- max(p_e, max_n p_n - 1); *changed set when anything rose
+// one Jacobi sweep of p_e <- max(p_e, max_n p_n - 1)
 __global__ void k_smooth(const int8_t* __restrict__ p_in, const int32_t* __restrict__ nbr, int nf, int E,
-                         int8_t* __restrict__ p_out, int* __restrict__ changed) {
+                         int8_t* __restrict__ p_out) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= E) return;
   int p = p_in[e];
@@ -191,63 +188,15 @@ __global__ void k_smooth(const int8_t* __restrict__ p_in, const int32_t* __restr
     const int n = nbr[(int64_t)e * nf + f];
     if (n >= 0) p = max(p, (int)p_in[n] - 1);
   }
-  if (p != p_in[e]) atomicOr(changed, 1);
   p_out[e] = (int8_t)p;
 }
 
-// stable counting sort by (p, id): per-block counts of each degree
-constexpr int kSortBlock = 1024;
-__global__ void k_sort_count(const int8_t* __restrict__ p, int E, int* __restrict__ blk_counts) {
-  __shared__ int cnt[kMaxDeg + 1];
-  if (threadIdx.x <= kMaxDeg) cnt[threadIdx.x] = 0;
-  __syncthreads();
-  const int e = blockIdx.x * kSortBlock + threadIdx.x;
-  if (e < E) atomicAdd(&cnt[p[e]], 1);
-  __syncthreads();
-  if (threadIdx.x <= kMaxDeg) blk_counts[blockIdx.x * (kMaxDeg + 1) + threadIdx.x] = cnt[threadIdx.x];
-}
-
-// exclusive offsets: blk_off[b][p] = bucket_base[p] + sum_{b' < b} counts[b'][p]
-__global__ void k_sort_scan(const int* __restrict__ blk_counts, int nb, int* __restrict__ blk_off,
-                            int* __restrict__ totals) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  int tot[kMaxDeg + 1] = {0};
-  for (int b = 0; b < nb; ++b)
-    for (int p = 0; p <= kMaxDeg; ++p) tot[p] += blk_counts[b * (kMaxDeg + 1) + p];
-  int base[kMaxDeg + 1];
-  int run = 0;
-  for (int p = 0; p <= kMaxDeg; ++p) {
-    base[p] = run;
-    run += tot[p];
-    totals[p] = tot[p];
-  }
-  for (int b = 0; b < nb; ++b)
-    for (int p = 0; p <= kMaxDeg; ++p) {
-      blk_off[b * (kMaxDeg + 1) + p] = base[p];
-      base[p] += blk_counts[b * (kMaxDeg + 1) + p];
-    }
-}
-
-// rank of each element among the block's elements of its degree (stable)
-__global__ void k_sort_scatter(const int8_t* __restrict__ p, int E, const int* __restrict__ blk_off,
-                               int32_t* __restrict__ new_slot_elem, int32_t* __restrict__ new_elem_slot) {
-  __shared__ int warp_cnt[kSortBlock / 32][kMaxDeg + 1];
-  const int e = blockIdx.x * kSortBlock + threadIdx.x;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int pe = e < E ? p[e] : -1;
-  int rank_in_warp = 0;
-  for (int pp = 0; pp <= kMaxDeg; ++pp) {
-    const unsigned m = __ballot_sync(0xffffffffu, pe == pp);
-    if (pe == pp) rank_in_warp = __popc(m & ((1u << lane) - 1u));
-    if (lane == 0) warp_cnt[warp][pp] = __popc(m);
-  }
-  __syncthreads();
-  if (e >= E) return;
-  int before = 0;
-  for (int w = 0; w < warp; ++w) before += warp_cnt[w][pe];
-  const int slot = blk_off[blockIdx.x * (kMaxDeg + 1) + pe] + before + rank_in_warp;
-  new_slot_elem[slot] = e;
-  new_elem_slot[e] = slot;
+// dst[0, *n) = src[0, *n): the transferred state back into the caller's buffer
+// (its length is still on the device)
+template <typename T>
+__global__ void k_copy_n(const T* __restrict__ src, T* __restrict__ dst, const int64_t* __restrict__ n) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < *n; i += (int64_t)gridDim.x * blockDim.x)
+    dst[i] = src[i];
 }
 
 // state transfer: one block per new slot; 1D operator applied in each direction
@@ -300,26 +249,6 @@ __global__ void k_transfer(const T* __restrict__ q_old, T* __restrict__ q_new,
     for (int k = threadIdx.x; k < nsn; k += blockDim.x) dst[v * nsn + k] = (T)in[k];
     __syncthreads();
   }
-}
-
-__global__ void k_new_offsets(const int32_t* __restrict__ new_slot_elem, const int8_t* __restrict__ p_new,
-                              const int* __restrict__ totals, int E, int nd, int nv,
-                              int64_t* __restrict__ new_state_off) {
-  // bucket bases in values, then offset within the bucket
-  const int slot = blockIdx.x * blockDim.x + threadIdx.x;
-  if (slot >= E) return;
-  const int p = p_new[new_slot_elem[slot]];
-  int64_t base = 0;
-  int first = 0;
-  for (int pp = 0; pp < p; ++pp) {
-    const int P = pp + 1;
-    const int64_t nsp = nd == 2 ? P * P : P * P * P;
-    base += (int64_t)totals[pp] * nv * nsp;
-    first += totals[pp];
-  }
-  const int P = p + 1;
-  const int64_t nsp = nd == 2 ? P * P : P * P * P;
-  new_state_off[slot] = base + (int64_t)(slot - first) * nv * nsp;
 }
 
 static fr_status ensure_transfer_tables(fr_ctx* c, double** out) {
@@ -392,92 +321,59 @@ fr_status p_rebucket(fr_ctx* c, const double* eta_dev, const double* eta_max_dev
   }
   cudaStream_t s = (cudaStream_t)stream;
   const int E = c->E, nf = c->nf;
-  const int nb = (E + kSortBlock - 1) / kSortBlock;
-  // integer workspace: p_old, p_a, p_b (bytes) ; counts, offsets, totals, slots (ints)
-  if (!c->d_adapt_i32) {
-    const size_t ints = (size_t)2 * nb * (kMaxDeg + 1) + (kMaxDeg + 1) + 2 * (size_t)E + 4;
-    if (cudaMalloc(&c->d_adapt_i32, sizeof(int) * ints) != cudaSuccess) return FR_ERR_NOMEM;
-    if (cudaMalloc(&c->d_adapt_i8, 3 * (size_t)E) != cudaSuccess) return FR_ERR_NOMEM;
-    if (!c->d_adapt_f64 && cudaMalloc(&c->d_adapt_f64, sizeof(double) * 1024) != cudaSuccess) return FR_ERR_NOMEM;
-    if (cudaMalloc(&c->d_old_state_off, sizeof(int64_t) * E) != cudaSuccess) return FR_ERR_NOMEM;
-    if (cudaMalloc(&c->d_new_state_off, sizeof(int64_t) * E) != cudaSuccess) return FR_ERR_NOMEM;
-    if (cudaMalloc(&c->d_old_elem_slot, sizeof(int32_t) * E) != cudaSuccess) return FR_ERR_NOMEM;
-    if (cudaMalloc(&c->d_old_slot_p, E) != cudaSuccess) return FR_ERR_NOMEM;
-    if (cudaMallocHost(&c->h_flag, sizeof(int) * 4) != cudaSuccess) return FR_ERR_NOMEM;
+  if (!c->d_adapt_i8) {
+    const bool ok = cudaMalloc(&c->d_adapt_i8, 2 * (size_t)E) == cudaSuccess &&
+                    cudaMalloc(&c->d_old_state_off, sizeof(int64_t) * E) == cudaSuccess &&
+                    cudaMalloc(&c->d_old_elem_slot, sizeof(int32_t) * E) == cudaSuccess &&
+                    cudaMalloc(&c->d_old_slot_p, E) == cudaSuccess;
+    if (!ok) return FR_ERR_NOMEM;
   }
-  int* blk_counts = c->d_adapt_i32;
-  int* blk_off = blk_counts + nb * (kMaxDeg + 1);
-  int* totals = blk_off + nb * (kMaxDeg + 1);
-  int32_t* new_slot_elem = totals + (kMaxDeg + 1);
-  int32_t* new_elem_slot = new_slot_elem + E;
-  int* changed = new_elem_slot + E;
-  int8_t* p_old = c->d_adapt_i8;
-  int8_t* pa = p_old + E;
-  int8_t* pb = pa + E;
-  // current degree of every element (host copy is authoritative)
-  cudaMemcpyAsync(p_old, c->p.data(), E, cudaMemcpyHostToDevice, s);
-  const unsigned ge = (unsigned)((E + 255) / 256);
-  FR_LAUNCH(c, "rebucket", s, k_decide<<<ge, 256, 0, s>>>(eta_dev, eta_max_dev, p_old, o->nu_max, o->nu_min,
-                                                           o->p_min, o->p_max, E, pa));
-  // jump limit: Jacobi sweeps to the fixed point (at most p_max - p_min + 1 rises)
-  int sweeps = 0;
-  for (;; ++sweeps) {
-    if (sweeps > 2 * kMaxDeg + 2) {
-      set_error("p_rebucket: neighbour smoothing did not reach its fixed point");
-      return FR_ERR_NOT_CONVERGED;
-    }
-    cudaMemsetAsync(changed, 0, sizeof(int), s);
-    FR_LAUNCH(c, "rebucket", s, k_smooth<<<ge, 256, 0, s>>>(pa, c->d_nbr, nf, E, pb, changed));
-    cudaMemcpyAsync(c->h_flag, changed, sizeof(int), cudaMemcpyDeviceToHost, s);
-    if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_check(cudaGetLastError(), "p_rebucket");
-    std::swap(pa, pb);
-    if (c->h_flag[0] == 0) break;
-  }
-  // stable counting sort by (p, id)
-  FR_LAUNCH(c, "rebucket", s, k_sort_count<<<nb, kSortBlock, 0, s>>>(pa, E, blk_counts));
-  FR_LAUNCH(c, "rebucket", s, k_sort_scan<<<1, 32, 0, s>>>(blk_counts, nb, blk_off, totals));
-  FR_LAUNCH(c, "rebucket", s, k_sort_scatter<<<nb, kSortBlock, 0, s>>>(pa, E, blk_off, new_slot_elem, new_elem_slot));
-  FR_LAUNCH(c, "rebucket", s, k_new_offsets<<<ge, 256, 0, s>>>(new_slot_elem, pa, totals, E, c->nd, c->nv,
-                                                                c->d_new_state_off));
-  // keep the old layout for the transfer
-  cudaMemcpyAsync(c->d_old_state_off, c->d_state_off, sizeof(int64_t) * E, cudaMemcpyDeviceToDevice, s);
-  cudaMemcpyAsync(c->d_old_elem_slot, c->d_elem_slot, sizeof(int32_t) * E, cudaMemcpyDeviceToDevice, s);
-  cudaMemcpyAsync(c->d_old_slot_p, c->d_slot_p, E, cudaMemcpyDeviceToDevice, s);
   double* xfer = nullptr;
   fr_status e = ensure_transfer_tables(c, &xfer);
   if (e != FR_OK) return e;
-  // new degrees to the host (bucket metadata and face lists are rebuilt there)
-  std::vector<int8_t> pnew(E);
-  cudaMemcpyAsync(pnew.data(), pa, E, cudaMemcpyDeviceToHost, s);
-  if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_check(cudaGetLastError(), "p_rebucket");
-  int64_t ndof_new = 0;
-  for (int i = 0; i < E; ++i) {
-    const int P = pnew[i] + 1;
-    ndof_new += (int64_t)c->nv * (c->nd == 2 ? P * P : P * P * P);
-  }
   void* tmp = prec == FR_F64 ? (void*)vec64(c, 10) : (void*)vec32(c, 3);
   if (!tmp) return FR_ERR_NOMEM;
-  if (c->nd == 2) {
-    if (prec == FR_F64)
-      FR_LAUNCH(c, "rebucket", s, k_transfer<double, 2><<<E, 128, 0, s>>>((const double*)q_dev, (double*)tmp, new_slot_elem, c->d_old_elem_slot, c->d_old_state_off, c->d_old_slot_p, pa, c->d_new_state_off, xfer, E));
-    else
-      FR_LAUNCH(c, "rebucket", s, k_transfer<float, 2><<<E, 128, 0, s>>>((const float*)q_dev, (float*)tmp, new_slot_elem, c->d_old_elem_slot, c->d_old_state_off, c->d_old_slot_p, pa, c->d_new_state_off, xfer, E));
-  } else {
-    if (prec == FR_F64)
-      FR_LAUNCH(c, "rebucket", s, k_transfer<double, 3><<<E, 128, 0, s>>>((const double*)q_dev, (double*)tmp, new_slot_elem, c->d_old_elem_slot, c->d_old_state_off, c->d_old_slot_p, pa, c->d_new_state_off, xfer, E));
-    else
-      FR_LAUNCH(c, "rebucket", s, k_transfer<float, 3><<<E, 128, 0, s>>>((const float*)q_dev, (float*)tmp, new_slot_elem, c->d_old_elem_slot, c->d_old_state_off, c->d_old_slot_p, pa, c->d_new_state_off, xfer, E));
+  int8_t* pa = c->d_adapt_i8;
+  int8_t* pb = pa + E;
+  const unsigned ge = (unsigned)((E + 255) / 256);
+  FR_LAUNCH(c, "rebucket", s, k_decide<<<ge, 256, 0, s>>>(eta_dev, eta_max_dev, c->d_p, o->nu_max, o->nu_min,
+                                                           o->p_min, o->p_max, E, pa));
+  // jump limit: after k Jacobi sweeps an element holds max_n (p_n - d(e, n)) over
+  // the elements within k faces, and one further away than p_max - p_min - 1
+  // cannot raise it above p_min: the fixed point, without asking the device
+  for (int k = 0; k < o->p_max - o->p_min - 1; ++k) {
+    FR_LAUNCH(c, "rebucket", s, k_smooth<<<ge, 256, 0, s>>>(pa, c->d_nbr, nf, E, pb));
+    std::swap(pa, pb);
   }
-  const size_t esz = prec == FR_F64 ? 8 : 4;
-  cudaMemcpyAsync(q_dev, tmp, esz * ndof_new, cudaMemcpyDeviceToDevice, s);
-  if (perm_out_dev) cudaMemcpyAsync(perm_out_dev, new_slot_elem, sizeof(int32_t) * E, cudaMemcpyDeviceToDevice, s);
+  // keep the old layout for the transfer, then the new one and the state
+  cudaMemcpyAsync(c->d_old_state_off, c->d_state_off, sizeof(int64_t) * E, cudaMemcpyDeviceToDevice, s);
+  cudaMemcpyAsync(c->d_old_elem_slot, c->d_elem_slot, sizeof(int32_t) * E, cudaMemcpyDeviceToDevice, s);
+  cudaMemcpyAsync(c->d_old_slot_p, c->d_slot_p, E, cudaMemcpyDeviceToDevice, s);
+  if ((e = layout_device(c, pa, s)) != FR_OK) return e;
+  cudaMemcpyAsync(c->d_p, pa, E, cudaMemcpyDeviceToDevice, s);
+  const unsigned gc = (unsigned)std::max<int64_t>(1, std::min<int64_t>((c->n_dof_cap + 255) / 256, (int64_t)c->sms * 16));
+#define FR_TRANSFER(T, ND)                                                                                            \
+  do {                                                                                                                \
+    FR_LAUNCH(c, "rebucket", s,                                                                                       \
+              k_transfer<T, ND><<<E, 128, 0, s>>>((const T*)q_dev, (T*)tmp, c->d_slot_elem, c->d_old_elem_slot,       \
+                                                  c->d_old_state_off, c->d_old_slot_p, pa, c->d_state_off, xfer, E)); \
+    FR_LAUNCH(c, "rebucket", s, k_copy_n<T><<<gc, 256, 0, s>>>((const T*)tmp, (T*)q_dev, layout_n_dof(c)));            \
+  } while (0)
+  if (c->nd == 2) {
+    if (prec == FR_F64) FR_TRANSFER(double, 2);
+    else FR_TRANSFER(float, 2);
+  } else {
+    if (prec == FR_F64) FR_TRANSFER(double, 3);
+    else FR_TRANSFER(float, 3);
+  }
+#undef FR_TRANSFER
+  if (perm_out_dev) cudaMemcpyAsync(perm_out_dev, c->d_slot_elem, sizeof(int32_t) * E, cudaMemcpyDeviceToDevice, s);
   if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_check(cudaGetLastError(), "p_rebucket");
-  // host metadata: buckets, slot tables and face lists for the new degrees
-  const bool same = std::equal(pnew.begin(), pnew.end(), c->p.begin());
-  c->p = pnew;
-  if (!same) {
-    e = build_layout(c);
-    if (e != FR_OK) return e;
+  const int8_t* pnew = layout_degrees(c);
+  if (!std::equal(pnew, pnew + E, c->p.begin())) {   // unchanged degrees: the tables were rewritten as they were
+    c->p.assign(pnew, pnew + E);
+    if ((e = layout_host(c, s)) != FR_OK) return e;
+    if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_check(cudaGetLastError(), "p_rebucket");   // its tile table
   }
   return cuda_check(cudaGetLastError(), "p_rebucket");
 }

@@ -1,5 +1,5 @@
-// Context creation: validation, metric terms, per-degree buckets and face
-// lists; the C-ABI entry points that only need host logic.
+// Context creation: validation and metric terms; the C-ABI entry points that
+// only need host logic.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -151,9 +151,6 @@ static bool element_is_affine(const fr_ctx* c, int e) {
   return twist <= 1e-13 * scale;
 }
 
-// ---------------------------------------------------------------------------
-// Layout: buckets in ascending (p, id) order, offsets, face lists.
-// ---------------------------------------------------------------------------
 void collect_graph_timers(fr_ctx* c) {
   for (int k = 0; k < 2; ++k)
     if (c->graph_timers_live[k]) {
@@ -174,212 +171,12 @@ void clear_graphs(fr_ctx* c) {
   }
 }
 
-// Work table of the multi-bucket launch: tiles of epb_multi elements, ordered
-// by decreasing element weight per tile (higher degrees first), bucket order
-// kept among equal weights.  Built on the host and uploaded synchronously.
-fr_status rebuild_work_table(fr_ctx* c) {
-  cudaFree(c->d_work);
-  c->d_work = nullptr;
-  c->n_work = 0;
-  std::vector<std::pair<double, WorkItem>> items;
-  for (size_t bi = 0; bi < c->buckets.size(); ++bi) {
-    const Bucket& b = c->buckets[bi];
-    const int P = b.p + 1, e = epb_multi(c->nd, P, mesh_threads(c));
-    for (int f = 0; f < b.count; f += e) {
-      const int ne = std::min(e, b.count - f);
-      items.push_back({ne * element_weight(c->epb_tab[0][0][1], ipow(P, c->nd), P), WorkItem{(int32_t)bi, (int32_t)f}});
-    }
-  }
-  if (items.empty()) return FR_OK;
-  std::stable_sort(items.begin(), items.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
-  std::vector<WorkItem> h(items.size());
-  for (size_t i = 0; i < items.size(); ++i) h[i] = items[i].second;
-  void* d = nullptr;
-  if (cudaMalloc(&d, sizeof(WorkItem) * h.size()) != cudaSuccess) {
-    cudaGetLastError();  // out of memory: launches go per bucket instead
-    return FR_ERR_NOMEM;
-  }
-  if (cudaMemcpy(d, h.data(), sizeof(WorkItem) * h.size(), cudaMemcpyHostToDevice) != cudaSuccess) {
-    cudaFree(d);
-    return cuda_check(cudaGetLastError(), "work table upload");
-  }
-  c->d_work = static_cast<WorkItem*>(d);
-  c->n_work = (int)h.size();
-  return FR_OK;
-}
-
 void clear_work_cache(fr_ctx* c) {
   c->pc_ready = false;   // the layout or the tuning changed: blocks must be rebuilt
   clear_graphs(c);
-  rebuild_work_table(c);
-}
-
-// The fused JVP's tables: compact-trace bases of the buckets and, when every
-// face is interior and conforming, the neighbour of every element face with
-// the master / slave assignment of the face records (higher degree, then lower
-// element id, then lower face index).
-static fr_status build_fused_table(fr_ctx* c, const std::vector<int32_t>& elem_slot) {
-  const int nd = c->nd, nf = c->nf, E = c->E;
-  const int ct = c->visc ? 2 * c->nv : c->nv;
-  int64_t cb = 0;
-  std::vector<int> bucket_of_p(kMaxDeg + 1, -1);
-  for (size_t k = 0; k < c->buckets.size(); ++k) {
-    Bucket& b = c->buckets[k];
-    b.ctrace_base = cb;
-    cb += (int64_t)b.count * nf * ct * ipow(b.p + 1, nd - 1);
-    bucket_of_p[b.p] = (int)k;
-  }
-  c->fused_ok = c->bgroups.empty() && cb <= c->trace_cap;
-  // the compact face kernel finds a block at the trace-gradient offset scaled
-  // by ct / nvt: true when every bucket's compact base is its trace base so scaled
-  for (const auto& b : c->buckets)
-    if (b.trace_base % c->nvt != 0 || b.trace_base / c->nvt * ct != b.ctrace_base) c->fused_ok = false;
-  for (const auto& g : c->fgroups)
-    if (g.pm != g.ps) c->fused_ok = false;
-  if (!c->fused_ok) return FR_OK;
-  std::vector<FusedNbr> h((size_t)E * nf);
-  for (int s = 0; s < E; ++s) {
-    const int e = c->slot_elem[s];
-    for (int f = 0; f < nf; ++f) {
-      const int n = c->nbr[(size_t)e * nf + f];
-      const int g = c->nbr_face[(size_t)e * nf + f];
-      if (n < 0 || c->p[n] != c->p[e]) {
-        c->fused_ok = false;
-        return FR_OK;
-      }
-      const bool master = e < n || (e == n && f < g);
-      const Bucket& b = c->buckets[bucket_of_p[c->p[n]]];
-      FusedNbr r;
-      r.nloc = elem_slot[n] - b.slot_begin;
-      r.nelem = n;
-      r.g = g;
-      r.code = (int32_t)(uint8_t)c->orient[(size_t)e * nf + f] | (master ? 256 : 0);
-      h[(size_t)s * nf + f] = r;
-    }
-  }
-  if (!c->d_fnbr) FR_CUDA(cudaMalloc(&c->d_fnbr, sizeof(FusedNbr) * (size_t)E * nf));
-  FR_CUDA(cudaMemcpy(c->d_fnbr, h.data(), sizeof(FusedNbr) * h.size(), cudaMemcpyHostToDevice));
-  return FR_OK;
-}
-
-fr_status build_layout(fr_ctx* c) {
-  const int nd = c->nd, nv = c->nv, nf = c->nf, E = c->E;
-  c->pc_ready = false;
-  clear_graphs(c);
-  // free previous face groups
-  for (auto& g : c->fgroups) cudaFree(g.d_recs);
-  for (auto& g : c->bgroups) cudaFree(g.d_recs);
-  c->fgroups.clear();
-  c->bgroups.clear();
-  c->buckets.clear();
-  c->slot_elem.resize(E);
-  std::vector<int32_t> elem_slot(E);
-  int slot = 0;
-  int64_t sbase = 0, tbase = 0, obase = 0;
-  for (int p = c->p_min; p <= c->p_max; ++p) {
-    Bucket b;
-    b.p = p;
-    b.slot_begin = slot;
-    b.state_base = sbase;
-    b.trace_base = tbase;
-    b.out_base = obase;
-    for (int e = 0; e < E; ++e)
-      if (c->p[e] == p) {
-        elem_slot[e] = slot;
-        c->slot_elem[slot++] = e;
-      }
-    b.count = slot - b.slot_begin;
-    const int P = p + 1, NSP = ipow(P, nd), NFP = ipow(P, nd - 1);
-    sbase += (int64_t)b.count * nv * NSP;
-    tbase += (int64_t)b.count * nf * c->nvt * NFP;
-    obase += (int64_t)b.count * nf * 3 * nv * NFP;
-    if (b.count > 0) c->buckets.push_back(b);
-  }
-  c->n_dof = sbase;
-  // per-slot host tables
-  std::vector<int64_t> canon_off(E + 1, 0), state_off(E), trace_off(E), out_off(E);
-  for (int e = 0; e < E; ++e) canon_off[e + 1] = canon_off[e] + (int64_t)nv * ipow(c->p[e] + 1, nd);
-  std::vector<int64_t> slot_canon(E);
-  std::vector<int8_t> slot_p(E);
-  for (const auto& b : c->buckets) {
-    const int P = b.p + 1, NSP = ipow(P, nd), NFP = ipow(P, nd - 1);
-    for (int i = 0; i < b.count; ++i) {
-      const int s = b.slot_begin + i, e = c->slot_elem[s];
-      state_off[e] = b.state_base + (int64_t)i * nv * NSP;
-      trace_off[e] = b.trace_base + (int64_t)i * nf * c->nvt * NFP;
-      out_off[e] = b.out_base + (int64_t)i * nf * 3 * nv * NFP;
-      slot_canon[s] = canon_off[e];
-      slot_p[s] = (int8_t)b.p;
-    }
-  }
-  std::vector<int64_t> slot_state(E);
-  for (int s = 0; s < E; ++s) slot_state[s] = state_off[c->slot_elem[s]];
-  FR_CUDA(cudaMemcpy(c->d_slot_elem, c->slot_elem.data(), sizeof(int32_t) * E, cudaMemcpyHostToDevice));
-  FR_CUDA(cudaMemcpy(c->d_elem_slot, elem_slot.data(), sizeof(int32_t) * E, cudaMemcpyHostToDevice));
-  FR_CUDA(cudaMemcpy(c->d_canon_off, slot_canon.data(), sizeof(int64_t) * E, cudaMemcpyHostToDevice));
-  FR_CUDA(cudaMemcpy(c->d_state_off, slot_state.data(), sizeof(int64_t) * E, cudaMemcpyHostToDevice));
-  FR_CUDA(cudaMemcpy(c->d_slot_p, slot_p.data(), E, cudaMemcpyHostToDevice));
-
-  // faces: master = higher degree; ties -> lower element id, then lower face
-  std::map<std::pair<int, int>, std::vector<FaceRec>> inter;
-  std::map<std::pair<int, int>, std::vector<BndRec>> bnd;
-  for (int e = 0; e < E; ++e) {
-    const int pe = c->p[e];
-    const int NFPe = ipow(pe + 1, nd - 1);
-    for (int f = 0; f < nf; ++f) {
-      const int n = c->nbr[(size_t)e * nf + f];
-      const int64_t mt = trace_off[e] + (int64_t)f * c->nvt * NFPe;
-      const int64_t mo = out_off[e] + (int64_t)f * 3 * nv * NFPe;
-      if (n < 0) {
-        bnd[{pe, n}].push_back(BndRec{mt, mo, e, f});
-        continue;
-      }
-      const int g = c->nbr_face[(size_t)e * nf + f];
-      const int pn = c->p[n];
-      const bool master = pe > pn || (pe == pn && (e < n || (e == n && f < g)));
-      if (!master) continue;
-      const int NFPn = ipow(pn + 1, nd - 1);
-      FaceRec r;
-      r.mt = mt;
-      r.mo = mo;
-      r.st = trace_off[n] + (int64_t)g * c->nvt * NFPn;
-      r.so = out_off[n] + (int64_t)g * 3 * nv * NFPn;
-      r.me = e;
-      r.se = n;
-      r.mf = f;
-      r.sf = g;
-      r.orient = c->orient[(size_t)e * nf + f];
-      auto& v = inter[{pe, pn}];
-      r.idx = (int32_t)v.size();
-      v.push_back(r);
-    }
-  }
-  for (auto& kv : inter) {
-    // master-face direction as the major key (element order kept within a
-    // direction): warps then see one normal axis, which the diagonal-metric
-    // face kernel branches on
-    std::stable_sort(kv.second.begin(), kv.second.end(),
-                     [](const FaceRec& a, const FaceRec& b) { return (a.mf >> 1) < (b.mf >> 1); });
-    FaceGroup g;
-    g.pm = kv.first.first;
-    g.ps = kv.first.second;
-    g.n = (int)kv.second.size();
-    FR_CUDA(cudaMalloc(&g.d_recs, sizeof(FaceRec) * g.n));
-    FR_CUDA(cudaMemcpy(g.d_recs, kv.second.data(), sizeof(FaceRec) * g.n, cudaMemcpyHostToDevice));
-    c->fgroups.push_back(g);
-  }
-  for (auto& kv : bnd) {
-    BndGroup g;
-    g.p = kv.first.first;
-    g.kind = kv.first.second;
-    g.n = (int)kv.second.size();
-    FR_CUDA(cudaMalloc(&g.d_recs, sizeof(BndRec) * g.n));
-    FR_CUDA(cudaMemcpy(g.d_recs, kv.second.data(), sizeof(BndRec) * g.n, cudaMemcpyHostToDevice));
-    c->bgroups.push_back(g);
-  }
-  FR_TRY(build_fused_table(c, elem_slot));
-  rebuild_work_table(c);   // a failure leaves no table: launches go per bucket
-  return FR_OK;
+  cudaDeviceSynchronize();   // launches still reading the tile table
+  rebuild_work_table(c, nullptr);
+  cudaStreamSynchronize(nullptr);
 }
 
 template <typename T>
@@ -600,6 +397,7 @@ static fr_status create_impl(const fr_mesh_desc* m, const fr_physics* ph, const 
   FR_CUDA(cudaMalloc(&c->d_status, sizeof(int)));
   FR_CUDA(cudaMemset(c->d_status, 0, sizeof(int)));
   FR_CUDA(cudaMemcpy(c->d_nbr, c->nbr.data(), sizeof(int32_t) * E * nf, cudaMemcpyHostToDevice));
+  FR_TRY(layout_alloc(c));
   return build_layout(c);
 }
 
@@ -634,12 +432,16 @@ static void destroy_impl(fr_ctx* c) {
   cudaFree(c->d_state_off);
   cudaFree(c->d_slot_p);
   cudaFree(c->d_nbr);
-  for (auto& g : c->fgroups) cudaFree(g.d_recs);
-  for (auto& g : c->bgroups) cudaFree(g.d_recs);
   clear_graphs(c);
+  cudaFree(c->d_p);
+  cudaFree(c->d_nbr_face);
+  cudaFree(c->d_orient);
+  cudaFree(c->d_recs);
+  cudaFree(c->d_brecs);
+  cudaFree(c->d_lay);
+  cudaFree(c->d_face_hist);
+  if (c->h_lay) cudaFreeHost(c->h_lay);
   cudaFree(c->d_work);
-  c->d_work = nullptr;
-  c->n_work = 0;
   cudaFree(c->d_fnbr);
   cudaFree(c->d_status);
   cudaFree(c->d_jidx);
@@ -659,14 +461,11 @@ static void destroy_impl(fr_ctx* c) {
   cudaFree(c->d_gm);
   if (c->h_gm) cudaFreeHost(c->h_gm);
   cudaFree(c->d_xfer);
-  cudaFree(c->d_adapt_i32);
   cudaFree(c->d_adapt_i8);
   cudaFree(c->d_adapt_f64);
   cudaFree(c->d_old_state_off);
-  cudaFree(c->d_new_state_off);
   cudaFree(c->d_old_elem_slot);
   cudaFree(c->d_old_slot_p);
-  if (c->h_flag) cudaFreeHost(c->h_flag);
   delete c;
 }
 

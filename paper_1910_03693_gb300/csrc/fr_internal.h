@@ -51,7 +51,7 @@ struct FaceRec {
   int64_t mt, st, mo, so;
   int32_t me, se;      // element ids (geometry lookup)
   int32_t mf, sf;      // face indices
-  int32_t orient, idx; // master's orientation code; index of the face in its group
+  int32_t orient, pad; // master's orientation code
 };
 struct BndRec {
   int64_t mt, mo;
@@ -186,7 +186,6 @@ struct fr_ctx {
   bool df_ready = false;
   // layout
   std::vector<frgb::Bucket> buckets;     // one per degree present, ascending p
-  std::vector<int32_t> slot_elem;        // bucket position -> element id
   int64_t n_dof = 0, n_dof_cap = 0;
   int32_t* d_slot_elem = nullptr;        // [E]
   int64_t* d_canon_off = nullptr;        // [E] canonical offset of the element at each slot
@@ -201,6 +200,15 @@ struct fr_ctx {
   void* d_fout = nullptr;
   void* d_fbar = nullptr;                // VJP: adjoints of the face outputs
   void* d_trbar = nullptr;               // VJP: adjoints of the traces
+  // layout tables (layout.cu), sized by the mesh alone
+  int8_t* d_p = nullptr;                 // [E] current degree of every element
+  int8_t* d_nbr_face = nullptr;          // [E][nf]
+  int8_t* d_orient = nullptr;            // [E][nf]
+  frgb::FaceRec* d_recs = nullptr;       // interior faces, grouped
+  frgb::BndRec* d_brecs = nullptr;       // boundary faces, grouped
+  void* d_lay = nullptr;                 // counts read back by the host, sort scratch
+  int* d_face_hist = nullptr;            // face sort scratch
+  void* h_lay = nullptr;                 // pinned mirror of the counts, then the degrees
   // faces
   std::vector<frgb::FaceGroup> fgroups;
   std::vector<frgb::BndGroup> bgroups;
@@ -234,9 +242,8 @@ struct fr_ctx {
   // tables of the multi-bucket launch by (precision, kind)
   int epb_tab[2][3][frgb::kPM + 1] = {};
   bool multi_launch = true;
-  // work table of the multi-bucket launch (the same for every precision and
-  // kernel kind), rebuilt eagerly whenever the layout or the weight model
-  // changes, so that no launch ever allocates it
+  // tile table of the multi-bucket launch (the same for every precision and
+  // kernel kind), filled again whenever the layout or the weight model changes
   frgb::WorkItem* d_work = nullptr;
   int n_work = 0;
   // fused JVP: every face interior and conforming (then the exact JVP runs as
@@ -275,21 +282,25 @@ struct fr_ctx {
   int* h_jidx = nullptr;                        // pinned, h_jidx[j] = j
   // adaptation workspaces (lazily allocated)
   double* d_xfer = nullptr;              // prolongation / projection matrices [Po][Pn][6][6]
-  int* d_adapt_i32 = nullptr;
   int8_t* d_adapt_i8 = nullptr;
   double* d_adapt_f64 = nullptr;
   int64_t* d_old_state_off = nullptr;
-  int64_t* d_new_state_off = nullptr;
   int32_t* d_old_elem_slot = nullptr;
   int8_t* d_old_slot_p = nullptr;
-  int* h_flag = nullptr;
 };
 
 namespace frgb {
 // threads a CTA of the element kernels should use on this mesh
 inline int mesh_threads(const fr_ctx* c) { return spread_threads(c->n_dof / c->nv, 256, c->sms); }
 void clear_work_cache(fr_ctx* c);
-fr_status rebuild_work_table(fr_ctx* c);
+fr_status rebuild_work_table(fr_ctx* c, cudaStream_t s);
+// layout.cu
+fr_status layout_alloc(fr_ctx* c);
+fr_status layout_device(fr_ctx* c, const int8_t* d_p, cudaStream_t s);
+fr_status layout_host(fr_ctx* c, cudaStream_t s);
+fr_status build_layout(fr_ctx* c);
+const int8_t* layout_degrees(const fr_ctx* c);
+const int64_t* layout_n_dof(const fr_ctx* c);
 void clear_graphs(fr_ctx* c);
 void collect_graph_timers(fr_ctx* c);
 // launchers (kernels_*.cu)

@@ -454,13 +454,15 @@ fr_status fr_precond_build(fr_ctx* c, const double* q64_dev, double sigma, void*
   // block offsets per slot (floats), -1 for blocks larger than kPcMax
   std::vector<int64_t> off(E, -1);
   std::vector<int32_t> slot_color(E);
+  int next[kMaxDeg + 1] = {};   // next slot of each degree: slots hold the elements in (p, id) order
+  for (const auto& b : c->buckets) next[b.p] = b.slot_begin;
+  for (int el = 0; el < E; ++el) slot_color[next[c->p[el]]++] = c->color[el];
   int64_t total = 0;
   int kmax = 0;
   for (const auto& b : c->buckets) {
     const int nb = nv * nsp_host(nd, b.p);
     for (int i = 0; i < b.count; ++i) {
       const int sl = b.slot_begin + i;
-      slot_color[sl] = c->color[c->slot_elem[sl]];
       if (nb <= kPcMax) {
         off[sl] = total;
         total += (int64_t)nb * nb;
