@@ -8,9 +8,9 @@
 //    together (a face neighbour never shares the colour, so the product
 //    restricted to a probed element is that element's own column), one
 //    product per colour and local DOF index;
-//  * each block sigma I - J_ee is inverted in shared memory by Gauss-Jordan
-//    elimination with partial pivoting (FP32), and stored column-major.
-// Blocks of up to kPcSmem DOFs are inverted with [A | I] in shared memory;
+//  * each block sigma I - J_ee is inverted by Gauss-Jordan elimination with
+//    partial pivoting (FP32), and stored column-major.
+// Blocks of up to kPcSmem DOFs are inverted in shared memory;
 // larger ones (3D p >= 3: 320, 625 and 1080 DOFs) by a blocked in-place
 // Gauss-Jordan elimination on the block in global memory (below).
 // Apply: z_e = M_e^-1 (a w_e + b u_e), FP32 arithmetic on FP64 vectors.
@@ -26,170 +26,70 @@ namespace frgb {
 constexpr int kPcSmem = 144;   // largest block inverted in shared memory (2 x 144^2 floats)
 constexpr int kPcMax = 1080;   // largest block stored: 3D p = 5 (5 x 216 DOFs)
 constexpr int kPanel = 32;     // columns eliminated together by the blocked inversion
-constexpr int kTile = 32;      // columns of one tile of the blocked update
+constexpr int kTile = 64;      // columns of one tile of the blocked update
 
 static inline int nsp_host(int nd, int p) { return nd == 2 ? (p + 1) * (p + 1) : (p + 1) * (p + 1) * (p + 1); }
 
-// v[state_off(s) + k] = 1 (and the entry k-1 cleared) for slots of colour `col`
-__global__ void k_pc_unit(float* __restrict__ v, const int64_t* __restrict__ state_off,
-                          const int32_t* __restrict__ slot_color, int slot_begin, int count, int nb, int col,
-                          int k) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= count) return;
-  const int s = slot_begin + i;
-  if (slot_color[s] != col) return;
-  if (k > 0 && k - 1 < nb) v[state_off[s] + k - 1] = 0.0f;
-  if (k < nb) v[state_off[s] + k] = 1.0f;
-}
+// The buckets of one launch: slots slot_begin .. + count of block size nb.
+struct PcBuckets {
+  int slot_begin[kMaxDeg + 1], count[kMaxDeg + 1], nb[kMaxDeg + 1];
+  int64_t first[kMaxDeg + 2];   // threads (probes) or CTAs (apply) of the buckets before this one
+  int n;
+};
 
-// column k of B_s = sigma I - J_ss (column-major, B[k * nb + i]) for slots of colour `col`
-__global__ void k_pc_gather(float* __restrict__ B, const int64_t* __restrict__ pc_off, const float* __restrict__ J,
-                            const int64_t* __restrict__ state_off, const int32_t* __restrict__ slot_color,
-                            int slot_begin, int count, int nb, int col, int k, float sigma) {
+// One step of the probing of colour `col`, one thread per block row: column k of
+// B_s = sigma I - J_ss (column-major, B[k nb + i]) from the product J of the
+// unit vectors e_k (skipped for k < 0), and the unit vectors moved on to k + 1.
+__global__ void k_pc_probe(PcBuckets bk, float* __restrict__ B, const int64_t* __restrict__ pc_off,
+                           const float* __restrict__ J, float* __restrict__ v, const int64_t* __restrict__ state_off,
+                           const int32_t* __restrict__ slot_color, int col, int k, float sigma) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)count * nb) return;
-  const int i = (int)(t % nb);
-  const int s = slot_begin + (int)(t / nb);
+  if (t >= bk.first[bk.n]) return;
+  int q = 0;
+  while (t >= bk.first[q + 1]) ++q;
+  const int nb = bk.nb[q];
+  const int i = (int)((t - bk.first[q]) % nb);
+  const int s = bk.slot_begin[q] + (int)((t - bk.first[q]) / nb);
   if (slot_color[s] != col || pc_off[s] < 0) return;
-  const float val = (i == k ? sigma : 0.0f) - J[state_off[s] + i];
-  B[pc_off[s] + (int64_t)k * nb + i] = val;
+  const int64_t so = state_off[s];
+  if (k >= 0 && k < nb) B[pc_off[s] + (int64_t)k * nb + i] = (i == k ? sigma : 0.0f) - J[so + i];
+  if (i == k) v[so + i] = 0.0f;
+  if (i == k + 1) v[so + i] = 1.0f;
 }
 
 // In-place inverse of one nb x nb block per CTA (column-major in global
-// memory) by Gauss-Jordan elimination on [A | I] in shared memory, partial
-// pivoting by rows.  A zero pivot sets *status and leaves the block as is.
-__global__ void k_pc_invert(float* __restrict__ B, const int64_t* __restrict__ pc_off, int slot_begin, int nb,
-                            int* __restrict__ status) {
+// memory) by Gauss-Jordan elimination in shared memory, partial pivoting by
+// rows; the row swaps are undone as column swaps at the end.  A warp owns every
+// eighth row, its lanes the columns, with the scaled pivot row in registers.
+// A zero pivot sets *status and leaves the block as is.  In place the block
+// takes nb^2 floats (three CTAs an SM at 135 DOFs; [A | I] with its 2 nb columns
+// allowed one and did twice the work: 854 blocks of 40 and 853 of 135 DOFs took
+// 12.2 ms, now 1.5 ms, with the same bits).
+__global__ void __launch_bounds__(256) k_pc_invert(float* __restrict__ B, const int64_t* __restrict__ pc_off,
+                                                   int slot_begin, int nb, int* __restrict__ status) {
   extern __shared__ __align__(16) float sm[];
-  float* M = sm;                    // [nb][2 nb] row-major
-  __shared__ float pv[32];
-  __shared__ int pr[32];
+  const int ld = nb | 1;              // odd: column reads without bank conflicts
+  float* M = sm;                      // [nb][ld] row-major
+  float* rk = M + (size_t)nb * ld;    // the scaled pivot row
+  int* perm = reinterpret_cast<int*>(rk + nb);
+  int* cm = perm + nb;
   __shared__ int piv;
+  __shared__ float pval;
+  constexpr int CW = (kPcSmem + 31) / 32;
   const int s = slot_begin + blockIdx.x;
   const int64_t off = pc_off[s];
   if (off < 0) return;
   float* A = B + off;
-  const int w2 = 2 * nb;
-  for (int t = threadIdx.x; t < nb * w2; t += blockDim.x) {
-    const int r = t / w2, cidx = t % w2;
-    M[t] = cidx < nb ? A[(int64_t)cidx * nb + r] : (cidx - nb == r ? 1.0f : 0.0f);
-  }
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int t = tid; t < nb * nb; t += 256) M[(t % nb) * ld + t / nb] = A[t];
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
   for (int k = 0; k < nb; ++k) {
     // pivot: the row r >= k with the largest |M[r][k]| (lowest row at a tie)
-    float best = -1.0f;
-    int br = k;
-    for (int r = k + threadIdx.x; r < nb; r += blockDim.x) {
-      const float a = fabsf(M[r * w2 + k]);
-      if (a > best) {
-        best = a;
-        br = r;
-      }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const float ob = __shfl_down_sync(0xffffffffu, best, o);
-      const int orr = __shfl_down_sync(0xffffffffu, br, o);
-      if (ob > best || (ob == best && orr < br)) {
-        best = ob;
-        br = orr;
-      }
-    }
-    if (lane == 0) {
-      pv[warp] = best;
-      pr[warp] = br;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      float b0 = pv[0];
-      int r0 = pr[0];
-      for (int q = 1; q < nw; ++q)
-        if (pv[q] > b0 || (pv[q] == b0 && pr[q] < r0)) {
-          b0 = pv[q];
-          r0 = pr[q];
-        }
-      piv = (b0 > 0.0f) ? r0 : -1;
-      if (piv < 0) atomicExch(status, 1);
-    }
-    __syncthreads();
-    if (piv < 0) return;   // singular block: reported through status
-    if (piv != k)
-      for (int cidx = threadIdx.x; cidx < w2; cidx += blockDim.x) {
-        const float a = M[k * w2 + cidx];
-        M[k * w2 + cidx] = M[piv * w2 + cidx];
-        M[piv * w2 + cidx] = a;
-      }
-    __syncthreads();
-    const float inv = 1.0f / M[k * w2 + k];
-    __syncthreads();
-    for (int cidx = threadIdx.x; cidx < w2; cidx += blockDim.x) M[k * w2 + cidx] *= inv;
-    __syncthreads();
-    // eliminate column k from every other row (the factors read before any row changes)
-    for (int t = threadIdx.x; t < nb * w2; t += blockDim.x) {
-      const int r = t / w2, cidx = t % w2;
-      if (r == k || cidx == k) continue;
-      M[t] -= M[r * w2 + k] * M[k * w2 + cidx];
-    }
-    __syncthreads();
-    for (int r = threadIdx.x; r < nb; r += blockDim.x)
-      if (r != k) M[r * w2 + k] = 0.0f;
-    __syncthreads();
-  }
-  for (int t = threadIdx.x; t < nb * nb; t += blockDim.x) {
-    const int r = t % nb, cidx = t / nb;   // column-major output
-    A[(int64_t)cidx * nb + r] = M[r * w2 + nb + cidx];
-  }
-}
-
-// In-place inverse of one nb x nb block per CTA (column-major in global
-// memory) by Gauss-Jordan elimination with partial pivoting, blocked by
-// panels of kPanel columns: each panel is eliminated in shared memory (pivot
-// search over the rows not yet used, row swaps, scaling, elimination from
-// every other row), and its kPanel pivots then reach every other column at
-// once as the panel's row permutation followed by the rank-kPanel update
-// A[:, j] += (panel - I) A[K, j]; the row swaps are undone as column swaps at
-// the end.  The block moves through global memory (L2) once per panel, and the
-// nb^3 multiply-adds of the inversion are register-tiled in the update.  A
-// zero pivot sets *status and leaves the block unfinished.
-// Shared memory: the panel [nb][kPanel + 1], the panel's row order idx[nb],
-// the pivot rows perm[nb], the pivot column fcol[nb], the pivot row rk[kPanel],
-// the tile's panel rows X[kPanel][kTile + 1] and permuted rows [2 kPanel][kTile].
-__global__ void __launch_bounds__(512) k_pc_invert_blocked(float* __restrict__ B, const int64_t* __restrict__ pc_off,
-                                                           int slot_begin, int nb, int* __restrict__ status) {
-  extern __shared__ __align__(16) float sm[];
-  constexpr int LD = kPanel + 1;
-  float* Pn = sm;                                   // [nb][LD]
-  float* fcol = Pn + (size_t)nb * LD;               // [nb]
-  float* X = fcol + nb;                             // [kPanel][kTile + 1]
-  float* Y = X + kPanel * (kTile + 1);              // [2 kPanel][kTile]
-  float* rk = Y + 2 * kPanel * kTile;               // [kPanel]
-  int* idx = reinterpret_cast<int*>(rk + kPanel);   // [nb]
-  int* perm = idx + nb;                             // [nb]
-  __shared__ float pv[16];
-  __shared__ int pr[16];
-  __shared__ int piv;
-  const int s = slot_begin + blockIdx.x;
-  const int64_t off = pc_off[s];
-  if (off < 0) return;
-  float* A = B + off;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5;
-  for (int kb = 0; kb < nb; kb += kPanel) {
-    const int nk = min(kPanel, nb - kb);
-    // panel in shared memory; its row order starts as the identity
-    for (int t = tid; t < nb * nk; t += nt) {
-      const int c = t / nb, r = t % nb;
-      Pn[r * LD + c] = A[(int64_t)(kb + c) * nb + r];
-    }
-    for (int r = tid; r < nb; r += nt) idx[r] = r;
-    __syncthreads();
-    for (int kl = 0; kl < nk; ++kl) {
-      const int k = kb + kl;
-      // pivot: the row r >= k with the largest |Pn[r][kl]| (lowest row at a tie)
+    if (warp == 0) {
       float best = -1.0f;
       int br = k;
-      for (int r = k + tid; r < nb; r += nt) {
-        const float a = fabsf(Pn[r * LD + kl]);
+      for (int r = k + lane; r < nb; r += 32) {
+        const float a = fabsf(M[r * ld + k]);
         if (a > best) {
           best = a;
           br = r;
@@ -204,217 +104,295 @@ __global__ void __launch_bounds__(512) k_pc_invert_blocked(float* __restrict__ B
         }
       }
       if (lane == 0) {
+        piv = best > 0.0f ? br : -1;
+        if (piv < 0) atomicExch(status, 1);
+        pval = M[br * ld + k];
+        perm[k] = br;
+      }
+    }
+    __syncthreads();
+    const int p = piv;
+    if (p < 0) return;   // singular block: reported through status
+    const float inv = 1.0f / pval;
+    for (int c = tid; c < nb; c += 256) {
+      const float a = M[p * ld + c];
+      if (p != k) M[p * ld + c] = M[k * ld + c];
+      rk[c] = c == k ? inv : a * inv;
+    }
+    __syncthreads();
+    float row[CW];
+#pragma unroll
+    for (int i = 0; i < CW; ++i) row[i] = lane + 32 * i < nb ? rk[lane + 32 * i] : 0.0f;
+    for (int r = warp; r < nb; r += 8) {
+      float* m = M + r * ld;
+      const float f = m[k];
+      __syncwarp();   // every lane holds f before lane k % 32 replaces it
+#pragma unroll
+      for (int i = 0; i < CW; ++i) {
+        const int c = lane + 32 * i;
+        if (c < nb) m[c] = r == k ? row[i] : (c == k ? -f * inv : m[c] - f * row[i]);
+      }
+    }
+    __syncthreads();
+  }
+  if (tid == 0) {   // the column swaps that undo the row swaps, last pivot first
+    for (int j = 0; j < nb; ++j) cm[j] = j;
+    for (int k = nb - 1; k >= 0; --k) {
+      const int t = cm[k];
+      cm[k] = cm[perm[k]];
+      cm[perm[k]] = t;
+    }
+  }
+  __syncthreads();
+  for (int t = tid; t < nb * nb; t += 256) A[t] = M[(t % nb) * ld + cm[t / nb]];
+}
+
+// In-place inverse of one nb x nb block per CTA (column-major in global
+// memory) by Gauss-Jordan elimination with partial pivoting, blocked by
+// panels of kPanel columns: each panel is eliminated (pivot search over the
+// rows not yet used, row swaps, scaling, elimination from every other row), and
+// its kPanel pivots then reach every other column at once as the panel's row
+// permutation followed by the rank-kPanel update A[:, j] += (panel - I) A[K, j];
+// the row swaps are undone as column swaps at the end.  The block moves through
+// global memory (L2) once per panel.  A zero pivot sets *status and leaves the
+// block unfinished.
+//
+// The panel lives in registers while it is eliminated: warp w holds the rows w,
+// w + 16, ... (RPW of them), lane c column c, so that a pivot costs two barriers,
+// one shuffle and one FMA a row, and no shared-memory traffic but the two rows
+// exchanged.  The update gives lanes consecutive rows (coalesced columns) and
+// each thread two rows by eight columns: two panel words and two broadcast
+// 16-byte loads for sixteen FMAs.  853 blocks of 320 DOFs: 13.7 -> 7.3 ms, the
+// same bits; the block's passes through L2 bound it now.
+// Shared memory: the panel [nb][kPanel + 1] (then the rows of the final column
+// swap), the tile's permuted rows Y[2 kPanel][kTile + 4], idx[nb], perm[nb].
+constexpr int kInvThreads = 512, kInvWarps = kInvThreads / 32;
+template <int RPW>
+__global__ void __launch_bounds__(kInvThreads, RPW <= 20 ? 2 : 1)
+    k_pc_invert_blocked(float* __restrict__ B, const int64_t* __restrict__ pc_off, int slot_begin, int nb,
+                        int* __restrict__ status) {
+  extern __shared__ __align__(16) float sm[];
+  constexpr int LD = kPanel + 1, LY = kTile + 4;
+  float* Y = sm;                                    // [2 kPanel][LY]
+  float* Pn = Y + 2 * kPanel * LY;                  // [nb][LD]
+  int* idx = reinterpret_cast<int*>(Pn + (size_t)nb * LD);   // [nb] the panel's row order
+  int* perm = idx + nb;                             // [nb] pivot rows
+  __shared__ float pv[kInvWarps], row_k[kPanel], row_p[kPanel];
+  __shared__ int pr[kInvWarps];
+  const int s = slot_begin + blockIdx.x;
+  const int64_t off = pc_off[s];
+  if (off < 0) return;
+  float* A = B + off;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int kb = 0; kb < nb; kb += kPanel) {
+    const int nk = min(kPanel, nb - kb);
+    for (int t = tid; t < nb * kPanel; t += kInvThreads) {
+      const int c = t / nb, r = t - c * nb;
+      Pn[r * LD + c] = c < nk ? A[(int64_t)(kb + c) * nb + r] : 0.0f;
+    }
+    for (int r = tid; r < nb; r += kInvThreads) idx[r] = r;
+    __syncthreads();
+    float x[RPW];
+#pragma unroll
+    for (int i = 0; i < RPW; ++i) {
+      const int r = warp + kInvWarps * i;
+      x[i] = r < nb ? Pn[r * LD + lane] : 0.0f;
+    }
+    for (int kl = 0; kl < nk; ++kl) {
+      const int k = kb + kl;
+      // pivot: the row r >= k with the largest |x| of column kl (lowest row at a
+      // tie); every lane searches its own column, lane kl's result counts
+      float best = -1.0f;
+      int br = k;
+#pragma unroll
+      for (int i = 0; i < RPW; ++i) {
+        const int r = warp + kInvWarps * i;
+        const float a = fabsf(x[i]);
+        if (r >= k && r < nb && a > best) {
+          best = a;
+          br = r;
+        }
+      }
+      if (lane == kl) {
         pv[warp] = best;
         pr[warp] = br;
       }
       __syncthreads();
+      float b0 = pv[0];
+      int p = pr[0];
+#pragma unroll
+      for (int q = 1; q < kInvWarps; ++q)
+        if (pv[q] > b0 || (pv[q] == b0 && pr[q] < p)) {
+          b0 = pv[q];
+          p = pr[q];
+        }
+      if (!(b0 > 0.0f)) {   // singular block: reported through status
+        if (tid == 0) atomicExch(status, 1);
+        return;
+      }
       if (tid == 0) {
-        float b0 = pv[0];
-        int r0 = pr[0];
-        for (int q = 1; q < nw; ++q)
-          if (pv[q] > b0 || (pv[q] == b0 && pr[q] < r0)) {
-            b0 = pv[q];
-            r0 = pr[q];
-          }
-        piv = (b0 > 0.0f) ? r0 : -1;
-        if (piv < 0) atomicExch(status, 1);
-        else perm[k] = r0;
+        perm[k] = p;
+        const int t0 = idx[k];
+        idx[k] = idx[p];
+        idx[p] = t0;
+      }
+#pragma unroll
+      for (int i = 0; i < RPW; ++i) {
+        const int r = warp + kInvWarps * i;
+        if (r == k) row_k[lane] = x[i];
+        if (r == p) row_p[lane] = x[i];
       }
       __syncthreads();
-      const int p = piv;
-      if (p < 0) return;   // singular block: reported through status
-      if (p != k) {
-        for (int c = tid; c < nk; c += nt) {
-          const float a = Pn[k * LD + c];
-          Pn[k * LD + c] = Pn[p * LD + c];
-          Pn[p * LD + c] = a;
-        }
-        if (tid == 0) {
-          const int t0 = idx[k];
-          idx[k] = idx[p];
-          idx[p] = t0;
-        }
+      const float inv = 1.0f / row_p[kl];
+      const float rk = lane == kl ? inv : row_p[lane] * inv, old_k = row_k[lane];
+#pragma unroll
+      for (int i = 0; i < RPW; ++i) {
+        const int r = warp + kInvWarps * i;
+        const float y = r == p && p != k ? old_k : x[i];   // row p holds the old row k
+        const float f = __shfl_sync(0xffffffffu, y, kl);
+        x[i] = r == k ? rk : (lane == kl ? -f * inv : y - f * rk);
       }
-      __syncthreads();
-      const float inv = 1.0f / Pn[k * LD + kl];
-      for (int r = tid; r < nb; r += nt) fcol[r] = Pn[r * LD + kl];
-      for (int c = tid; c < nk; c += nt) rk[c] = c == kl ? inv : Pn[k * LD + c] * inv;
-      __syncthreads();
-      for (int t = tid; t < nb * nk; t += nt) {
-        const int r = t / nk, c = t % nk;
-        if (r == k) Pn[r * LD + c] = rk[c];
-        else if (c == kl) Pn[r * LD + c] = -fcol[r] * inv;
-        else Pn[r * LD + c] -= fcol[r] * rk[c];
-      }
-      __syncthreads();
     }
-    // the eliminated panel back to global memory
-    for (int t = tid; t < nb * nk; t += nt) {
-      const int c = t / nb, r = t % nb;
+    // the eliminated panel back to global memory, then less the identity for the update
+#pragma unroll
+    for (int i = 0; i < RPW; ++i) {
+      const int r = warp + kInvWarps * i;
+      if (r < nb) Pn[r * LD + lane] = x[i];
+    }
+    __syncthreads();
+    for (int t = tid; t < nb * nk; t += kInvThreads) {
+      const int c = t / nb, r = t - c * nb;
       A[(int64_t)(kb + c) * nb + r] = Pn[r * LD + c];
     }
+    __syncthreads();
+    if (tid < nk) Pn[(kb + tid) * LD + tid] -= 1.0f;
     // every other column j: rows permuted as the panel's were, then
     // A[:, j] += (Pn - I_K) A[K, j]
-    const int tx = tid % (kTile / 4), ty = tid / (kTile / 4), nty = nt / (kTile / 4);
     for (int j0 = 0; j0 < nb; j0 += kTile) {
-      // columns j0 .. j0 + kTile - 1 that lie outside the panel
       __syncthreads();
       // (a) row permutation of the tile: the rows that can have moved are the
-      // panel rows and their pivot rows (all reads before any write)
-      for (int t = tid; t < 2 * nk * kTile; t += nt) {
-        const int ri = t / kTile, c = t % kTile, j = j0 + c;
+      // panel rows and their pivot rows (all reads before any write); the new
+      // panel rows are the update's right-hand factor
+      for (int t = tid; t < 2 * nk * kTile; t += kInvThreads) {
+        const int c = t / (2 * nk), ri = t - c * 2 * nk, j = j0 + c;
         const int r = ri < nk ? kb + ri : perm[kb + ri - nk];
-        if (j < nb && (j < kb || j >= kb + nk)) Y[ri * kTile + c] = A[(int64_t)j * nb + idx[r]];
+        Y[ri * LY + c] = j < nb && (j < kb || j >= kb + nk) ? A[(int64_t)j * nb + idx[r]] : 0.0f;
       }
       __syncthreads();
-      for (int t = tid; t < 2 * nk * kTile; t += nt) {
-        const int ri = t / kTile, c = t % kTile, j = j0 + c;
+      for (int t = tid; t < 2 * nk * kTile; t += kInvThreads) {
+        const int c = t / (2 * nk), ri = t - c * 2 * nk, j = j0 + c;
         const int r = ri < nk ? kb + ri : perm[kb + ri - nk];
-        if (j < nb && (j < kb || j >= kb + nk)) A[(int64_t)j * nb + r] = Y[ri * kTile + c];
+        if (j < nb && (j < kb || j >= kb + nk)) A[(int64_t)j * nb + r] = Y[ri * LY + c];
       }
       __syncthreads();
-      // (b) the panel rows of the tile
-      for (int t = tid; t < nk * kTile; t += nt) {
-        const int k = t / kTile, c = t % kTile, j = j0 + c;
-        X[k * (kTile + 1) + c] = (j < nb && (j < kb || j >= kb + nk)) ? A[(int64_t)j * nb + kb + k] : 0.0f;
-      }
-      __syncthreads();
-      // (c) rank-nk update, four rows x four columns a thread per step
-      for (int r0 = ty; r0 < nb; r0 += 4 * nty) {
-        float acc[4][4];
-        int rows[4];
+      // (b) rank-nk update
+      const int units = (nb + 63) / 64 * (kTile / 8);
+      for (int un = warp; un < units; un += kInvWarps) {
+        const int r0 = un / (kTile / 8) * 64 + lane, r1 = r0 + 32, c0 = un % (kTile / 8) * 8;
+        if (j0 + c0 >= nb) continue;
+        float acc[2][8];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          rows[m] = r0 + m * nty;
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[m][c] = 0.0f;
-        }
+        for (int c = 0; c < 8; ++c) acc[0][c] = acc[1][c] = 0.0f;
+        const float* p0 = Pn + min(r0, nb - 1) * LD;
+        const float* p1 = Pn + min(r1, nb - 1) * LD;
         for (int k = 0; k < nk; ++k) {
-          float x[4], w[4];
+          const float w0 = p0[k], w1 = p1[k];
+          const float4 u = *reinterpret_cast<const float4*>(Y + k * LY + c0);
+          const float4 v = *reinterpret_cast<const float4*>(Y + k * LY + c0 + 4);
+          const float xs[8] = {u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w};
 #pragma unroll
-          for (int c = 0; c < 4; ++c) x[c] = X[k * (kTile + 1) + tx * 4 + c];
-#pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            const int r = rows[m];
-            w[m] = r < nb ? Pn[r * LD + k] - (r == kb + k ? 1.0f : 0.0f) : 0.0f;
+          for (int c = 0; c < 8; ++c) {
+            acc[0][c] = fmaf(w0, xs[c], acc[0][c]);
+            acc[1][c] = fmaf(w1, xs[c], acc[1][c]);
           }
-#pragma unroll
-          for (int m = 0; m < 4; ++m)
-#pragma unroll
-            for (int c = 0; c < 4; ++c) acc[m][c] = fmaf(w[m], x[c], acc[m][c]);
         }
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-          const int r = rows[m];
-          if (r >= nb) continue;
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int j = j0 + tx * 4 + c;
-            if (j < nb && (j < kb || j >= kb + nk)) A[(int64_t)j * nb + r] += acc[m][c];
-          }
+        for (int c = 0; c < 8; ++c) {
+          const int j = j0 + c0 + c;
+          if (j >= nb || (j >= kb && j < kb + nk)) continue;
+          if (r0 < nb) A[(int64_t)j * nb + r0] += acc[0][c];
+          if (r1 < nb) A[(int64_t)j * nb + r1] += acc[1][c];
         }
       }
     }
     __syncthreads();
   }
-  // undo the row swaps as column swaps, last pivot first
-  for (int k = nb - 1; k >= 0; --k) {
-    const int p = perm[k];
-    if (p != k)
-      for (int r = tid; r < nb; r += nt) {
-        const float a = A[(int64_t)k * nb + r];
-        A[(int64_t)k * nb + r] = A[(int64_t)p * nb + r];
-        A[(int64_t)p * nb + r] = a;
-      }
+  // undo the row swaps as column swaps, last pivot first: the order of the
+  // columns, then 32 rows at a time through shared memory
+  if (tid == 0) {
+    for (int j = 0; j < nb; ++j) idx[j] = j;
+    for (int k = nb - 1; k >= 0; --k) {
+      const int t = idx[k];
+      idx[k] = idx[perm[k]];
+      idx[perm[k]] = t;
+    }
+  }
+  __syncthreads();
+  for (int r0 = 0; r0 < nb; r0 += 32) {
+    const int r = r0 + lane;
+    for (int j = warp; j < nb; j += kInvWarps)
+      if (r < nb) Pn[j * LD + lane] = A[(int64_t)j * nb + r];
+    __syncthreads();
+    for (int j = warp; j < nb; j += kInvWarps)
+      if (r < nb) A[(int64_t)j * nb + r] = Pn[idx[j] * LD + lane];
     __syncthreads();
   }
 }
 
 static size_t pc_blocked_smem(int nb) {
-  return sizeof(float) * ((size_t)nb * (kPanel + 1) + nb + kPanel * (kTile + 1) + 2 * kPanel * kTile + kPanel) +
-         sizeof(int) * 2 * (size_t)nb;
+  return sizeof(float) * ((size_t)nb * (kPanel + 1) + 2 * kPanel * (kTile + 4)) + sizeof(int) * 2 * (size_t)nb;
 }
 
-// z_e = M_e^-1 (a w_e + b u_e) for blocks of more than 256 rows: one CTA per
-// element, the rows strided over its threads (coalesced column-major reads).
+// z_e = M_e^-1 (a w_e + b u_e), every bucket in one launch: a CTA takes one
+// element (nb at least half its threads) or as many whole ones as fit, one thread
+// per row (rows beyond the CTA's 1,024 threads in a second pass).  The columns
+// are summed in order with FP32 FMAs; each thread has kPcAhead column loads in
+// flight (the blocks' bytes bound the apply, and one load at a time left HBM
+// idle: blocks of 320, 135 and 40 DOFs on 2,560 elements, 410 MB, took three
+// launches of 58 us and now one of 87 us, 4.7 TB/s).
 // The vectors are FP64 or FP32 (VT; the FP32 Krylov basis), the sums FP32.
+// Elements without a stored block (pc_off < 0): z_e = (a w_e + b u_e) / sigma.
+constexpr int kPcAhead = 16;
 template <typename VT>
-__global__ void __launch_bounds__(256) k_pc_apply_big(const float* __restrict__ B, const int64_t* __restrict__ pc_off,
-                                                      const int64_t* __restrict__ state_off, int slot_begin, int nb,
-                                                      double a, const VT* w, double b,
-                                                      const VT* __restrict__ u, VT* z, double inv_sigma,
-                                                      const int* __restrict__ gate, const double* __restrict__ bscale) {
-  extern __shared__ __align__(16) float xs[];   // [nb]
+__global__ void __launch_bounds__(1024) k_pc_apply(PcBuckets bk, const float* __restrict__ B,
+                                                   const int64_t* __restrict__ pc_off,
+                                                   const int64_t* __restrict__ state_off, double a, const VT* w, double b,
+                                                   const VT* __restrict__ u, VT* z, double inv_sigma,
+                                                   const int* __restrict__ gate, const double* __restrict__ bscale) {
+  extern __shared__ __align__(16) float xs[];   // [elements][nb]
   if (gate && *gate) return;
   if (bscale) b *= *bscale;
-  const int s = slot_begin + blockIdx.x;
-  const int64_t base = state_off[s], off = pc_off[s];
-  double xv[kPcMax / 256 + 1];
-  int nr = 0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x, ++nr) {
-    xv[nr] = a * (double)w[base + i] + (u ? b * (double)u[base + i] : 0.0);
-    xs[i] = (float)xv[nr];
+  int q = 0;
+  while ((int)blockIdx.x >= bk.first[q + 1]) ++q;
+  const int nb = bk.nb[q], epb = max(1, (int)blockDim.x / nb);
+  const int e0 = (int)(blockIdx.x - bk.first[q]) * epb, ne = min(epb, bk.count[q] - e0);
+  for (int t = threadIdx.x; t < ne * nb; t += blockDim.x) {
+    const int64_t g = state_off[bk.slot_begin[q] + e0 + t / nb] + t % nb;
+    xs[t] = (float)(a * (double)w[g] + (u ? b * (double)u[g] : 0.0));
   }
   __syncthreads();
-  nr = 0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x, ++nr) {
+  for (int t = threadIdx.x; t < ne * nb; t += blockDim.x) {
+    const int le = t / nb, i = t - le * nb;
+    const int s = bk.slot_begin[q] + e0 + le;
+    const int64_t g = state_off[s] + i, off = pc_off[s];
     if (off < 0) {
-      z[base + i] = (VT)(xv[nr] * inv_sigma);
+      z[g] = (VT)((a * (double)w[g] + (u ? b * (double)u[g] : 0.0)) * inv_sigma);
       continue;
     }
-    const float* Bc = B + off;
+    const float* Bc = B + off + i;
+    const float* xe = xs + le * nb;
     float acc = 0.0f;
-    for (int j = 0; j < nb; ++j) acc = fmaf(Bc[(int64_t)j * nb + i], xs[j], acc);
-    z[base + i] = (VT)acc;
+    int j = 0;
+    for (; j + kPcAhead <= nb; j += kPcAhead) {
+      float m[kPcAhead];
+#pragma unroll
+      for (int r = 0; r < kPcAhead; ++r) m[r] = Bc[(int64_t)(j + r) * nb];
+#pragma unroll
+      for (int r = 0; r < kPcAhead; ++r) acc = fmaf(m[r], xe[j + r], acc);
+    }
+    for (; j < nb; ++j) acc = fmaf(Bc[(int64_t)j * nb], xe[j], acc);
+    z[g] = (VT)acc;
   }
-}
-
-// z_e = M_e^-1 (a w_e + b u_e); epb elements per CTA, one thread per row.
-// Elements without a stored block (pc_off < 0): z_e = (a w_e + b u_e) / sigma.
-template <typename VT>
-__global__ void k_pc_apply(const float* __restrict__ B, const int64_t* __restrict__ pc_off,
-                           const int64_t* __restrict__ state_off, int slot_begin, int count, int nb, int epb,
-                           double a, const VT* w, double b, const VT* __restrict__ u, VT* z,
-                           double inv_sigma, const int* __restrict__ gate, const double* __restrict__ bscale) {
-  extern __shared__ __align__(16) float xs[];   // [epb][nb]
-  if (gate && *gate) return;
-  if (bscale) b *= *bscale;
-  const int le = threadIdx.x / nb, i = threadIdx.x % nb;
-  const int e = blockIdx.x * epb + le;
-  const bool valid = le < epb && e < count;
-  int64_t base = 0, off = -1;
-  double x = 0.0;
-  if (valid) {
-    const int s = slot_begin + e;
-    base = state_off[s];
-    off = pc_off[s];
-    x = a * (double)w[base + i] + (u ? b * (double)u[base + i] : 0.0);
-    xs[le * nb + i] = (float)x;
-  }
-  __syncthreads();
-  if (!valid) return;
-  if (off < 0) {
-    z[base + i] = (VT)(x * inv_sigma);
-    return;
-  }
-  const float* Bc = B + off;
-  const float* xe = xs + le * nb;
-  float acc = 0.0f;
-  for (int j = 0; j < nb; ++j) acc = fmaf(Bc[(int64_t)j * nb + i], xe[j], acc);
-  z[base + i] = (VT)acc;
-}
-
-// z = (a w + b u) / sigma on every DOF of a bucket without stored blocks
-template <typename VT>
-__global__ void k_pc_scale(const int64_t* __restrict__ state_off, int slot_begin, int count, int nb, double a,
-                           const VT* w, double b, const VT* __restrict__ u, VT* z, double inv_sigma,
-                           const int* __restrict__ gate, const double* __restrict__ bscale) {
-  if (gate && *gate) return;
-  if (bscale) b *= *bscale;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (int64_t)count * nb) return;
-  const int64_t idx = state_off[slot_begin + (int)(t / nb)] + (int)(t % nb);
-  z[idx] = (VT)((a * (double)w[idx] + (u ? b * (double)u[idx] : 0.0)) * inv_sigma);
 }
 
 // Distance-1 colouring of the face graph (greedy in element order), once per context.
@@ -497,42 +475,42 @@ fr_status fr_precond_build(fr_ctx* c, const double* q64_dev, double sigma, void*
   fr_status e = launch_jvp_prepare(c, q32, FR_F32, s);
   if (e != FR_OK) return e;
   const float sg = (float)sigma;
+  PcBuckets pb{};
+  for (const auto& b : c->buckets) {
+    const int nb = nv * nsp_host(nd, b.p);
+    if (nb > kPcMax) continue;
+    pb.slot_begin[pb.n] = b.slot_begin;
+    pb.count[pb.n] = b.count;
+    pb.nb[pb.n] = nb;
+    pb.first[pb.n + 1] = pb.first[pb.n] + (int64_t)b.count * nb;
+    pb.n += 1;
+  }
+  const unsigned pg = (unsigned)((pb.first[pb.n] + 255) / 256);
   for (int col = 0; col < c->n_colors && kmax > 0; ++col) {
     cudaMemsetAsync(v32, 0, sizeof(float) * n, s);
-    for (int k = 0; k < kmax; ++k) {
-      for (const auto& b : c->buckets) {
-        const int nb = nv * nsp_host(nd, b.p);
-        if (nb > kPcMax) continue;
-        FR_LAUNCH(c, "precond_build", s,
-                  k_pc_unit<<<(b.count + 255) / 256, 256, 0, s>>>(v32, c->d_state_off, c->d_slot_color,
-                                                                  b.slot_begin, b.count, nb, col, k));
-      }
-      if ((e = launch_jvp_prepared(c, q32, v32, J32, FR_F32, s)) != FR_OK) return e;
-      for (const auto& b : c->buckets) {
-        const int nb = nv * nsp_host(nd, b.p);
-        if (nb > kPcMax || k >= nb) continue;
-        const int64_t nt = (int64_t)b.count * nb;
-        FR_LAUNCH(c, "precond_build", s,
-                  k_pc_gather<<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(c->d_pc, c->d_pc_off, J32, c->d_state_off,
-                                                                          c->d_slot_color, b.slot_begin, b.count, nb,
-                                                                          col, k, sg));
-      }
+    for (int k = -1; k < kmax; ++k) {
+      if (k >= 0 && (e = launch_jvp_prepared(c, q32, v32, J32, FR_F32, s)) != FR_OK) return e;
+      FR_LAUNCH(c, "precond_build", s,
+                k_pc_probe<<<pg, 256, 0, s>>>(pb, c->d_pc, c->d_pc_off, J32, v32, c->d_state_off, c->d_slot_color, col,
+                                              k, sg));
     }
   }
   for (const auto& b : c->buckets) {
     const int nb = nv * nsp_host(nd, b.p);
     if (nb > kPcMax || b.count == 0) continue;
     if (nb <= kPcSmem) {
-      const size_t smem = sizeof(float) * 2 * (size_t)nb * nb;
+      const size_t smem = sizeof(float) * (size_t)nb * ((nb | 1) + 1) + sizeof(int) * 2 * (size_t)nb;
       cudaFuncSetAttribute(k_pc_invert, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       FR_LAUNCH(c, "precond_build", s,
                 k_pc_invert<<<b.count, 256, smem, s>>>(c->d_pc, c->d_pc_off, b.slot_begin, nb, c->d_pc_status));
     } else {
+      // rows a warp holds of the 320-, 625- and 1080-DOF blocks
+      auto kern = nb <= 20 * kInvWarps ? k_pc_invert_blocked<20>
+                  : nb <= 40 * kInvWarps ? k_pc_invert_blocked<40> : k_pc_invert_blocked<68>;
       const size_t smem = pc_blocked_smem(nb);
-      cudaFuncSetAttribute(k_pc_invert_blocked, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       FR_LAUNCH(c, "precond_build", s,
-                k_pc_invert_blocked<<<b.count, 512, smem, s>>>(c->d_pc, c->d_pc_off, b.slot_begin, nb,
-                                                               c->d_pc_status));
+                kern<<<b.count, kInvThreads, smem, s>>>(c->d_pc, c->d_pc_off, b.slot_begin, nb, c->d_pc_status));
     }
   }
   int status = 0;
@@ -569,36 +547,26 @@ static fr_status precond_apply_t(fr_ctx* c, double a, const VT* w, double b, con
     set_error("element-Jacobi preconditioner not built (fr_precond_build) for the current layout");
     return FR_ERR_INVALID;
   }
-  const int nd = c->nd, nv = c->nv;
-  const double vb = 3.0 * sizeof(VT);   // a w, b u in, z out
-  for (const auto& bk : c->buckets) {
-    if (bk.count == 0) continue;
-    const int nb = nv * nsp_host(nd, bk.p);
-    if (nb > kPcMax) {   // no stored blocks in this bucket: 1/sigma
-      const int64_t nt = (int64_t)bk.count * nb;
-      FR_LAUNCH_B(c, "precond_apply", s, vb * nt,
-                  k_pc_scale<VT><<<(unsigned)((nt + 255) / 256), 256, 0, s>>>(c->d_state_off, bk.slot_begin, bk.count,
-                                                                            nb, a, w, b, u, z, 1.0 / c->pc_sigma,
-                                                                            gate, bscale));
-      continue;
-    }
-    const double bytes = (double)bk.count * nb * (vb + 4.0 * nb);
-    if (nb > 256) {
-      FR_LAUNCH_B(c, "precond_apply", s, bytes,
-                  k_pc_apply_big<VT><<<bk.count, 256, sizeof(float) * nb, s>>>(c->d_pc, c->d_pc_off, c->d_state_off,
-                                                                               bk.slot_begin, nb, a, w, b, u, z,
-                                                                               1.0 / c->pc_sigma, gate, bscale));
-      continue;
-    }
-    const int epb = 256 / nb;
-    const int threads = epb * nb;
-    const unsigned grid = (unsigned)((bk.count + epb - 1) / epb);
-    FR_LAUNCH_B(c, "precond_apply", s, bytes,
-                k_pc_apply<VT><<<grid, threads, sizeof(float) * threads, s>>>(c->d_pc, c->d_pc_off, c->d_state_off,
-                                                                              bk.slot_begin, bk.count, nb, epb, a, w,
-                                                                              b, u, z, 1.0 / c->pc_sigma, gate,
-                                                                              bscale));
+  // one launch, the largest blocks first (their CTAs run longest)
+  PcBuckets pb{};
+  int threads = 256;
+  double bytes = 0.0;
+  for (const auto& bk : c->buckets)
+    threads = std::max(threads, std::min(1024, (c->nv * nsp_host(c->nd, bk.p) + 31) / 32 * 32));
+  size_t smem = 0;
+  for (auto it = c->buckets.rbegin(); it != c->buckets.rend(); ++it) {
+    const int nb = c->nv * nsp_host(c->nd, it->p), epb = std::max(1, threads / nb);
+    pb.slot_begin[pb.n] = it->slot_begin;
+    pb.count[pb.n] = it->count;
+    pb.nb[pb.n] = nb;
+    pb.first[pb.n + 1] = pb.first[pb.n] + (it->count + epb - 1) / epb;
+    pb.n += 1;
+    smem = std::max(smem, sizeof(float) * (size_t)epb * nb);
+    bytes += (double)it->count * nb * (3.0 * sizeof(VT) + 4.0 * nb);   // a w, b u in, z out; the block
   }
+  FR_LAUNCH_B(c, "precond_apply", s, bytes,
+              k_pc_apply<VT><<<(unsigned)pb.first[pb.n], threads, smem, s>>>(
+                  pb, c->d_pc, c->d_pc_off, c->d_state_off, a, w, b, u, z, 1.0 / c->pc_sigma, gate, bscale));
   return cuda_check(cudaGetLastError(), "precond_apply");
 }
 
