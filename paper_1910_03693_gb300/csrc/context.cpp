@@ -450,6 +450,7 @@ static void destroy_impl(fr_ctx* c) {
   cudaFree(c->d_krylov);
   cudaFree(c->d_krylov32);
   cudaFree(c->d_step);
+  free_pc_lanes(c);
   cudaFree(c->d_pc);
   cudaFree(c->d_pc_off);
   cudaFree(c->d_slot_color);

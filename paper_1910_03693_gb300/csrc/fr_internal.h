@@ -141,6 +141,17 @@ inline double element_weight(int model, int nsp, int P) {
   }
 }
 
+// One of the streams that probe the preconditioner's blocks side by side: its
+// unit vectors, their product and the product's workspaces.
+struct PcLane {
+  cudaStream_t s = nullptr;
+  cudaEvent_t done = nullptr;
+  float* v = nullptr;
+  float* J = nullptr;
+  void* trace = nullptr;
+  void* fout = nullptr;
+};
+
 struct PhysParams {
   double gamma, mu, Pr, kappa;
   double q_inf[5];
@@ -225,6 +236,8 @@ struct fr_ctx {
   int32_t* d_slot_color = nullptr;       // [E] colour of each slot
   int* d_pc_status = nullptr;
   bool pc_ready = false;
+  std::vector<frgb::PcLane> pc_lanes;    // extra probing streams (small meshes)
+  cudaEvent_t pc_fork = nullptr;
   double pc_sigma = 0.0;
   int64_t step_cap = 0;                  // doubles in d_step            // (m+1) * n_dof_cap basis
   int krylov_m = 0;
@@ -293,6 +306,7 @@ namespace frgb {
 // threads a CTA of the element kernels should use on this mesh
 inline int mesh_threads(const fr_ctx* c) { return spread_threads(c->n_dof / c->nv, 256, c->sms); }
 void clear_work_cache(fr_ctx* c);
+void free_pc_lanes(fr_ctx* c);
 fr_status rebuild_work_table(fr_ctx* c, cudaStream_t s);
 // layout.cu
 fr_status layout_alloc(fr_ctx* c);
