@@ -378,24 +378,6 @@ static void launch_faces(fr_ctx* c, const T* trq, const T* trv, cudaStream_t s) 
                s, nb, nfl, kern<<<blocks, kFaceThreads, smem, s>>>(m));
 }
 
-template <typename T, int ND, bool VISC, bool DIAG = false>
-static void residual_impl(fr_ctx* c, const T* q, T* R, cudaStream_t s) {
-  T* trq = (T*)c->d_trace_q;
-  launch_traces<T, ND, VISC, DIAG>(c, q, trq, s);
-  launch_faces<T, ND, VISC, 0, DIAG>(c, trq, nullptr, s);
-  launch_vols<T, ND, VISC, 0, DIAG>(c, q, nullptr, R, s);
-}
-
-// Double-float residual: q is the FP64 state (converted on load), R written
-// in FP64 by the volume kernel.
-template <typename T, int ND, bool VISC, bool DIAG = false>
-static void residual_out64_impl(fr_ctx* c, const T* q, double* R, cudaStream_t s) {
-  T* trq = (T*)c->d_trace_q;
-  launch_traces<T, ND, VISC, DIAG>(c, q, trq, s);
-  launch_faces<T, ND, VISC, 0, DIAG>(c, trq, nullptr, s);
-  launch_vols<T, ND, VISC, 0, DIAG>(c, q, nullptr, nullptr, s, nullptr, R);
-}
-
 // ---------------------------------------------------------------------------
 // Fused JVP (every face interior and conforming): compact traces, then one
 // face-and-volume kernel per bucket
@@ -554,7 +536,7 @@ static void launch_cface_p(fr_ctx* c, const CFaceArgs<T>& a, cudaStream_t s) {
   // and a warp holds the tile's faces (3D p = 1, 3, 5); the two buffers then
   // stay within the 48 KB of static shared memory
   if constexpr (std::is_same<T, float>::value && (CT * NFP * (int)sizeof(T)) % 16 == 0 && FB <= 32 &&
-                2 * FB * 4 * CT * NFP * (int)sizeof(T) <= 48 * 1024) {
+                (2 * FB * 4 * CT * NFP + FB * cface_scratch<ND, P, VISC, DIAG, 1>()) * (int)sizeof(T) + 256 <= 48 * 1024) {
     if (c->use_tma) {
       const int ntiles = (a.n + FB - 1) / FB;
       const unsigned grid = (unsigned)std::max(1, std::min(ntiles, 4 * (int)sm_count(c)));
@@ -562,7 +544,11 @@ static void launch_cface_p(fr_ctx* c, const CFaceArgs<T>& a, cudaStream_t s) {
       return;
     }
   }
-  cface_kernel<T, ND, P, VISC, DIAG><<<nblocks(a.n, FB), FB * NFP, 0, s>>>(a);
+  const size_t smem = sizeof(T) * (size_t)cface_smem<ND, P, VISC, DIAG>();
+  auto kern = cface_kernel<T, ND, P, VISC, DIAG>;
+  static size_t configured = 48 * 1024;
+  ensure_smem(kern, smem, configured);
+  kern<<<nblocks(a.n, FB), FB * NFP, smem, s>>>(a);
 }
 
 template <typename T, int ND, int P, bool VISC, bool DIAG>
@@ -671,7 +657,7 @@ static void jvp_compact_impl(fr_ctx* c, const T* q, const T* v, T* Jv, cudaStrea
       m.P[m.ng] = g.pm + 1;
       m.block0[m.ng] = blocks;
       blocks += (int)nblocks(g.n, fb);
-      smem = std::max(smem, (size_t)fb * 4 * CT * nfp * sizeof(T));
+      smem = std::max(smem, (size_t)fb * (4 * CT + (kCommonTang<VISC, DIAG> ? 2 * NV : 0)) * nfp * sizeof(T));
       nb += face_bytes(g);
       m.ng += 1;
     }
@@ -694,6 +680,64 @@ static void jvp_compact_impl(fr_ctx* c, const T* q, const T* v, T* Jv, cudaStrea
     });
   }
   launch_vols<T, ND, VISC, 1, DIAG>(c, q, v, Jv, s, neg64);
+}
+
+// Traces and faces of the residual: on viscous meshes of axis-aligned elements
+// whose faces are all interior and conforming from compact traces (cres_kernel),
+// elsewhere the trace-gradient passes.  FP32 keeps the latter too: a residual
+// whose fluxes cancel in FP32 shows every change of rounding.
+template <typename T, int ND, bool VISC, bool DIAG>
+static void residual_faces(fr_ctx* c, const T* q, cudaStream_t s) {
+  T* trq = (T*)c->d_trace_q;
+  if constexpr (VISC && DIAG && !std::is_same<T, float>::value) {
+    if (c->fused_ok) {
+      constexpr int NV = ND + 2;
+      launch_ctraces<T, ND, VISC>(c, q, trq, s);
+      for (const auto& g : c->fgroups) {
+        CFaceArgs<T> a;
+        a.recs = g.d_recs;
+        a.trq = trq;
+        a.fout = (T*)c->d_fout;
+        a.basis = basis_ptr<T>(c);
+        a.geo = geo_view<T>(c, g.pm);
+        a.gamma = (T)c->phys.gamma;
+        a.mu = (T)c->phys.mu;
+        a.kappa = (T)c->phys.kappa;
+        a.flux = c->phys.flux;
+        a.n = g.n;
+        a.nvt = c->nvt;
+        const int P = g.pm + 1, nfp = ipow(P, ND - 1), fb = 128 / nfp;
+        const int64_t nm = (int64_t)g.n * nfp;
+        FR_LAUNCH_BF(c, kname<T>("face_res_f64", "", "face_res_df"), s, (double)nm * 8 * NV * sizeof(T),
+                     (double)nm * flops_face(ND, VISC, DIAG), {
+          switch (P) {
+            case 2: cres_kernel<T, ND, 2><<<nblocks(g.n, fb), fb * nfp, 0, s>>>(a); break;
+            case 3: cres_kernel<T, ND, 3><<<nblocks(g.n, fb), fb * nfp, 0, s>>>(a); break;
+            case 4: cres_kernel<T, ND, 4><<<nblocks(g.n, fb), fb * nfp, 0, s>>>(a); break;
+            case 5: cres_kernel<T, ND, 5><<<nblocks(g.n, fb), fb * nfp, 0, s>>>(a); break;
+            case 6: cres_kernel<T, ND, 6><<<nblocks(g.n, fb), fb * nfp, 0, s>>>(a); break;
+          }
+        });
+      }
+      return;
+    }
+  }
+  launch_traces<T, ND, VISC, DIAG>(c, q, trq, s);
+  launch_faces<T, ND, VISC, 0, DIAG>(c, trq, nullptr, s);
+}
+
+template <typename T, int ND, bool VISC, bool DIAG = false>
+static void residual_impl(fr_ctx* c, const T* q, T* R, cudaStream_t s) {
+  residual_faces<T, ND, VISC, DIAG>(c, q, s);
+  launch_vols<T, ND, VISC, 0, DIAG>(c, q, nullptr, R, s);
+}
+
+// Double-float residual: q is the FP64 state (converted on load), R written
+// in FP64 by the volume kernel.
+template <typename T, int ND, bool VISC, bool DIAG = false>
+static void residual_out64_impl(fr_ctx* c, const T* q, double* R, cudaStream_t s) {
+  residual_faces<T, ND, VISC, DIAG>(c, q, s);
+  launch_vols<T, ND, VISC, 0, DIAG>(c, q, nullptr, nullptr, s, nullptr, R);
 }
 
 // JVP; with q_traces_ready the traces of q in d_trace_q are reused (q is

@@ -12,6 +12,8 @@
 // order.  Element-face blocks have fixed strides (NVT*NFP and 3*NV*NFP values).
 #pragma once
 
+#include <type_traits>
+
 #include "fr_internal.h"
 #include "physics.cuh"
 
@@ -145,7 +147,19 @@ struct VolCfg {
 template <typename T, int P, int W>
 __device__ __forceinline__ void load_contig(const T* p, T (&x)[P]) {
   constexpr int BYTES = P * (int)sizeof(T);
-  if constexpr (W == 16 && BYTES % 16 == 0) {
+  if constexpr (std::is_same<T, double>::value && W == 16 && P % 2 == 0) {
+    // FP64 through double2: copying bytes into an array of doubles went through
+    // local memory
+#pragma unroll
+    for (int w = 0; w < P / 2; ++w) {
+      const double2 v = reinterpret_cast<const double2*>(p)[w];
+      x[2 * w] = v.x;
+      x[2 * w + 1] = v.y;
+    }
+  } else if constexpr (std::is_same<T, double>::value) {
+#pragma unroll
+    for (int k = 0; k < P; ++k) x[k] = p[k];
+  } else if constexpr (W == 16 && BYTES % 16 == 0) {
 #pragma unroll
     for (int w = 0; w < BYTES / 16; ++w) {
       const float4 v = reinterpret_cast<const float4*>(p)[w];

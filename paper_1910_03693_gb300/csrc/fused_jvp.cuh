@@ -75,15 +75,26 @@ __device__ __forceinline__ void trace_point(const T* sq, const BasisTab<T>& B, i
 #pragma unroll
       for (int k = 0; k < P; ++k) x[k] = sq[v * NSP + off[k]];
     }
-    T acc = T(0);
+    if constexpr (is_dfloat<T>::value) {
+      Acc<T> acc = acc_init(T(0)), an = acc_init(T(0));
 #pragma unroll
-    for (int k = 0; k < P; ++k) acc = xfma(B.ext[s][k], x[k], acc);
-    qf[v] = acc;
-    if (VISC) {
-      T an = T(0);
+      for (int k = 0; k < P; ++k) {
+        acc_madd(acc, B.ext[s][k], x[k]);
+        if (VISC) acc_madd(an, B.dext[s][k], x[k]);
+      }
+      qf[v] = acc_value(acc);
+      if (VISC) dn[v] = acc_value(an);
+    } else {
+      T acc = T(0);
 #pragma unroll
-      for (int k = 0; k < P; ++k) an = xfma(B.dext[s][k], x[k], an);
-      dn[v] = an;
+      for (int k = 0; k < P; ++k) acc = xfma(B.ext[s][k], x[k], acc);
+      qf[v] = acc;
+      if (VISC) {
+        T an = T(0);
+#pragma unroll
+        for (int k = 0; k < P; ++k) an = xfma(B.dext[s][k], x[k], an);
+        dn[v] = an;
+      }
     }
   }
 }
@@ -120,7 +131,7 @@ __device__ __forceinline__ void ctrace_body(const CTraceArgs<T>& a, const CTrace
   T* sq = reinterpret_cast<T*>(smem_raw) + le * NV * NSP;
   if (valid) {
 #pragma unroll
-    for (int v = 0; v < NV; ++v) sq[v * NSP + lt] = a.q[bk.state_base + (i * NV + v) * NSP + lt];
+    for (int v = 0; v < NV; ++v) sq[v * NSP + lt] = load_state(a.q, bk.state_base + (i * NV + v) * NSP + lt);
   }
   __syncthreads();
   if (!valid) return;
@@ -146,7 +157,7 @@ __device__ __forceinline__ void ctrace_body(const CTraceArgs<T>& a, const CTrace
 // instance of one degree 36 us; 32 vortices of five degrees: 10 launches a
 // product of 7 us each -> 2 of 13 us)
 template <typename T, int ND, int PF, bool VISC>
-__global__ void __launch_bounds__(256, PF == 0 ? 4 : 1) ctrace_kernel(const __grid_constant__ CTraceArgs<T> a) {
+__global__ void __launch_bounds__(256, PF == 0 ? 4 : sizeof(T) == 4 ? 8 : 3) ctrace_kernel(const __grid_constant__ CTraceArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (gate_closed(a.gate)) return;
   if constexpr (PF != 0) {
@@ -615,24 +626,145 @@ __device__ __forceinline__ void cface_geo(const CFaceArgs<T>& a, const FaceRec& 
   }
 }
 
+// Diagonal metrics (axis-aligned elements; both sides of a conforming face then
+// have the same tangential metric): the tangential part of the common gradient
+// is the tangential derivative of q^com itself, taken once from q^com of the
+// whole face in shared memory instead of from both sides' traces.  kCommonTang
+// faces need that memory (cface_scratch values a face) and a barrier among the
+// face's threads between cface_load and cface_flux (cface_sync).  The FP32
+// JVP face kernel reads 60 shared words a point for its derivatives instead of
+// 160 (32^3, p = 3: 112 -> 99 us a launch, and the arithmetic of one side saved).
+template <bool VISC, bool DIAG>
+constexpr bool kCommonTang = VISC && DIAG;
+template <int ND, int P, bool VISC, bool DIAG, int MODE>
+constexpr int cface_scratch() {
+  return kCommonTang<VISC, DIAG> ? (MODE == 1 ? 2 : 1) * (ND + 2) * (ND == 2 ? P : P * P) : 0;
+}
+// the threads of a face meet: lanes of one warp where its points divide a warp
+template <int ND, int P, bool VISC, bool DIAG>
+__device__ __forceinline__ void cface_sync() {
+  constexpr int NFP = ND == 2 ? P : P * P;
+  if constexpr (kCommonTang<VISC, DIAG>) {
+    if constexpr (32 % NFP == 0) __syncwarp();
+    else __syncthreads();
+  }
+}
+
+// q^com of this thread's point into the face's scratch [value, tangent][NV][NFP]
+template <int ND, int P, bool VISC, bool DIAG, int MODE, typename S, typename T>
+__device__ __forceinline__ void cface_common(const S* qM, const S* qS, int t, T* qcs) {
+  constexpr int NV = ND + 2, NFP = ND == 2 ? P : P * P;
+  if constexpr (kCommonTang<VISC, DIAG>) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const S qc = T(0.5) * (qM[v] + qS[v]);
+      qcs[v * NFP + t] = value(qc);
+      if (MODE == 1) qcs[(NV + v) * NFP + t] = tangent(qc);
+    }
+  }
+}
+
+// sum_m w_m y_m of P staged values (and their tangents, JVP)
+template <int P, int MODE, typename S, typename T>
+__device__ __forceinline__ S staged_sum(const T* w, const T (&y)[P], const T (&dy)[P]) {
+  S r;
+  if constexpr (is_dfloat<T>::value) {
+    Acc<T> a = acc_init(T(0));
+#pragma unroll
+    for (int m = 0; m < P; ++m) acc_madd(a, w[m], y[m]);
+    r = acc_value(a);
+  } else {
+    T a = T(0), d = T(0);
+#pragma unroll
+    for (int m = 0; m < P; ++m) {
+      a = xfma(w[m], y[m], a);
+      if (MODE == 1) d = xfma(w[m], dy[m], d);
+    }
+    set_scalar(r, a, d);
+  }
+  return r;
+}
+
+// The common gradient at point t (diagonal metrics): the tangential derivatives
+// of q^com from the face's scratch, the normal one the mean of both sides'
+// (dnM, dnS: reference normal derivatives) with their liftings.
+template <typename T, int ND, int P, int MODE, typename S>
+__device__ __forceinline__ void common_gradient(const BasisTab<T>& B, const CFaceGeo<T, ND>& g, int dm, int t, T sgm_dgf_M,
+                                                T sgs_dgf_S, const S* qM, const S* qS, const S* qc, const S* dnM,
+                                                const S* dnS, const T* qcs, S (*Gc)[ND + 2]) {
+  constexpr int NV = ND + 2, NFP = ND == 2 ? P : P * P;
+  constexpr int SZ = (int)sizeof(T);
+  constexpr int W = (NFP * SZ) % 16 == 0 && (P * SZ) % 16 == 0 ? 16 : (NFP * SZ) % 8 == 0 && (P * SZ) % 8 == 0 ? 8 : 1;
+  const int ia = t % P, ib = ND == 3 ? t / P : 0;
+  const int ta = dm == 0 ? 1 : 0;     // first tangential direction (the second is the remaining axis)
+  T wa[P], wb[P];
+#pragma unroll
+  for (int m = 0; m < P; ++m) {
+    wa[m] = B.D[ia][m];
+    wb[m] = ND == 3 ? B.D[ib][m] : T(0);
+  }
+  T h[ND], nM = T(0), nS = T(0), cM = T(0), cS = T(0);
+#pragma unroll
+  for (int j = 0; j < ND; ++j) {
+    h[j] = g.SfM[j][j] * g.JiM;
+    if (j == dm) {
+      nM = h[j];
+      nS = g.SfS[j][j] * g.JiS;
+      cM = sgm_dgf_M * nM;
+      cS = sgs_dgf_S * nS;
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    const T* y = qcs + v * NFP;
+    const T* z = qcs + (NV + v) * NFP;
+    T yl[P], zl[P] = {};
+    load_contig<T, P, W>(y + (ND == 2 ? 0 : P * ib), yl);
+    if (MODE == 1) load_contig<T, P, W>(z + (ND == 2 ? 0 : P * ib), zl);
+    const S da = staged_sum<P, MODE, S>(wa, yl, zl);
+    S db = szero<S>();
+    if (ND == 3) {
+#pragma unroll
+      for (int m = 0; m < P; ++m) {
+        yl[m] = y[ia + P * m];
+        if (MODE == 1) zl[m] = z[ia + P * m];
+      }
+      db = staged_sum<P, MODE, S>(wb, yl, zl);
+    }
+    const S dn = T(0.5) * ((nM * dnM[v] + nS * dnS[v]) + (cM * (qc[v] - qM[v]) + cS * (qc[v] - qS[v])));
+#pragma unroll
+    for (int j = 0; j < ND; ++j) Gc[j][v] = j == dm ? dn : h[j] * (j == ta ? da : db);
+  }
+}
+
+// The two sides' q at point t of a face (the slave's numbering at g.u), and
+// q^com into the face's scratch.
+template <typename T, int ND, int P, bool VISC, bool DIAG>
+__device__ __forceinline__ void cface_load(int t, int u, const T* XqM, const T* XvM, const T* XqS, const T* XvS,
+                                           Dual<T>* qM, Dual<T>* qS, T* qcs) {
+  constexpr int NV = ND + 2;
+  constexpr int NFP = ND == 2 ? P : P * P;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    qM[v] = Dual<T>{XqM[v * NFP + t], XvM[v * NFP + t]};
+    qS[v] = Dual<T>{XqS[v * NFP + u], XvS[v * NFP + u]};
+  }
+  cface_common<ND, P, VISC, DIAG, 1>(qM, qS, t, qcs);
+}
+
 // Common flux, BR2 gradient and lifting at point t of one face from its four
 // staged compact blocks (master q, master v, slave q, slave v), written as the
 // face outputs of both sides.
 template <typename T, int ND, int P, bool VISC, bool DIAG>
-__device__ __forceinline__ void cface_point(const CFaceArgs<T>& a, const FaceRec& r, int t, const CFaceGeo<T, ND>& g,
-                                            const T* XqM, const T* XvM, const T* XqS, const T* XvS) {
+__device__ __forceinline__ void cface_flux(const CFaceArgs<T>& a, const FaceRec& r, int t, const CFaceGeo<T, ND>& g,
+                                           const T* XqM, const T* XvM, const T* XqS, const T* XvS, const Dual<T>* qM,
+                                           const Dual<T>* qS, const T* qcs) {
   using S = Dual<T>;
   constexpr int NV = ND + 2;
   constexpr int NFP = ND == 2 ? P : P * P;
   const BasisTab<T>& B = a.basis[P];
   const int dm = r.mf >> 1, sm = r.mf & 1, ss = r.sf & 1;
   const int u = g.u;
-  S qM[NV], qS[NV];
-#pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    qM[v] = S{XqM[v * NFP + t], XvM[v * NFP + t]};
-    qS[v] = S{XqS[v * NFP + u], XvS[v * NFP + u]};
-  }
   const T sgm = sm ? T(1) : T(-1);
   T A[ND], n[ND];
 #pragma unroll
@@ -646,29 +778,15 @@ __device__ __forceinline__ void cface_point(const CFaceArgs<T>& a, const FaceRec
   if (VISC) {
 #pragma unroll
     for (int v = 0; v < NV; ++v) qc[v] = T(0.5) * (qM[v] + qS[v]);
-    T cM[ND], cS[ND];
-    const T gJM = B.dgf[sm] * g.JiM;
-    const T gJS = B.dgf[ss] * g.JiS;
+    S Gc[ND][NV];
+    if constexpr (DIAG) {
+      S dnM[NV], dnS[NV];
 #pragma unroll
-    for (int j = 0; j < ND; ++j) {
-      cM[j] = gJM * g.rowM[j];
-      cS[j] = gJS * g.rowS[j];
-    }
-    S GM[ND][NV], GS[ND][NV], Gc[ND][NV];
-    face_grad_m<T, ND, P, DIAG>(XqM, XvM, r.mf, t, g.SfM, g.JiM, B, GM);
-    face_grad_m<T, ND, P, DIAG>(XqS, XvS, r.sf, u, g.SfS, g.JiS, B, GS);
-    if (DIAG) {
-#pragma unroll
-      for (int j = 0; j < ND; ++j)
-#pragma unroll
-        for (int v = 0; v < NV; ++v) Gc[j][v] = T(0.5) * (GM[j][v] + GS[j][v]);
-#pragma unroll
-      for (int j = 0; j < ND; ++j) {
-        if (j != dm) continue;
-#pragma unroll
-        for (int v = 0; v < NV; ++v)
-          Gc[j][v] = Gc[j][v] + T(0.5) * (cM[j] * (qc[v] - qM[v]) + cS[j] * (qc[v] - qS[v]));
+      for (int v = 0; v < NV; ++v) {
+        dnM[v] = S{XqM[(NV + v) * NFP + t], XvM[(NV + v) * NFP + t]};
+        dnS[v] = S{XqS[(NV + v) * NFP + u], XvS[(NV + v) * NFP + u]};
       }
+      common_gradient<T, ND, P, 1>(B, g, dm, t, B.dgf[sm], B.dgf[ss], qM, qS, qc, dnM, dnS, qcs, Gc);
       S fr[NV];
       flux_viscous_row<ND>(qc, Gc, a.gamma, a.mu, a.kappa, dm, fr);
       T Ad = T(0);
@@ -678,6 +796,17 @@ __device__ __forceinline__ void cface_point(const CFaceArgs<T>& a, const FaceRec
 #pragma unroll
       for (int v = 0; v < NV; ++v) Fn[v] = Fn[v] - fr[v] * Ad;
     } else {
+      T cM[ND], cS[ND];
+      const T gJM = B.dgf[sm] * g.JiM;
+      const T gJS = B.dgf[ss] * g.JiS;
+#pragma unroll
+      for (int j = 0; j < ND; ++j) {
+        cM[j] = gJM * g.rowM[j];
+        cS[j] = gJS * g.rowS[j];
+      }
+      S GM[ND][NV], GS[ND][NV];
+      face_grad_m<T, ND, P, DIAG>(XqM, XvM, r.mf, t, g.SfM, g.JiM, B, GM);
+      face_grad_m<T, ND, P, DIAG>(XqS, XvS, r.sf, u, g.SfS, g.JiS, B, GS);
 #pragma unroll
       for (int j = 0; j < ND; ++j)
 #pragma unroll
@@ -694,21 +823,11 @@ __device__ __forceinline__ void cface_point(const CFaceArgs<T>& a, const FaceRec
       }
     }
   }
-  T* om = a.fout + r.mo;
-  T* os = a.fout + r.so;
   const T sgs = ss ? T(1) : T(-1);
+  store_face_side<ND, VISC, 1>(a.fout + r.mo, NFP, t, sgm, Fn, qc, qM);
 #pragma unroll
-  for (int v = 0; v < NV; ++v) {
-    om[v * NFP + t] = tangent(sgm * Fn[v]);
-    os[v * NFP + u] = tangent(sgs * (T(0) - Fn[v]));
-    if (VISC) {
-      const S dM = qc[v] - qM[v], dS = qc[v] - qS[v];
-      om[(NV + v) * NFP + t] = value(dM);
-      om[(2 * NV + v) * NFP + t] = tangent(dM);
-      os[(NV + v) * NFP + u] = value(dS);
-      os[(2 * NV + v) * NFP + u] = tangent(dS);
-    }
-  }
+  for (int v = 0; v < NV; ++v) Fn[v] = T(0) - Fn[v];
+  store_face_side<ND, VISC, 1>(a.fout + r.so, NFP, u, sgs, Fn, qc, qS);
 }
 
 template <typename T, int ND, int P, bool VISC, bool DIAG>
@@ -744,18 +863,88 @@ __device__ __forceinline__ void cface_body(const CFaceArgs<T>& a, int block, T* 
       for (int c = 0; c < CT; ++c) mine[w * BLK + c * NFP + t] = buf[w][c];
   }
   __syncthreads();
+  Dual<T> qM[NV], qS[NV];
+  T* qcs = sh + FB * 4 * BLK + lf * cface_scratch<ND, P, VISC, DIAG, 1>();
+  if (valid) cface_load<T, ND, P, VISC, DIAG>(t, g.u, mine, mine + BLK, mine + 2 * BLK, mine + 3 * BLK, qM, qS, qcs);
+  cface_sync<ND, P, VISC, DIAG>();
   if (!valid) return;
-  cface_point<T, ND, P, VISC, DIAG>(a, r, t, g, mine, mine + BLK, mine + 2 * BLK, mine + 3 * BLK);
+  cface_flux<T, ND, P, VISC, DIAG>(a, r, t, g, mine, mine + BLK, mine + 2 * BLK, mine + 3 * BLK, qM, qS, qcs);
+}
+
+// values of shared memory of one CTA of cface_body
+template <int ND, int P, bool VISC, bool DIAG>
+constexpr int cface_smem() {
+  constexpr int NFP = ND == 2 ? P : P * P, FB = NFP >= 128 ? 1 : 128 / NFP;
+  return FB * (4 * CompactWidth<VISC, ND + 2>::value * NFP + cface_scratch<ND, P, VISC, DIAG, 1>());
 }
 
 // FP64 (viscous, 3D) keeps 255 registers: at four CTAs an SM it spilled 1.4 KB a thread
 template <typename T, int ND, int P, bool VISC, bool DIAG>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2) cface_kernel(CFaceArgs<T> a) {
-  constexpr int NFP = ND == 2 ? P : P * P;
-  constexpr int FB = NFP >= 128 ? 1 : 128 / NFP;
-  __shared__ T sh[FB * 4 * CompactWidth<VISC, ND + 2>::value * NFP];
+  extern __shared__ __align__(16) unsigned char smem_raw[];   // cface_smem
   if (gate_closed(a.gate)) return;   // before any barrier
-  cface_body<T, ND, P, VISC, DIAG>(a, blockIdx.x, sh);
+  cface_body<T, ND, P, VISC, DIAG>(a, blockIdx.x, reinterpret_cast<T*>(smem_raw));
+}
+
+// Compact residual faces (viscous, diagonal metrics): both sides' compact traces
+// of q at the thread's point straight from memory, q^com of the face in shared
+// memory for its tangential derivatives (common_gradient).  Against the
+// trace-gradient passes the traces hold 2 NV instead of NV (1 + ND) values a face
+// point and the tangential derivatives are taken once a face instead of on
+// both its sides.  Measured at 32^3, p = 3: double-float traces 213 -> 105 us, faces
+// 232 -> 218; FP64 traces 613 -> 221, faces 831 -> 829 (the FP64 pipe and, double-
+// float, the FP32 pipe bound both).
+template <typename T, int ND, int P>
+__global__ void __launch_bounds__(128, is_dfloat<T>::value || sizeof(T) == 4 ? 4 : 3) cres_kernel(CFaceArgs<T> a) {
+  constexpr int NV = ND + 2, NFP = ND == 2 ? P : P * P, CT = 2 * NV;
+  constexpr int FB = NFP >= 128 ? 1 : 128 / NFP, SC = cface_scratch<ND, P, true, true, 0>();
+  __shared__ __align__(16) T sqc[FB * SC];
+  const int lf = threadIdx.x / NFP, t = threadIdx.x % NFP;
+  const int64_t fidx = (int64_t)blockIdx.x * FB + lf;
+  const bool valid = lf < FB && fidx < a.n;
+  T* const qcs = sqc + min(lf, FB - 1) * SC;
+  const BasisTab<T>& B = a.basis[P];
+  FaceRec r{};
+  CFaceGeo<T, ND> g{};
+  T qM[NV], qS[NV], dnM[NV], dnS[NV];
+  if (valid) {
+    r = a.recs[fidx];
+    const int u = orient_map(r.orient, t, P, ND);
+    const T* xm = a.trq + r.mt / a.nvt * CT + t;
+    const T* xs = a.trq + r.st / a.nvt * CT + u;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      qM[v] = xm[v * NFP];
+      qS[v] = xs[v * NFP];
+      dnM[v] = xm[(NV + v) * NFP];
+      dnS[v] = xs[(NV + v) * NFP];
+    }
+    cface_geo<T, ND, P, true>(a, r, t, g);
+    cface_common<ND, P, true, true, 0>(qM, qS, t, qcs);
+  }
+  cface_sync<ND, P, true, true>();
+  if (!valid) return;
+  const int dm = r.mf >> 1, sm = r.mf & 1, ss = r.sf & 1;
+  const T sgm = sm ? T(1) : T(-1), sgs = ss ? T(1) : T(-1);
+  T n[ND], Ad = T(0);
+#pragma unroll
+  for (int j = 0; j < ND; ++j) {
+    const T A = sgm * g.rowM[j];
+    n[j] = A * g.inv_absA;
+    if (j == dm) Ad = A;
+  }
+  T Fn[NV], qc[NV], Gc[ND][NV], fr[NV];
+  common_flux<ND>(a.flux, qM, qS, n, g.absA, a.gamma, Fn);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) qc[v] = T(0.5) * (qM[v] + qS[v]);
+  common_gradient<T, ND, P, 0>(B, g, dm, t, B.dgf[sm], B.dgf[ss], qM, qS, qc, dnM, dnS, qcs, Gc);
+  flux_viscous_row<ND>(qc, Gc, a.gamma, a.mu, a.kappa, dm, fr);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) Fn[v] = Fn[v] - fr[v] * Ad;
+  store_face_side<ND, true, 0>(a.fout + r.mo, NFP, t, sgm, Fn, qc, qM);
+#pragma unroll
+  for (int v = 0; v < NV; ++v) Fn[v] = T(0) - Fn[v];
+  store_face_side<ND, true, 0>(a.fout + r.so, NFP, g.u, sgs, Fn, qc, qS);
 }
 
 // The face groups of a mesh of several degrees (a batch of conforming meshes)
@@ -844,11 +1033,14 @@ __global__ void __launch_bounds__(128, 4) cface_tma_kernel(CFaceArgs<T> a, int* 
   constexpr int BLK = CT * NFP;
   constexpr uint32_t BYTES = BLK * sizeof(T);
   static_assert(BYTES % 16 == 0 && FB <= 32, "bulk-copied blocks: multiples of 16 bytes, at most one warp of faces");
+  constexpr int SC = cface_scratch<ND, P, VISC, DIAG, 1>();
   __shared__ __align__(128) T sh[2][FB][4][BLK];
+  __shared__ __align__(16) T sqc[FB * SC + 4];
   __shared__ __align__(8) uint64_t bar[2];
   if (gate_closed(a.gate)) return;   // before any barrier is armed or copy issued
   const int lf = threadIdx.x / NFP, t = threadIdx.x % NFP;
   const int ntiles = (a.n + FB - 1) / FB;
+  T* const qcs = sqc + min(lf, FB - 1) * SC;
   if (threadIdx.x == 0) {
     mbar_init(&bar[0], 1);
     mbar_init(&bar[1], 1);
@@ -892,8 +1084,12 @@ __global__ void __launch_bounds__(128, 4) cface_tma_kernel(CFaceArgs<T> a, int* 
     // whole CTA
     const bool ok = mbar_wait(&bar[b], (uint32_t)((it >> 1) & 1), kTmaWaitLimit);
     if (!ok) atomicOr(status, 1);
+    Dual<T> qM[NV], qS[NV];
     if (ok && valid)
-      cface_point<T, ND, P, VISC, DIAG>(a, r, t, g, sh[b][lf][0], sh[b][lf][1], sh[b][lf][2], sh[b][lf][3]);
+      cface_load<T, ND, P, VISC, DIAG>(t, g.u, sh[b][lf][0], sh[b][lf][1], sh[b][lf][2], sh[b][lf][3], qM, qS, qcs);
+    cface_sync<ND, P, VISC, DIAG>();
+    if (ok && valid)
+      cface_flux<T, ND, P, VISC, DIAG>(a, r, t, g, sh[b][lf][0], sh[b][lf][1], sh[b][lf][2], sh[b][lf][3], qM, qS, qcs);
     if (__syncthreads_or(!ok)) {
       stop = true;
       break;
@@ -943,7 +1139,8 @@ struct CFaceVt {
   static constexpr bool OK = 32 % NFP == 0 && FB <= 32 && QB % 16 == 0 && EB % 16 == 0;
   // [2][FB][2][BLK] q traces, [FB][2][EL] elements of v, [FB][2][BLK] tangent traces
   static constexpr size_t Q_OFF = 0, E_OFF = (size_t)2 * FB * 2 * BLK, V_OFF = E_OFF + (size_t)FB * 2 * EL;
-  static constexpr size_t SMEM = (V_OFF + (size_t)FB * 2 * BLK) * sizeof(T);
+  static constexpr size_t C_OFF = V_OFF + (size_t)FB * 2 * BLK;   // q^com scratch (diagonal metrics)
+  static constexpr size_t SMEM = (C_OFF + (size_t)FB * 2 * NV * NFP) * sizeof(T);
 };
 
 template <typename T, int ND, int P, bool VISC, bool DIAG>
@@ -1061,9 +1258,12 @@ __global__ void __launch_bounds__(128, 4) cface_vt_kernel(CFaceArgs<T> a, int* s
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       issue_v(next, b ^ 1);
     }
-    if (ok && valid) cface_point<T, ND, P, VISC, DIAG>(a, r, t, g, sb + C::Q_OFF + (size_t)(b * FB + lf) * 2 * BLK,
-                                                        xv, sb + C::Q_OFF + (size_t)(b * FB + lf) * 2 * BLK + BLK,
-                                                        xv + BLK);
+    const T* xq = sb + C::Q_OFF + (size_t)(b * FB + lf) * 2 * BLK;
+    T* qcs = sb + C::C_OFF + (size_t)lf * 2 * NV * NFP;
+    Dual<T> qM[NV], qS[NV];
+    if (ok && valid) cface_load<T, ND, P, VISC, DIAG>(t, g.u, xq, xv, xq + BLK, xv + BLK, qM, qS, qcs);
+    cface_sync<ND, P, VISC, DIAG>();
+    if (ok && valid) cface_flux<T, ND, P, VISC, DIAG>(a, r, t, g, xq, xv, xq + BLK, xv + BLK, qM, qS, qcs);
     if (__syncthreads_or(!ok)) {
       stop = true;
       break;
