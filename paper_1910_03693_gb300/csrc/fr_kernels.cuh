@@ -883,7 +883,7 @@ struct VolMulti {
 
 // as trace_multi_kernel; FP64 holds two CTAs an SM but for the 3D viscous JVP
 template <typename T, int ND, bool VISC, int MODE, bool DIAG>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : (ND == 3 && VISC && MODE == 1 ? 1 : 2))
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? (ND == 2 && !VISC ? 4 : 3) : (ND == 3 && VISC && MODE == 1 ? 1 : 2))
     vol_multi_kernel(const __grid_constant__ VolMulti<T> m) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (gate_closed(m.b[0].gate)) return;

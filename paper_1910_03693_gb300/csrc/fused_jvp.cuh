@@ -157,7 +157,7 @@ __device__ __forceinline__ void ctrace_body(const CTraceArgs<T>& a, const CTrace
 // instance of one degree 36 us; 32 vortices of five degrees: 10 launches a
 // product of 7 us each -> 2 of 13 us)
 template <typename T, int ND, int PF, bool VISC>
-__global__ void __launch_bounds__(256, PF == 0 ? 4 : sizeof(T) == 4 ? 8 : 3) ctrace_kernel(const __grid_constant__ CTraceArgs<T> a) {
+__global__ void __launch_bounds__(256, sizeof(T) == 4 && (PF != 0 || !VISC) ? 8 : PF == 0 ? 4 : 3) ctrace_kernel(const __grid_constant__ CTraceArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   if (gate_closed(a.gate)) return;
   if constexpr (PF != 0) {
@@ -957,7 +957,7 @@ struct CFaceMulti {
 };
 
 template <typename T, int ND, bool VISC, bool DIAG>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2) cface_multi_kernel(const __grid_constant__ CFaceMulti<T> m) {
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (VISC ? 4 : 8) : 2) cface_multi_kernel(const __grid_constant__ CFaceMulti<T> m) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sh = reinterpret_cast<T*>(smem_raw);
   if (gate_closed(m.g[0].gate)) return;

@@ -103,17 +103,25 @@ __device__ __forceinline__ Dual<T> dsqrt(Dual<T> x) {
   T r = dsqrt(x.v);
   return {r, x.d / (T(2) * r)};
 }
+// 1 / x; the tangent -x.d / x^2 from the reciprocal, not by a second division
+// (a division is the longest operation here, of the FP64 pipe above all)
+template <typename S>
+__device__ __forceinline__ S recip(S x) { return S(1) / x; }
+template <typename T>
+__device__ __forceinline__ Dual<T> recip(Dual<T> x) {
+  const T r = T(1) / x.v;
+  return {r, -(r * r) * x.d};
+}
+// sqrt(x) given its value c
+template <typename T>
+__device__ __forceinline__ T sqrt_given(T, T c) { return c; }
+template <typename T>
+__device__ __forceinline__ Dual<T> sqrt_given(Dual<T> x, T c) { return {c, x.d / (T(2) * c)}; }
 // |x| with d|x| = sign(x) dx, sign(0) := +1
 __device__ __forceinline__ double dabs(double x) { return fabs(x); }
 __device__ __forceinline__ float dabs(float x) { return fabsf(x); }
 template <typename T>
 __device__ __forceinline__ Dual<T> dabs(Dual<T> x) { return x.v < T(0) ? Dual<T>{-x.v, -x.d} : x; }
-// max(a, b); at a tie the first argument (the "-" side) is taken
-template <typename T>
-__device__ __forceinline__ T dmax(T a, T b) { return b > a ? b : a; }
-template <typename T>
-__device__ __forceinline__ Dual<T> dmax(Dual<T> a, Dual<T> b) { return b.v > a.v ? b : a; }
-
 template <typename S>
 __device__ __forceinline__ S szero() { return S{}; }
 
@@ -126,7 +134,7 @@ __device__ __forceinline__ void set_scalar(Dual<T>& x, T v, T d) { x.v = v; x.d 
 template <int ND, typename S, typename T>
 __device__ __forceinline__ void flux_inviscid(const S* q, T gamma, S (*f)[ND + 2]) {
   constexpr int NV = ND + 2;
-  const S rinv = T(1) / q[0];
+  const S rinv = recip(q[0]);
   S vel[ND];
   S mu2 = szero<S>();
 #pragma unroll
@@ -147,32 +155,32 @@ __device__ __forceinline__ void flux_inviscid(const S* q, T gamma, S (*f)[ND + 2
   }
 }
 
-// Normal flux f(q).n and the wave speed |u.n| + c of one state (one reciprocal,
-// one square root).
+// Normal flux f(q).n of one state, with its normal velocity and the square of its
+// sound speed.
 template <int ND, typename S, typename T>
-__device__ __forceinline__ S normal_flux(const S* q, const T* n, T gamma, S* fn) {
+__device__ __forceinline__ void normal_flux(const S* q, const T* n, T gamma, S* fn, S& un, S& c2) {
   constexpr int NV = ND + 2;
-  const S rinv = T(1) / q[0];
+  const S rinv = recip(q[0]);
   S mn = szero<S>(), mu2 = szero<S>();
 #pragma unroll
   for (int i = 0; i < ND; ++i) {
     mn = mn + q[1 + i] * n[i];
     mu2 = mu2 + q[1 + i] * q[1 + i];
   }
-  const S un = mn * rinv;
+  un = mn * rinv;
   const S pres = (gamma - T(1)) * (q[NV - 1] - T(0.5) * mu2 * rinv);
   fn[0] = mn;
 #pragma unroll
   for (int i = 0; i < ND; ++i) fn[1 + i] = q[1 + i] * un + pres * n[i];
   fn[NV - 1] = (q[NV - 1] + pres) * un;
-  return dabs(un) + dsqrt(gamma * pres * rinv);
+  c2 = gamma * pres * rinv;
 }
 
 // Normal flux f(q).n alone (no wave speed).
 template <int ND, typename S, typename T>
 __device__ __forceinline__ void normal_flux_only(const S* q, const T* n, T gamma, S* fn) {
   constexpr int NV = ND + 2;
-  const S rinv = T(1) / q[0];
+  const S rinv = recip(q[0]);
   S mn = szero<S>(), mu2 = szero<S>();
 #pragma unroll
   for (int i = 0; i < ND; ++i) {
@@ -198,7 +206,7 @@ __device__ __forceinline__ void roe(const S* qL, const S* qR, const T* n, T absA
   S fL[NV], fR[NV];
   normal_flux_only<ND>(qL, n, gamma, fL);
   normal_flux_only<ND>(qR, n, gamma, fR);
-  const S riL = T(1) / qL[0], riR = T(1) / qR[0];
+  const S riL = recip(qL[0]), riR = recip(qR[0]);
   S uL[ND], uR[ND], kL = szero<S>(), kR = szero<S>();
 #pragma unroll
   for (int i = 0; i < ND; ++i) {
@@ -211,7 +219,7 @@ __device__ __forceinline__ void roe(const S* qL, const S* qR, const T* n, T absA
   const S pR = (gamma - T(1)) * (qR[NV - 1] - T(0.5) * kR);
   const S HL = (qL[NV - 1] + pL) * riL, HR = (qR[NV - 1] + pR) * riR;
   const S sL = dsqrt(qL[0]), sR = dsqrt(qR[0]);
-  const S wi = T(1) / (sL + sR);
+  const S wi = recip(sL + sR);
   S u[ND], q2 = szero<S>(), un = szero<S>(), dun = szero<S>(), udu = szero<S>();
   S du[ND];
 #pragma unroll
@@ -228,7 +236,7 @@ __device__ __forceinline__ void roe(const S* qL, const S* qR, const T* n, T absA
   const S c = dsqrt(c2);
   const S rho = sL * sR;
   const S dp = pR - pL, drho = qR[0] - qL[0];
-  const S ic2 = T(1) / c2;
+  const S ic2 = recip(c2);
   const S a1 = T(0.5) * (dp - rho * c * dun) * ic2;
   const S a3 = T(0.5) * (dp + rho * c * dun) * ic2;
   const S a2 = drho - dp * ic2;
@@ -244,15 +252,18 @@ __device__ __forceinline__ void roe(const S* qL, const S* qR, const T* n, T absA
 }
 
 // Rusanov normal flux times the face area: ((fL.n + fR.n)/2 - lam/2 (qR - qL)) |A|,
-// lam = max(|u.n| + c) over the two sides (the "-" side at a tie).
+// lam = max(|u.n| + c) over the two sides (the "-" side at a tie); the tangent of
+// the wave speed is formed on that side only.
 template <int ND, typename S, typename T>
 __device__ __forceinline__ void rusanov(const S* qL, const S* qR, const T* n, T absA, T gamma,
                                         S* Fn) {
   constexpr int NV = ND + 2;
-  S fL[NV], fR[NV];
-  const S lamL = normal_flux<ND>(qL, n, gamma, fL);
-  const S lamR = normal_flux<ND>(qR, n, gamma, fR);
-  const S lam = dmax(lamL, lamR);
+  S fL[NV], fR[NV], uL, uR, c2L, c2R;
+  normal_flux<ND>(qL, n, gamma, fL, uL, c2L);
+  normal_flux<ND>(qR, n, gamma, fR, uR, c2R);
+  const T cL = dsqrt(value(c2L)), cR = dsqrt(value(c2R));
+  const bool right = dabs(value(uR)) + cR > dabs(value(uL)) + cL;
+  const S lam = dabs(right ? uR : uL) + sqrt_given(right ? c2R : c2L, right ? cR : cL);
 #pragma unroll
   for (int v = 0; v < NV; ++v) Fn[v] = (T(0.5) * (fL[v] + fR[v]) - T(0.5) * lam * (qR[v] - qL[v])) * absA;
 }
@@ -271,7 +282,7 @@ template <int ND, typename S, typename T>
 __device__ __forceinline__ void flux_viscous(const S* q, const S (*G)[ND + 2], T gamma, T mu,
                                              T kappa, S (*fv)[ND + 2]) {
   constexpr int NV = ND + 2;
-  const S rinv = T(1) / q[0];
+  const S rinv = recip(q[0]);
   S vel[ND];
 #pragma unroll
   for (int i = 0; i < ND; ++i) vel[i] = q[1 + i] * rinv;
@@ -314,7 +325,7 @@ template <int ND, typename S, typename T>
 __device__ __forceinline__ void flux_viscous_row(const S* q, const S (*G)[ND + 2], T gamma, T mu, T kappa,
                                                  int d, S* fr) {
   constexpr int NV = ND + 2;
-  const S rinv = T(1) / q[0];
+  const S rinv = recip(q[0]);
   S vel[ND];
 #pragma unroll
   for (int i = 0; i < ND; ++i) vel[i] = q[1 + i] * rinv;

@@ -188,7 +188,7 @@ __device__ __forceinline__ void rusanov_adjoint(const T* qL, const T* qR, const 
                                                 T* qLb, T* qRb) {
   constexpr int NV = ND + 2;
   const T lamL = wave_speed<ND>(qL, n, gamma), lamR = wave_speed<ND>(qR, n, gamma);
-  const bool right = lamR > lamL;     // the "-" side at a tie, as dmax
+  const bool right = lamR > lamL;     // the "-" side at a tie, as rusanov
   const T hl = T(0.5) * (right ? lamR : lamL);
   T half[NV], lamb = T(0);
 #pragma unroll
