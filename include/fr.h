@@ -387,10 +387,10 @@ fr_status esdirk_step(fr_ctx* ctx, const fr_tableau* tab, double dt, double* q_i
  * and write the table, 2 x 3 x 7 int32 [precision f64 (also used by the
  * double-float kernels, same operand size), f32][kernel trace,
  * volume residual, volume JVP][P = p+1]: for P >= 2 the elements per CTA
- * of the one-launch-per-bucket kernels, 0 = default (as many whole elements
- * as fit 256 threads, or on small meshes as few whole warps as give every SM
- * four CTAs; a value whose elements exceed 256 threads also falls back to it;
- * the multi-bucket launch always uses the default);
+ * of the one-launch-per-bucket kernels, 0 = default (a rule on the precision
+ * and the element's points, at most 256 threads, on small meshes as few whole
+ * warps as give every SM four CTAs; a value whose elements exceed 256 threads
+ * also falls back to it; the multi-bucket launch has tiles of its own);
  * the slot P = 0 holds the multi-bucket choice of that precision and kernel
  * (0 undecided: one launch over all buckets, but for the double-float
  * kernels on meshes of more than 512 points per SM; 1 one launch over all

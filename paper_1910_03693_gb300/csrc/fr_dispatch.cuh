@@ -3,6 +3,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <type_traits>
 #include <vector>
@@ -88,13 +89,46 @@ static inline int nsp_of(int nd, int P) { return nd == 2 ? P * P : P * P * P; }
 
 static inline unsigned sm_count(const fr_ctx* c) { return (unsigned)c->sms; }
 
-// elements per CTA: tuned value, else as many whole elements as fit the
-// threads a CTA of this mesh should use
-static inline int epb_for(fr_ctx* c, int prec, int kind, int P) {
-  const int t = c->epb_tab[prec][kind][P];
+// Elements per CTA of a kernel with one thread per solution point, by what bounds
+// it (n_sp points an element, at most `threads` a CTA):
+//  - FP64: the lanes in use of the warps a CTA takes (the FP64 pipe spends a warp
+//    instruction on idle lanes too), fewer warps among equals.  3D p = 2: 7
+//    elements (189 of 192 lanes) 681 us, 9 (243 of 256) 719, 1 (27 of 32) 793;
+//  - FP32 (loads and shared memory between barriers): few warps a barrier, then
+//    lanes in use.  JVP volume kernel, 3D p = 3: 1 element 73.4 us, 2 75.7, 4 83.7; p =
+//    2: 1 77.1, 7 84.6, 9 89.7; p = 4: 1 84.0, 2 92.6; 2D p = 4: 1 32.9, 5 31.0, 10 33.5;
+//    volume adjoint, 3D p = 3: 156 -> 136;
+//  - double-float: as many as fit (its large code wants full CTAs; 3D p = 3: 4 253
+//    us, 1 279).
+enum class EpbRule { kFull, kLanes, kFewWarps };
+static inline int epb_by_rule(EpbRule rule, int nsp, int threads) {
+  const int most = std::max(1, threads / nsp);
+  if (rule == EpbRule::kFull) return most;
+  int best = most;
+  double best_score = 1e300;
+  for (int e = 1; e <= most; ++e) {
+    const int warps = (e * nsp + 31) / 32;
+    const double idle = 32.0 * warps / (e * nsp);    // lanes paid for per lane in use
+    const double score = rule == EpbRule::kLanes ? idle * (1.0 + 0.002 * warps) : std::pow(idle, 0.4) * (1.0 + 0.023 * warps);
+    if (score < best_score - 1e-12) {
+      best_score = score;
+      best = e;
+    }
+  }
+  return best;
+}
+template <typename T>
+constexpr EpbRule epb_rule() {
+  return is_dfloat<T>::value ? EpbRule::kFull : std::is_same<T, double>::value ? EpbRule::kLanes : EpbRule::kFewWarps;
+}
+
+// elements per CTA of a launch over one bucket: tuned value, else by the rule
+template <typename T>
+static inline int epb_for(fr_ctx* c, int kind, int P) {
+  const int t = c->epb_tab[prec_row<T>()][kind][P];
   const int nsp = nsp_of(c->nd, P);
   if (t > 0 && t * nsp <= 256) return t;
-  return std::max(1, mesh_threads(c) / nsp);
+  return epb_by_rule(epb_rule<T>(), nsp, mesh_threads(c));
 }
 
 // One launch over all buckets for this precision and kernel kind: the master
@@ -180,7 +214,7 @@ static void launch_traces(fr_ctx* c, const T* q, T* trace, cudaStream_t s) {
     int block = 32;
     for (size_t i = 0; i < c->buckets.size(); ++i) {
       const Bucket& b = c->buckets[i];
-      const int P = b.p + 1, e = epb_multi(ND, P, mesh_threads(c));
+      const int P = b.p + 1, e = epb_multi(ND, P, tile_threads(c));
       block = std::max(block, (e * nsp_of(ND, P) + 31) / 32 * 32);
       m.b[i] = trace_args<T, ND, VISC>(c, b, q, trace);
       m.P[i] = P;
@@ -196,7 +230,7 @@ static void launch_traces(fr_ctx* c, const T* q, T* trace, cudaStream_t s) {
   }
   for (const auto& b : c->buckets) {
     const TraceArgs<T> a = trace_args<T, ND, VISC>(c, b, q, trace);
-    const int P = b.p + 1, e = epb_for(c, prec, 0, P);
+    const int P = b.p + 1, e = epb_for<T>(c, 0, P);
     const double nbb = (double)b.count * values_trace(ND, P, VISC) * sizeof(T);
     const double nfb = (double)b.count * 2 * ND * ipow(P, ND - 1) * flops_trace(ND, P, VISC, DIAG);
     FR_LAUNCH_BF(c, name, s, nbb, nfb, {
@@ -269,7 +303,7 @@ static void launch_vols(fr_ctx* c, const T* q, const T* v, T* out, cudaStream_t 
     int block = 32;
     for (size_t i = 0; i < c->buckets.size(); ++i) {
       const Bucket& b = c->buckets[i];
-      const int P = b.p + 1, e = epb_multi(ND, P, mesh_threads(c));
+      const int P = b.p + 1, e = epb_multi(ND, P, tile_threads(c));
       block = std::max(block, (e * nsp_of(ND, P) + 31) / 32 * 32);
       m.b[i] = vol_args<T>(c, b, q, v, out, out_neg64, out64);
       m.P[i] = P;
@@ -285,7 +319,7 @@ static void launch_vols(fr_ctx* c, const T* q, const T* v, T* out, cudaStream_t 
   }
   for (const auto& b : c->buckets) {
     const VolArgs<T> a = vol_args<T>(c, b, q, v, out, out_neg64, out64);
-    const int P = b.p + 1, e = epb_for(c, prec, kind, P);
+    const int P = b.p + 1, e = epb_for<T>(c, kind, P);
     const double nbb = (double)b.count * values_volume(ND, P, VISC, MODE == 1, out_ratio) * sizeof(T);
     const double nfb = MODE == 1 ? 0.0 : (double)b.count * nsp_of(ND, P) * flops_volume(ND, P, VISC, DIAG);
     FR_LAUNCH_BF(c, name, s, nbb, nfb, {
@@ -442,7 +476,7 @@ static void launch_ctraces(fr_ctx* c, const T* q, T* out, cudaStream_t s) {
   double nb = 0.0;
   for (int i = 0; i < a.nb; ++i) {
     const Bucket& b = c->buckets[i];
-    const int P = b.p + 1, nsp = nsp_of(ND, P), e = epb_multi(ND, P, mesh_threads(c));
+    const int P = b.p + 1, nsp = nsp_of(ND, P), e = epb_multi(ND, P, tile_threads(c));
     a.b[i] = CTraceBucket{b.state_base, b.ctrace_base, b.count, P, e, blocks};
     blocks += (int)nblocks(b.count, e);
     threads = std::max(threads, (e * nsp + 31) / 32 * 32);
@@ -818,7 +852,7 @@ static void vjp_impl(fr_ctx* c, const T* q, const T* w, T* out, cudaStream_t s) 
     a.out_base = b.out_base;
     a.count = b.count;
     a.slot_begin = b.slot_begin;
-    const int P = b.p + 1, e = epb_multi(ND, P, mesh_threads(c));
+    const int P = b.p + 1, e = epb_by_rule(epb_rule<T>(), nsp_of(ND, P), mesh_threads(c));
     FR_LAUNCH_B(c, sizeof(T) == 8 ? "vol_adj_f64" : "vol_adj_f32", s,
                 (double)b.count * NV * nsp_of(ND, P) * sizeof(T) * 2, {
       switch (P) {

@@ -308,7 +308,7 @@ fr_status rebuild_work_table(fr_ctx* c, cudaStream_t s) {
   std::vector<std::pair<double, WorkRun>> runs;
   for (size_t bi = 0; bi < c->buckets.size(); ++bi) {
     const Bucket& b = c->buckets[bi];
-    const int P = b.p + 1, e = epb_multi(c->nd, P, mesh_threads(c));
+    const int P = b.p + 1, e = epb_multi(c->nd, P, tile_threads(c));
     const double w = element_weight(c->epb_tab[0][0][1], pw(P, c->nd), P);
     const int full = b.count / e, rest = b.count % e;
     if (full) runs.push_back({e * w, WorkRun{(int)bi, 0, e, 0, full}});
