@@ -716,6 +716,26 @@ static void jvp_compact_impl(fr_ctx* c, const T* q, const T* v, T* Jv, cudaStrea
   launch_vols<T, ND, VISC, 1, DIAG>(c, q, v, Jv, s, neg64);
 }
 
+// arguments of the compact face kernels for one group, traces of q at trq
+template <typename T>
+static CFaceArgs<T> compact_face_args(fr_ctx* c, const FaceGroup& g, const T* trq) {
+  CFaceArgs<T> a;
+  a.gate = c->gate;
+  a.recs = g.d_recs;
+  a.trq = trq;
+  a.trv = nullptr;
+  a.fout = (T*)c->d_fout;
+  a.basis = basis_ptr<T>(c);
+  a.geo = geo_view<T>(c, g.pm);
+  a.gamma = (T)c->phys.gamma;
+  a.mu = (T)c->phys.mu;
+  a.kappa = (T)c->phys.kappa;
+  a.flux = c->phys.flux;
+  a.n = g.n;
+  a.nvt = c->nvt;
+  return a;
+}
+
 // Traces and faces of the residual: on viscous meshes of axis-aligned elements
 // whose faces are all interior and conforming from compact traces (cres_kernel),
 // elsewhere the trace-gradient passes.  FP32 keeps the latter too: a residual
@@ -728,18 +748,7 @@ static void residual_faces(fr_ctx* c, const T* q, cudaStream_t s) {
       constexpr int NV = ND + 2;
       launch_ctraces<T, ND, VISC>(c, q, trq, s);
       for (const auto& g : c->fgroups) {
-        CFaceArgs<T> a;
-        a.recs = g.d_recs;
-        a.trq = trq;
-        a.fout = (T*)c->d_fout;
-        a.basis = basis_ptr<T>(c);
-        a.geo = geo_view<T>(c, g.pm);
-        a.gamma = (T)c->phys.gamma;
-        a.mu = (T)c->phys.mu;
-        a.kappa = (T)c->phys.kappa;
-        a.flux = c->phys.flux;
-        a.n = g.n;
-        a.nvt = c->nvt;
+        const CFaceArgs<T> a = compact_face_args<T>(c, g, trq);
         const int P = g.pm + 1, nfp = ipow(P, ND - 1), fb = 128 / nfp;
         const int64_t nm = (int64_t)g.n * nfp;
         FR_LAUNCH_BF(c, kname<T>("face_res_f64", "", "face_res_df"), s, (double)nm * 8 * NV * sizeof(T),
@@ -828,7 +837,14 @@ static void vjp_impl(fr_ctx* c, const T* q, const T* w, T* out, cudaStream_t s) 
     if (nm != ns) jsmem = std::max(jsmem, (size_t)g.fb * NV * nm * sizeof(T));
     fsmem = std::max(fsmem, (size_t)g.fb * AdjFace<ND, VISC>::stride(nm, ns) * sizeof(T));
   }
-  launch_traces<T, ND, VISC, DIAG>(c, q, trq, s);
+  // compact traces where the compact face adjoint runs
+  const bool compact = VISC && DIAG && c->fused_ok;
+  if (compact) {
+    m.ct = 2 * NV;
+    launch_ctraces<T, ND, VISC>(c, q, trq, s);
+  } else {
+    launch_traces<T, ND, VISC, DIAG>(c, q, trq, s);
+  }
   if (VISC && blocks > 0) {
     auto kern = jump_kernel<T, ND>;
     static size_t configured = 48 * 1024;
@@ -864,7 +880,23 @@ static void vjp_impl(fr_ctx* c, const T* q, const T* w, T* out, cudaStream_t s) 
       }
     });
   }
-  if (blocks > 0) {
+  if (compact) {
+    if constexpr (VISC && DIAG) {
+      for (const auto& g : c->fgroups) {
+        const CFaceArgs<T> a = compact_face_args<T>(c, g, trq);
+        const int P = g.pm + 1, nfp = ipow(P, ND - 1), fb = 128 / nfp;
+        FR_LAUNCH(c, "face_adj", s, {
+          switch (P) {
+            case 2: cface_adj_kernel<T, ND, 2><<<nblocks(g.n, fb), fb * nfp, 0, s>>>(a, am.fbar, am.trbar); break;
+            case 3: cface_adj_kernel<T, ND, 3><<<nblocks(g.n, fb), fb * nfp, 0, s>>>(a, am.fbar, am.trbar); break;
+            case 4: cface_adj_kernel<T, ND, 4><<<nblocks(g.n, fb), fb * nfp, 0, s>>>(a, am.fbar, am.trbar); break;
+            case 5: cface_adj_kernel<T, ND, 5><<<nblocks(g.n, fb), fb * nfp, 0, s>>>(a, am.fbar, am.trbar); break;
+            case 6: cface_adj_kernel<T, ND, 6><<<nblocks(g.n, fb), fb * nfp, 0, s>>>(a, am.fbar, am.trbar); break;
+          }
+        });
+      }
+    }
+  } else if (blocks > 0) {
     auto kern = face_adj_kernel<T, ND, VISC, DIAG>;
     static size_t configured = 48 * 1024;
     ensure_smem(kern, fsmem, configured);

@@ -373,6 +373,7 @@ struct FaceMulti {
   T gamma, mu, kappa;
   T qinf[5];
   int ng, nvt;
+  int ct = 0;                       // components of compact traces at trq (jump_kernel), 0: trace-gradient layout
   int flux;                         // common inviscid flux: 0 Rusanov, 1 Roe
   const int* gate = nullptr;        // see gate_closed
 };

@@ -24,7 +24,7 @@
 // the trace; FP32: the shared-memory lines and the face data's bytes.
 #pragma once
 
-#include "fr_kernels.cuh"
+#include "fused_jvp.cuh"
 
 namespace frgb {
 
@@ -352,12 +352,12 @@ __global__ void __launch_bounds__(kFaceThreads) jump_kernel(const __grid_constan
   FaceRec r{};
   if (valid) {
     r = g.recs[f0 + lf];
-    load_trace_pt<ND>(m.trq, (const T*)nullptr, r.mt, 0, NV, NFPm, t, qM);
+    load_trace_pt<ND>(m.trq, (const T*)nullptr, m.ct ? r.mt / m.nvt * m.ct : r.mt, 0, NV, NFPm, t, qM);
   }
   if (Pm == Ps) {
     if (!valid) return;
     const int u = orient_map(r.orient, t, Pm, ND);
-    load_trace_pt<ND>(m.trq, (const T*)nullptr, r.st, 0, NV, NFPs, u, qG);
+    load_trace_pt<ND>(m.trq, (const T*)nullptr, m.ct ? r.st / m.nvt * m.ct : r.st, 0, NV, NFPs, u, qG);
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const T qc = T(0.5) * (qM[v] + qG[v]);
@@ -938,6 +938,124 @@ __global__ void __launch_bounds__(kFaceThreads, sizeof(T) == 4 ? 4 : 1)
   }
   if (VISC) __syncthreads();
   if (vp) store_adj_side<ND, VISC>(am.trbar + rp.st, Ps, NFPs, pt, qSb, nS, tang, m.basis[Ps]);
+}
+
+// Compact face adjoint (viscous, diagonal metrics, conforming faces; the
+// transpose of the compact face passes): both sides' compact traces and
+// face-output adjoints in, the tangential part of the common gradient taken
+// from q^com (common_gradient) and transposed once a face.  24^3, p = 4, FP32:
+// traces 81 -> 27 us, jumps 26 -> 24, face adjoint 121 -> 87 (VJP 384 -> 296); 12^3, FP64,
+// traces 81 -> 32, face adjoint 183 -> 162.
+template <typename T, int ND, int P>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2)
+    cface_adj_kernel(CFaceArgs<T> a, const T* __restrict__ fbar, T* __restrict__ trbar) {
+  constexpr int NV = ND + 2, NFP = ND == 2 ? P : P * P, CT = 2 * NV;
+  constexpr int FB = NFP >= 128 ? 1 : 128 / NFP, SC = NV * NFP, ST = (ND - 1) * NV * NFP;
+  __shared__ __align__(16) T sqc[FB * SC];
+  __shared__ __align__(16) T stang[FB * ST];
+  const int lf = threadIdx.x / NFP, t = threadIdx.x % NFP;
+  const int64_t fidx = (int64_t)blockIdx.x * FB + lf;
+  const bool valid = lf < FB && fidx < a.n;
+  T* const qcs = sqc + min(lf, FB - 1) * SC;
+  T* const tang = stang + min(lf, FB - 1) * ST;
+  const BasisTab<T>& B = a.basis[P];
+  FaceRec r{};
+  CFaceGeo<T, ND> g{};
+  T qM[NV], qS[NV], qMb[NV], qSb[NV], qcb[NV], nM[NV], nS[NV];
+  const T *xm = nullptr, *xs = nullptr;
+  if (valid) {
+    r = a.recs[fidx];
+    cface_geo<T, ND, P, true>(a, r, t, g);
+    xm = a.trq + r.mt / a.nvt * CT + t;
+    xs = a.trq + r.st / a.nvt * CT + g.u;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      qM[v] = xm[v * NFP];
+      qS[v] = xs[v * NFP];
+    }
+    cface_common<ND, P, true, true, 0>(qM, qS, t, qcs);
+  }
+  cface_sync<ND, P, true, true>();
+  if (valid) {
+    const int dm = r.mf >> 1, sm = r.mf & 1, ss = r.sf & 1;
+    const T sgm = sm ? T(1) : T(-1), sgs = ss ? T(1) : T(-1);
+    T n[ND], Ad = T(0), h[ND], hM = T(0), hS = T(0);
+#pragma unroll
+    for (int j = 0; j < ND; ++j) {
+      const T A = sgm * g.rowM[j];
+      n[j] = A * g.inv_absA;
+      h[j] = g.SfM[j][j] * g.JiM;
+      if (j == dm) {
+        Ad = A;
+        hM = h[j];
+        hS = g.SfS[j][j] * g.JiS;
+      }
+    }
+    const T* fm = fbar + r.mo + t;
+    const T* fs = fbar + r.so + g.u;
+    T Fnb[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const T x = fm[(NV + v) * NFP], y = fs[(NV + v) * NFP];
+      Fnb[v] = sgm * fm[v * NFP] - sgs * fs[v * NFP];
+      qcb[v] = x + y;
+      qMb[v] = -x;
+      qSb[v] = -y;
+    }
+    flux_adjoint<ND>(a.flux, qM, qS, n, g.absA, a.gamma, Fnb, qMb, qSb);
+    T qc[NV], dnM[NV], dnS[NV], Gc[ND][NV], fvb[ND][NV], Gcb[ND][NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      qc[v] = T(0.5) * (qM[v] + qS[v]);
+      dnM[v] = xm[(NV + v) * NFP];
+      dnS[v] = xs[(NV + v) * NFP];
+    }
+    common_gradient<T, ND, P, 0>(B, g, dm, t, B.dgf[sm], B.dgf[ss], qM, qS, qc, dnM, dnS, qcs, Gc);
+#pragma unroll
+    for (int j = 0; j < ND; ++j)
+#pragma unroll
+      for (int v = 0; v < NV; ++v) fvb[j][v] = j == dm ? -Fnb[v] * Ad : T(0);
+    viscous_adjoint<ND>(qc, Gc, fvb, a.gamma, a.mu, a.kappa, qcb, Gcb);
+    const T cM = B.dgf[sm] * hM, cS = B.dgf[ss] * hS;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      T gn = T(0);
+#pragma unroll
+      for (int j = 0; j < ND; ++j) {
+        if (j == dm) gn = T(0.5) * Gcb[j][v];
+        else tang[((j > dm ? j - 1 : j) * NV + v) * NFP + t] = h[j] * Gcb[j][v];
+      }
+      nM[v] = hM * gn;
+      nS[v] = hS * gn;
+      qcb[v] += (cM + cS) * gn;
+      qMb[v] -= cM * gn;
+      qSb[v] -= cS * gn;
+    }
+  }
+  cface_sync<ND, P, true, true>();
+  if (!valid) return;
+  const int ia = t % P, ib = ND == 3 ? t / P : 0;
+  T* om = trbar + r.mt + t;
+  T* os = trbar + r.st + g.u;
+  T wa[P], wb[P];
+#pragma unroll
+  for (int c = 0; c < P; ++c) {
+    wa[c] = B.D[c][ia];
+    wb[c] = ND == 3 ? B.D[c][ib] : T(0);
+  }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    T x = qcb[v];
+#pragma unroll
+    for (int c = 0; c < P; ++c) {
+      x += wa[c] * tang[v * NFP + c + P * ib];
+      if (ND == 3) x += wb[c] * tang[(NV + v) * NFP + ia + P * c];
+    }
+    om[v * NFP] = qMb[v] + T(0.5) * x;
+    om[(NV + v) * NFP] = nM[v];
+    os[v * NFP] = qSb[v] + T(0.5) * x;
+    os[(NV + v) * NFP] = nS[v];
+  }
 }
 
 // ---------------------------------------------------------------------------

@@ -1,5 +1,5 @@
-"""Viscous boxes of axis-aligned elements: the residual from compact traces and
-the common gradient whose tangential part is taken from q^com, against the
+"""Viscous boxes of axis-aligned elements: the residual, product and transposed
+product from compact traces and the common gradient whose tangential part is taken from q^com, against the
 oracle, for every degree, both fluxes, stretched boxes, and elements turned by
 180 degrees (negative diagonal metrics, flipped orientation codes)."""
 import numpy as np
@@ -52,11 +52,12 @@ def test_against_oracle(p, n, kind, flux):
     qt = torch.from_numpy(q)
     v = torch.from_numpy((cases.uniform(610 + p, q.size) - 0.5) * np.abs(q).mean())
     qs, vs = ctx.pack(qt.cuda()), ctx.pack(v.cuda())
-    R, J = fr.residual(qt).numpy(), L.jvp(fr, qt, v).numpy()
+    R, J, A = fr.residual(qt).numpy(), L.jvp(fr, qt, v).numpy(), L.vjp(fr, qt, v).numpy()
     get = lambda t: ctx.unpack(t).cpu().numpy()
     # the suite's bounds: FP64 1e-12, double-float 2e-10, FP32 2e-5
     for gpu, ref, tol in ((ctx.residual(qs), R, 1e-12), (ctx.residual(qs, double_float=True), R, 2e-10),
                           (ctx.jvp(qs, vs), J, 1e-12), (ctx.residual(qs.float()), R, 2e-5),
-                          (ctx.jvp(qs.float(), vs.float()), J, 2e-5)):
+                          (ctx.jvp(qs.float(), vs.float()), J, 2e-5), (ctx.vjp(qs, vs), A, 1e-12),
+                          (ctx.vjp(qs.float(), vs.float()), A, 2e-5)):
         ok = Hp.parity_ok(get(gpu), ref, m, q, tol)
         assert ok[0], ok
