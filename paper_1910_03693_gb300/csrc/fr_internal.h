@@ -285,6 +285,7 @@ struct fr_ctx {
   // vector and control words on the device with their pinned host mirror, and
   // the iteration count of the last cycle (the size of the next first batch)
   const int* gate = nullptr;
+  bool chain = true;   // launches may be scheduled while their predecessor drains (launch_chained)
   const double* vscale = nullptr;   // scale of the stored column a device-driven product reads (VolArgs)
   bool device_gmres = true;
   double* d_gm = nullptr;

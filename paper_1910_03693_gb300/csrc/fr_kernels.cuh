@@ -100,6 +100,16 @@ __device__ __forceinline__ T load_state(const T* q, int64_t i) {
 // nothing waits on it.
 __device__ __forceinline__ bool gate_closed(const int* gate) { return gate != nullptr && *gate != 0; }
 
+// Entry of the kernels launched by launch_chained: the next kernel of the
+// stream may take its place on the SMs as soon as every CTA of this one has
+// started, and nothing is read or written before all work of the previous one
+// has completed (its CTAs do the same, so no kernel runs ahead by two).  The
+// pointers these kernels read through are not declared __restrict__, so no load
+// can go through the read-only path and move above the wait.
+__device__ __forceinline__ void chain_entry() {
+  asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory");
+}
+
 template <typename T>
 __device__ __forceinline__ T geo_vol(const GeoView<T>& g, int64_t e, int k, int sp) {
   return g.vol[e * g.ves + (int64_t)k * g.vks + (int64_t)sp * g.vps];
@@ -123,13 +133,6 @@ struct TraceArgs {
   int64_t state_base, trace_base;
   int count, slot_begin, nvt;
   const int* gate = nullptr;   // see gate_closed
-};
-
-template <int ND, int P>
-struct VolCfg {
-  static constexpr int NSP = Shape<ND, P>::NSP;
-  static constexpr int EPB = NSP >= 256 ? 1 : 256 / NSP;
-  static constexpr int THREADS = EPB * NSP;
 };
 
 // One thread per solution point for the load, then per face point: the q
@@ -294,6 +297,7 @@ __device__ __forceinline__ void trace_body(const TraceArgs<T>& a, int64_t i0, in
 template <typename T, int ND, int P, bool VISC, bool DIAG>
 __global__ void __launch_bounds__(256) trace_kernel(TraceArgs<T> a, int epb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  chain_entry();
   if (gate_closed(a.gate)) return;
   trace_body<T, ND, P, VISC, DIAG>(a, (int64_t)blockIdx.x * epb, epb, smem_raw);
 }
@@ -318,6 +322,7 @@ struct TraceMulti {
 template <typename T, int ND, bool VISC, bool DIAG>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) trace_multi_kernel(const __grid_constant__ TraceMulti<T> m) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  chain_entry();
   if (gate_closed(m.b[0].gate)) return;
   const WorkItem it = m.items[blockIdx.x];
   const int b = it.bucket;
@@ -509,6 +514,7 @@ __global__ void __launch_bounds__(kFaceThreads, (is_dfloat<T>::value || sizeof(T
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int64_t sst[kFaceThreads];       // mixed groups: the faces' slave trace blocks, elements and faces
   __shared__ int32_t sse[kFaceThreads], ssf[kFaceThreads];
+  chain_entry();
   if (gate_closed(m.gate)) return;
   int gi = 0;
   while (gi + 1 < m.ng && (int)blockIdx.x >= m.g[gi + 1].block0) ++gi;
@@ -870,6 +876,7 @@ __device__ __forceinline__ void vol_body(const VolArgs<T>& a, int64_t i0, int ep
 template <typename T, int ND, int P, bool VISC, int MODE, bool DIAG>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : (is_dfloat<T>::value ? 2 : 1)) vol_kernel(VolArgs<T> a, int epb) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  chain_entry();
   if (gate_closed(a.gate)) return;
   vol_body<T, ND, P, VISC, MODE, DIAG>(a, (int64_t)blockIdx.x * epb, epb, smem_raw);
 }
@@ -887,6 +894,7 @@ template <typename T, int ND, bool VISC, int MODE, bool DIAG>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? (ND == 2 && !VISC ? 4 : 3) : (ND == 3 && VISC && MODE == 1 ? 1 : 2))
     vol_multi_kernel(const __grid_constant__ VolMulti<T> m) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  chain_entry();
   if (gate_closed(m.b[0].gate)) return;
   const WorkItem it = m.items[blockIdx.x];
   const int b = it.bucket;

@@ -159,6 +159,7 @@ __device__ __forceinline__ void ctrace_body(const CTraceArgs<T>& a, const CTrace
 template <typename T, int ND, int PF, bool VISC>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 && (PF != 0 || !VISC) ? 8 : PF == 0 ? 4 : 3) ctrace_kernel(const __grid_constant__ CTraceArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  chain_entry();
   if (gate_closed(a.gate)) return;
   if constexpr (PF != 0) {
     ctrace_body<T, ND, PF, VISC>(a, a.b[0], smem_raw);
@@ -882,6 +883,7 @@ constexpr int cface_smem() {
 template <typename T, int ND, int P, bool VISC, bool DIAG>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2) cface_kernel(CFaceArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];   // cface_smem
+  chain_entry();
   if (gate_closed(a.gate)) return;   // before any barrier
   cface_body<T, ND, P, VISC, DIAG>(a, blockIdx.x, reinterpret_cast<T*>(smem_raw));
 }
@@ -899,6 +901,7 @@ __global__ void __launch_bounds__(128, is_dfloat<T>::value || sizeof(T) == 4 ? 4
   constexpr int NV = ND + 2, NFP = ND == 2 ? P : P * P, CT = 2 * NV;
   constexpr int FB = NFP >= 128 ? 1 : 128 / NFP, SC = cface_scratch<ND, P, true, true, 0>();
   __shared__ __align__(16) T sqc[FB * SC];
+  chain_entry();
   const int lf = threadIdx.x / NFP, t = threadIdx.x % NFP;
   const int64_t fidx = (int64_t)blockIdx.x * FB + lf;
   const bool valid = lf < FB && fidx < a.n;
@@ -960,6 +963,7 @@ template <typename T, int ND, bool VISC, bool DIAG>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (VISC ? 4 : 8) : 2) cface_multi_kernel(const __grid_constant__ CFaceMulti<T> m) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sh = reinterpret_cast<T*>(smem_raw);
+  chain_entry();
   if (gate_closed(m.g[0].gate)) return;
   int gi = 0;
   while (gi + 1 < m.ng && (int)blockIdx.x >= m.block0[gi + 1]) ++gi;
