@@ -260,7 +260,14 @@ typedef struct {
   double low_above;        /* exact mode: F uses the residual in precision
                               low_prec while the last ||F|| / ||F(q^{0})|| is
                               above this value, the FP64 residual below it (0:
-                              FP64 throughout).  Convergence is only declared
+                              FP64 throughout).  The FP64 phase also begins
+                              when an iterate reduced ||F|| by less than 10 %
+                              and rounding may be why: FR_F32, at the first
+                              such iterate; FR_DF, once ||F|| is within ten
+                              times the double-float residual's noise, which
+                              one FP64 evaluation measures at the first such
+                              iterate (of a stage, or of the step in
+                              esdirk_step).  Convergence is only declared
                               on an FP64 F, and the last F of the stage is
                               always FP64.                                    */
   int32_t precond;         /* left element-Jacobi preconditioning in GMRES;

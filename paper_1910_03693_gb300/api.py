@@ -369,7 +369,9 @@ class FRContext:
         for j < stage-1 and receives R(q^stage) in slot stage-1 when not None.
         ``low_above`` > 0 (exact mode): F from the residual in
         ``low_precision`` ("df" double-float, or "f32") while ||F||/||F0|| is
-        above it, FP64 below; convergence is decided in FP64."""
+        above it, FP64 below, and also once iterates that reduce ||F|| by less
+        than 10 % may be bound by rounding ("df": ||F|| within ten times the
+        noise, measured by one FP64 evaluation); convergence is decided in FP64."""
         S = len(A)
         tab = _lib.Tableau()
         tab.s = S

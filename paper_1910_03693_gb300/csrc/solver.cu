@@ -1566,9 +1566,11 @@ fr_status gmres_solve(fr_ctx* c, const fr_shifted_op* op, const double* b_dev, d
   return gmres_impl(c, op, R0, b_dev, x_dev, opts, stats, s);
 }
 
-fr_status esdirk_stage(fr_ctx* c, const fr_tableau* tab, int32_t stage, double dt, const double* qn_dev,
-                       double* const* Rstages_dev, double* qi_dev, const fr_newton_opts* o,
-                       fr_stage_stats* st, void* stream) {
+// esdirk_stage; *noise: the rounding noise of the double-float residual,
+// ||F_df - F_64||, negative while it has not been measured.
+static fr_status stage_impl(fr_ctx* c, const fr_tableau* tab, int32_t stage, double dt, const double* qn_dev,
+                            double* const* Rstages_dev, double* qi_dev, const fr_newton_opts* o,
+                            fr_stage_stats* st, void* stream, double* noise) {
   if (!c || !tab || !qn_dev || !qi_dev || !o || !st || tab->s < 2 || tab->s > 6 || stage < 2 ||
       stage > tab->s || !(dt > 0.0) || !(o->tol > 0.0) || !(o->dtau_init > 0.0) || !(o->dtau_max > 0.0) ||
       !(o->low_above >= 0.0) || (o->low_above > 0.0 && o->low_prec != FR_F32 && o->low_prec != FR_DF) ||
@@ -1646,7 +1648,6 @@ fr_status esdirk_stage(fr_ctx* c, const fr_tableau* tab, int32_t stage, double d
   if ((e = evalF(&norm)) != FR_OK) return e;
   st->norm0 = norm;
   double dtau = o->dtau_init, norm_prev = -1.0;
-  int slow_run = 0;   // iterates in a row that reduced ||F|| by less than 10 %
   fr_shifted_op op;
   op.q64_dev = qi_dev;
   op.mode = o->mode;
@@ -1655,20 +1656,25 @@ fr_status esdirk_stage(fr_ctx* c, const fr_tableau* tab, int32_t stage, double d
   op.precond = o->precond;
   for (int m = 0; m < o->max_newton; ++m) {
     // FP64 from here on, starting with this F, once ||F|| is below the
-    // threshold, or once the iteration stalls (a reduction of less than 10 %):
-    // the noise floor of the low-precision residual may lie above the
-    // threshold.  The double-float floor is far below the first iterates
-    // (relative to the fluxes 2^-47): above 1e-3 ||F0|| slow iterates are the
-    // pseudo-time ramp, not noise (on a perturbed Taylor-Green flow the first four
-    // to six iterates reduce ||F|| by less than 10 % each, and all later F, 22 of
-    // 25 a stage, ran in FP64 at 3.1 times the cost), and only the eighth in a
-    // row counts.
+    // threshold, or once an iteration reduced it by less than 10 % and the
+    // noise of the low-precision residual may be why.  FP32: at the first such
+    // iterate.  Double-float: at the first one F is evaluated in FP64 too, which
+    // measures the noise; while ||F|| is more than ten times that, slow
+    // iterates are the pseudo-time ramp and the iteration stays in double-float.
+    // On a perturbed Taylor-Green flow the first four to six iterates reduce
+    // ||F|| by less than 10 % each with the noise ten orders below; in FP64 from
+    // the first of them on, 22 of 25 F a stage ran at 3.1 times the cost.
     const bool slow = norm_prev > 0.0 && norm > 0.9 * norm_prev;
-    slow_run = slow ? slow_run + 1 : 0;
-    const bool stalled = slow && (low32 || norm <= 1e-3 * st->norm0 || slow_run >= 8);
-    if (low && (norm <= o->low_above * st->norm0 || stalled)) {
+    if (low && (norm <= o->low_above * st->norm0 || (slow && (low32 || *noise < 0.0 || norm <= 10.0 * *noise)))) {
+      const bool measure = !low32 && norm > o->low_above * st->norm0 && *noise < 0.0;
+      if (measure) cudaMemcpyAsync(dq, F, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);   // dq: idle until the solve
       low = false;
       if ((e = evalF(&norm)) != FR_OK) return e;
+      if (measure) {
+        vaxpby(c, 1.0, F, -1.0, dq, n, s);
+        if ((e = norm2(c, dq, n, noise, s)) != FR_OK) return e;
+        low = norm > 10.0 * *noise && norm > o->tol * st->norm0;
+      }
     }
     if (!low && norm <= o->tol * st->norm0) {
       st->converged = 1;
@@ -1701,6 +1707,13 @@ fr_status esdirk_stage(fr_ctx* c, const fr_tableau* tab, int32_t stage, double d
   e = cuda_check(cudaStreamSynchronize(s), "esdirk_stage");
   if (e != FR_OK) return e;
   return st->converged ? FR_OK : FR_ERR_NOT_CONVERGED;
+}
+
+fr_status esdirk_stage(fr_ctx* c, const fr_tableau* tab, int32_t stage, double dt, const double* qn_dev,
+                       double* const* Rstages_dev, double* qi_dev, const fr_newton_opts* o,
+                       fr_stage_stats* st, void* stream) {
+  double noise = -1.0;
+  return stage_impl(c, tab, stage, dt, qn_dev, Rstages_dev, qi_dev, o, st, stream, &noise);
 }
 
 fr_status esdirk_step(fr_ctx* c, const fr_tableau* tab, double dt, double* q, const fr_newton_opts* o,
@@ -1746,11 +1759,13 @@ fr_status esdirk_step(fr_ctx* c, const fr_tableau* tab, double dt, double* q, co
   e = launch_residual(c, qn, Rst[0], FR_F64, s);
   if (e != FR_OK) return e;
   cudaMemcpyAsync(qi, qn, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
-  // stage i starts from the value of stage i-1
+  // stage i starts from the value of stage i-1; the fluxes whose rounding makes
+  // the double-float noise are those of one step, so it is measured once
+  double noise = -1.0;
   for (int i = 2; i <= S; ++i) {
     fr_stage_stats st;
     std::memset(&st, 0, sizeof(st));
-    e = esdirk_stage(c, tab, i, dt, qn, Rst, qi, o, &st, stream);
+    e = stage_impl(c, tab, i, dt, qn, Rst, qi, o, &st, stream, &noise);
     if (stats) stats[i - 2] = st;
     if (e != FR_OK) return e;
   }
