@@ -323,7 +323,11 @@ typedef struct {
  * reorder elements into (p, id) buckets, replacing the paper's repartition.
  * q_inout is a state-layout buffer of n_dof_capacity values; on return it
  * holds the state in the new layout.  perm_out (device, optional) receives
- * the element id at each new bucket position. */
+ * the element id at each new bucket position.  Calls of the context that are
+ * in flight on other streams finish on the layout they were queued with: the
+ * new tables are built beside the current ones (about 300 bytes a hexahedron,
+ * allocated on the first call), and when the degrees change the call waits for
+ * the device before it exchanges them. */
 fr_status p_rebucket(fr_ctx* ctx, const double* eta_dev, const double* eta_max_dev,
                      const fr_adapt_opts* opts, void* q_inout_dev, fr_prec prec,
                      int32_t* perm_out_dev, void* stream);

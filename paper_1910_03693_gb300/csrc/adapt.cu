@@ -105,7 +105,7 @@ static void launch_indicator(fr_ctx* c, const T* q, int var, double* eta, cudaSt
     const unsigned grid = (unsigned)((b.count + 127) / 128);
     const double nb = (double)b.count * NSP * sizeof(T);
 #define IND_CASE(PP) \
-  case PP: FR_LAUNCH_B(c, "indicator", s, nb, k_indicator<T, ND, PP><<<grid, 128, 0, s>>>(q, var, c->d_slot_elem, c->d_basis64, g, b.state_base, b.count, b.slot_begin, eta)); break;
+  case PP: FR_LAUNCH_B(c, "indicator", s, nb, k_indicator<T, ND, PP><<<grid, 128, 0, s>>>(q, var, c->lt.slot_elem, c->d_basis64, g, b.state_base, b.count, b.slot_begin, eta)); break;
     switch (P) {
       IND_CASE(2)
       IND_CASE(3)
@@ -321,16 +321,11 @@ fr_status p_rebucket(fr_ctx* c, const double* eta_dev, const double* eta_max_dev
   }
   cudaStream_t s = (cudaStream_t)stream;
   const int E = c->E, nf = c->nf;
-  if (!c->d_adapt_i8) {
-    const bool ok = cudaMalloc(&c->d_adapt_i8, 2 * (size_t)E) == cudaSuccess &&
-                    cudaMalloc(&c->d_old_state_off, sizeof(int64_t) * E) == cudaSuccess &&
-                    cudaMalloc(&c->d_old_elem_slot, sizeof(int32_t) * E) == cudaSuccess &&
-                    cudaMalloc(&c->d_old_slot_p, E) == cudaSuccess;
-    if (!ok) return FR_ERR_NOMEM;
-  }
-  double* xfer = nullptr;
-  fr_status e = ensure_transfer_tables(c, &xfer);
+  if (!c->d_adapt_i8 && cudaMalloc(&c->d_adapt_i8, 2 * (size_t)E) != cudaSuccess) return FR_ERR_NOMEM;
+  fr_status e = layout_spare(c);
   if (e != FR_OK) return e;
+  double* xfer = nullptr;
+  if ((e = ensure_transfer_tables(c, &xfer)) != FR_OK) return e;
   void* tmp = prec == FR_F64 ? (void*)vec64(c, 10) : (void*)vec32(c, 3);
   if (!tmp) return FR_ERR_NOMEM;
   int8_t* pa = c->d_adapt_i8;
@@ -345,18 +340,18 @@ fr_status p_rebucket(fr_ctx* c, const double* eta_dev, const double* eta_max_dev
     FR_LAUNCH(c, "rebucket", s, k_smooth<<<ge, 256, 0, s>>>(pa, c->d_nbr, nf, E, pb));
     std::swap(pa, pb);
   }
-  // keep the old layout for the transfer, then the new one and the state
-  cudaMemcpyAsync(c->d_old_state_off, c->d_state_off, sizeof(int64_t) * E, cudaMemcpyDeviceToDevice, s);
-  cudaMemcpyAsync(c->d_old_elem_slot, c->d_elem_slot, sizeof(int32_t) * E, cudaMemcpyDeviceToDevice, s);
-  cudaMemcpyAsync(c->d_old_slot_p, c->d_slot_p, E, cudaMemcpyDeviceToDevice, s);
-  if ((e = layout_device(c, pa, s)) != FR_OK) return e;
+  // the new layout beside the current one, which the transfer reads and which
+  // calls in flight on other streams of this context may still be reading
+  const LayoutTables& now = c->lt;
+  const LayoutTables& next = c->lt_spare;
+  if ((e = layout_device(c, pa, next, s)) != FR_OK) return e;
   cudaMemcpyAsync(c->d_p, pa, E, cudaMemcpyDeviceToDevice, s);
   const unsigned gc = (unsigned)std::max<int64_t>(1, std::min<int64_t>((c->n_dof_cap + 255) / 256, (int64_t)c->sms * 16));
 #define FR_TRANSFER(T, ND)                                                                                            \
   do {                                                                                                                \
     FR_LAUNCH(c, "rebucket", s,                                                                                       \
-              k_transfer<T, ND><<<E, 128, 0, s>>>((const T*)q_dev, (T*)tmp, c->d_slot_elem, c->d_old_elem_slot,       \
-                                                  c->d_old_state_off, c->d_old_slot_p, pa, c->d_state_off, xfer, E)); \
+              k_transfer<T, ND><<<E, 128, 0, s>>>((const T*)q_dev, (T*)tmp, next.slot_elem, now.elem_slot,            \
+                                                  now.state_off, now.slot_p, pa, next.state_off, xfer, E));           \
     FR_LAUNCH(c, "rebucket", s, k_copy_n<T><<<gc, 256, 0, s>>>((const T*)tmp, (T*)q_dev, layout_n_dof(c)));            \
   } while (0)
   if (c->nd == 2) {
@@ -367,10 +362,14 @@ fr_status p_rebucket(fr_ctx* c, const double* eta_dev, const double* eta_max_dev
     else FR_TRANSFER(float, 3);
   }
 #undef FR_TRANSFER
-  if (perm_out_dev) cudaMemcpyAsync(perm_out_dev, c->d_slot_elem, sizeof(int32_t) * E, cudaMemcpyDeviceToDevice, s);
+  if (perm_out_dev) cudaMemcpyAsync(perm_out_dev, next.slot_elem, sizeof(int32_t) * E, cudaMemcpyDeviceToDevice, s);
   if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_check(cudaGetLastError(), "p_rebucket");
   const int8_t* pnew = layout_degrees(c);
-  if (!std::equal(pnew, pnew + E, c->p.begin())) {   // unchanged degrees: the tables were rewritten as they were
+  if (!std::equal(pnew, pnew + E, c->p.begin())) {   // unchanged degrees: the current tables stay
+    // once nothing in flight reads the current tables (nor the tile table,
+    // which layout_host rewrites), they become the next call's spare ones
+    if (cudaDeviceSynchronize() != cudaSuccess) return cuda_check(cudaGetLastError(), "p_rebucket");
+    std::swap(c->lt, c->lt_spare);
     c->p.assign(pnew, pnew + E);
     if ((e = layout_host(c, s)) != FR_OK) return e;
     if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_check(cudaGetLastError(), "p_rebucket");   // its tile table

@@ -388,11 +388,6 @@ static fr_status create_impl(const fr_mesh_desc* m, const fr_physics* ph, const 
   FR_CUDA(cudaMalloc(&c->d_trace_q, sizeof(double) * c->trace_cap));
   FR_CUDA(cudaMalloc(&c->d_trace_v, sizeof(double) * c->trace_cap));
   FR_CUDA(cudaMalloc(&c->d_fout, sizeof(double) * c->fout_cap));
-  FR_CUDA(cudaMalloc(&c->d_slot_elem, sizeof(int32_t) * E));
-  FR_CUDA(cudaMalloc(&c->d_elem_slot, sizeof(int32_t) * E));
-  FR_CUDA(cudaMalloc(&c->d_canon_off, sizeof(int64_t) * E));
-  FR_CUDA(cudaMalloc(&c->d_state_off, sizeof(int64_t) * E));
-  FR_CUDA(cudaMalloc(&c->d_slot_p, E));
   FR_CUDA(cudaMalloc(&c->d_nbr, sizeof(int32_t) * E * nf));
   FR_CUDA(cudaMalloc(&c->d_status, sizeof(int)));
   FR_CUDA(cudaMemset(c->d_status, 0, sizeof(int)));
@@ -426,23 +421,17 @@ static void destroy_impl(fr_ctx* c) {
   cudaFree(c->d_fout);
   cudaFree(c->d_fbar);
   cudaFree(c->d_trbar);
-  cudaFree(c->d_slot_elem);
-  cudaFree(c->d_elem_slot);
-  cudaFree(c->d_canon_off);
-  cudaFree(c->d_state_off);
-  cudaFree(c->d_slot_p);
+  layout_free(c->lt);
+  layout_free(c->lt_spare);
   cudaFree(c->d_nbr);
   clear_graphs(c);
   cudaFree(c->d_p);
   cudaFree(c->d_nbr_face);
   cudaFree(c->d_orient);
-  cudaFree(c->d_recs);
-  cudaFree(c->d_brecs);
   cudaFree(c->d_lay);
   cudaFree(c->d_face_hist);
   if (c->h_lay) cudaFreeHost(c->h_lay);
   cudaFree(c->d_work);
-  cudaFree(c->d_fnbr);
   cudaFree(c->d_status);
   cudaFree(c->d_jidx);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
@@ -464,9 +453,6 @@ static void destroy_impl(fr_ctx* c) {
   cudaFree(c->d_xfer);
   cudaFree(c->d_adapt_i8);
   cudaFree(c->d_adapt_f64);
-  cudaFree(c->d_old_state_off);
-  cudaFree(c->d_old_elem_slot);
-  cudaFree(c->d_old_slot_p);
   delete c;
 }
 

@@ -217,7 +217,7 @@ static TraceArgs<T> trace_args(fr_ctx* c, const Bucket& b, const T* q, T* trace)
   a.gate = c->gate;
   a.q = q;
   a.trace = trace;
-  a.slot_elem = c->d_slot_elem;
+  a.slot_elem = c->lt.slot_elem;
   a.basis = basis_ptr<T>(c);
   a.geo = geo_view<T>(c, b.p);
   a.state_base = b.state_base;
@@ -300,7 +300,7 @@ static VolArgs<T> vol_args(fr_ctx* c, const Bucket& b, const T* q, const T* v, T
   a.out_neg64 = out_neg64;
   a.out64 = out64;
   a.fout = (const T*)c->d_fout;
-  a.slot_elem = c->d_slot_elem;
+  a.slot_elem = c->lt.slot_elem;
   a.basis = basis_ptr<T>(c);
   a.geo = geo_view<T>(c, b.p);
   a.gamma = (T)c->phys.gamma;
@@ -565,8 +565,8 @@ static void jvp_fused_impl(fr_ctx* c, const T* q, const T* v, T* Jv, cudaStream_
     a.trv = trv;
     a.out = Jv;
     a.out_neg64 = neg64;
-    a.nbr = (const FusedNbr*)c->d_fnbr;
-    a.slot_elem = c->d_slot_elem;
+    a.nbr = c->lt.fnbr;
+    a.slot_elem = c->lt.slot_elem;
     a.basis = basis_ptr<T>(c);
     a.geo = geo_view<T>(c, b.p);
     a.gamma = (T)c->phys.gamma;
@@ -891,7 +891,7 @@ static void vjp_impl(fr_ctx* c, const T* q, const T* w, T* out, cudaStream_t s) 
     a.out = out;
     a.fout = (const T*)c->d_fout;
     a.fbar = (T*)c->d_fbar;
-    a.slot_elem = c->d_slot_elem;
+    a.slot_elem = c->lt.slot_elem;
     a.basis = basis_ptr<T>(c);
     a.geo = geo_view<T>(c, b.p);
     a.gamma = (T)c->phys.gamma;

@@ -153,6 +153,18 @@ struct PcLane {
   void* fout = nullptr;
 };
 
+// The device tables of one layout (layout.cu).
+struct LayoutTables {
+  int32_t* slot_elem = nullptr;   // [E]
+  int32_t* elem_slot = nullptr;   // [E] slot of each element
+  int64_t* canon_off = nullptr;   // [E] canonical offset of the element at each slot
+  int64_t* state_off = nullptr;   // [E] state offset of the element at each slot
+  int8_t* slot_p = nullptr;       // [E] degree at each slot
+  FaceRec* recs = nullptr;        // interior faces, grouped
+  BndRec* brecs = nullptr;        // boundary faces, grouped
+  FusedNbr* fnbr = nullptr;       // [E][nf] in slot order; null: the fused JVP is not offered
+};
+
 struct PhysParams {
   double gamma, mu, Pr, kappa;
   double q_inf[5];
@@ -199,11 +211,8 @@ struct fr_ctx {
   // layout
   std::vector<frgb::Bucket> buckets;     // one per degree present, ascending p
   int64_t n_dof = 0, n_dof_cap = 0;
-  int32_t* d_slot_elem = nullptr;        // [E]
-  int64_t* d_canon_off = nullptr;        // [E] canonical offset of the element at each slot
-  int64_t* d_state_off = nullptr;        // [E] state offset of the element at each slot
-  int8_t* d_slot_p = nullptr;            // [E] degree at each slot
-  int32_t* d_elem_slot = nullptr;        // [E] slot of each element
+  frgb::LayoutTables lt;                 // tables of the current layout
+  frgb::LayoutTables lt_spare;           // p_rebucket fills these while work in flight may read lt
   // workspaces (bytes sized for FP64 at capacity)
   int nvt = 0;                           // trace components per face point
   int64_t trace_cap = 0, fout_cap = 0;
@@ -216,8 +225,6 @@ struct fr_ctx {
   int8_t* d_p = nullptr;                 // [E] current degree of every element
   int8_t* d_nbr_face = nullptr;          // [E][nf]
   int8_t* d_orient = nullptr;            // [E][nf]
-  frgb::FaceRec* d_recs = nullptr;       // interior faces, grouped
-  frgb::BndRec* d_brecs = nullptr;       // boundary faces, grouped
   void* d_lay = nullptr;                 // counts read back by the host, sort scratch
   int* d_face_hist = nullptr;            // face sort scratch
   void* h_lay = nullptr;                 // pinned mirror of the counts, then the degrees
@@ -261,11 +268,9 @@ struct fr_ctx {
   frgb::WorkItem* d_work = nullptr;
   int n_work = 0;
   // fused JVP: every face interior and conforming (then the exact JVP runs as
-  // compact traces + one face-and-volume kernel); the neighbour of every
-  // element face, slot-major (frgb::FusedNbr)
+  // compact traces + one face-and-volume kernel)
   bool fused_ok = false;
   bool use_fused = true;
-  void* d_fnbr = nullptr;
   // CUDA graph of one Arnoldi matrix-vector product -J(q) V[j] (per precision),
   // with the column index read from d_jidx; keyed by the pointers it captured
   cudaGraphExec_t jvp_graph[2] = {nullptr, nullptr};
@@ -299,9 +304,6 @@ struct fr_ctx {
   double* d_xfer = nullptr;              // prolongation / projection matrices [Po][Pn][6][6]
   int8_t* d_adapt_i8 = nullptr;
   double* d_adapt_f64 = nullptr;
-  int64_t* d_old_state_off = nullptr;
-  int32_t* d_old_elem_slot = nullptr;
-  int8_t* d_old_slot_p = nullptr;
 };
 
 namespace frgb {
@@ -325,7 +327,9 @@ void free_pc_lanes(fr_ctx* c);
 fr_status rebuild_work_table(fr_ctx* c, cudaStream_t s);
 // layout.cu
 fr_status layout_alloc(fr_ctx* c);
-fr_status layout_device(fr_ctx* c, const int8_t* d_p, cudaStream_t s);
+fr_status layout_spare(fr_ctx* c);
+void layout_free(LayoutTables& t);
+fr_status layout_device(fr_ctx* c, const int8_t* d_p, const LayoutTables& t, cudaStream_t s);
 fr_status layout_host(fr_ctx* c, cudaStream_t s);
 fr_status build_layout(fr_ctx* c);
 const int8_t* layout_degrees(const fr_ctx* c);

@@ -101,14 +101,14 @@ fr_status launch_pack(fr_ctx* c, const double* canon, void* q, fr_prec prec, boo
   const unsigned g = (unsigned)std::min<int64_t>(c->E, 1 << 20);
   if (!unpack) {
     if (prec == FR_F64)
-      FR_LAUNCH_B(c, "pack", s, (double)c->n_dof * (8 + (prec == FR_F64 ? 8 : 4)), pack_kernel<double><<<g, 128, 0, s>>>(canon, (double*)q, c->d_canon_off, c->d_state_off, c->d_slot_p, c->E, c->nd, c->nv));
+      FR_LAUNCH_B(c, "pack", s, (double)c->n_dof * (8 + (prec == FR_F64 ? 8 : 4)), pack_kernel<double><<<g, 128, 0, s>>>(canon, (double*)q, c->lt.canon_off, c->lt.state_off, c->lt.slot_p, c->E, c->nd, c->nv));
     else
-      FR_LAUNCH_B(c, "pack", s, (double)c->n_dof * (8 + (prec == FR_F64 ? 8 : 4)), pack_kernel<float><<<g, 128, 0, s>>>(canon, (float*)q, c->d_canon_off, c->d_state_off, c->d_slot_p, c->E, c->nd, c->nv));
+      FR_LAUNCH_B(c, "pack", s, (double)c->n_dof * (8 + (prec == FR_F64 ? 8 : 4)), pack_kernel<float><<<g, 128, 0, s>>>(canon, (float*)q, c->lt.canon_off, c->lt.state_off, c->lt.slot_p, c->E, c->nd, c->nv));
   } else {
     if (prec == FR_F64)
-      FR_LAUNCH_B(c, "pack", s, (double)c->n_dof * (8 + (prec == FR_F64 ? 8 : 4)), unpack_kernel<double><<<g, 128, 0, s>>>((const double*)q, const_cast<double*>(canon), c->d_canon_off, c->d_state_off, c->d_slot_p, c->E, c->nd, c->nv));
+      FR_LAUNCH_B(c, "pack", s, (double)c->n_dof * (8 + (prec == FR_F64 ? 8 : 4)), unpack_kernel<double><<<g, 128, 0, s>>>((const double*)q, const_cast<double*>(canon), c->lt.canon_off, c->lt.state_off, c->lt.slot_p, c->E, c->nd, c->nv));
     else
-      FR_LAUNCH_B(c, "pack", s, (double)c->n_dof * (8 + (prec == FR_F64 ? 8 : 4)), unpack_kernel<float><<<g, 128, 0, s>>>((const float*)q, const_cast<double*>(canon), c->d_canon_off, c->d_state_off, c->d_slot_p, c->E, c->nd, c->nv));
+      FR_LAUNCH_B(c, "pack", s, (double)c->n_dof * (8 + (prec == FR_F64 ? 8 : 4)), unpack_kernel<float><<<g, 128, 0, s>>>((const float*)q, const_cast<double*>(canon), c->lt.canon_off, c->lt.state_off, c->lt.slot_p, c->E, c->nd, c->nv));
   }
   return cuda_check(cudaGetLastError(), "pack kernel launch");
 }

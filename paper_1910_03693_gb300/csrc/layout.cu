@@ -328,15 +328,45 @@ fr_status rebuild_work_table(fr_ctx* c, cudaStream_t s) {
   return st;
 }
 
+template <typename T>
+static bool get(T** p, size_t bytes) {
+  return cudaMalloc((void**)p, std::max<size_t>(bytes, 1)) == cudaSuccess;
+}
+
+void layout_free(LayoutTables& t) {
+  cudaFree(t.slot_elem);
+  cudaFree(t.elem_slot);
+  cudaFree(t.canon_off);
+  cudaFree(t.state_off);
+  cudaFree(t.slot_p);
+  cudaFree(t.recs);
+  cudaFree(t.brecs);
+  cudaFree(t.fnbr);
+  t = LayoutTables{};
+}
+
+// One set of tables but fnbr; all of it or nothing.
+static fr_status tables_alloc(fr_ctx* c, LayoutTables& t) {
+  const int64_t E = c->E;
+  int64_t inner = 0, bnd = 0;
+  for (int32_t n : c->nbr) (n >= 0 ? inner : bnd) += 1;
+  if (get(&t.slot_elem, sizeof(int32_t) * E) && get(&t.elem_slot, sizeof(int32_t) * E) &&
+      get(&t.canon_off, sizeof(int64_t) * E) && get(&t.state_off, sizeof(int64_t) * E) && get(&t.slot_p, E) &&
+      get(&t.recs, sizeof(FaceRec) * (inner / 2)) && get(&t.brecs, sizeof(BndRec) * bnd))
+    return FR_OK;
+  cudaGetLastError();
+  layout_free(t);
+  set_error("layout tables: allocation failed");
+  return FR_ERR_NOMEM;
+}
+
 // Buffers whose size the mesh decides, and the pinned mirror of what the host reads.
 fr_status layout_alloc(fr_ctx* c) {
   const int64_t E = c->E, ef = E * c->nf;
-  int64_t inner = 0, bnd = 0;
-  for (int32_t n : c->nbr) (n >= 0 ? inner : bnd) += 1;
   const int nb = (int)((E + kSortBlock - 1) / kSortBlock), nfb = (int)((ef + kFaceBlock - 1) / kFaceBlock);
-  auto get = [](auto** p, size_t bytes) { return cudaMalloc((void**)p, std::max<size_t>(bytes, 1)) == cudaSuccess; };
+  const fr_status st = tables_alloc(c, c->lt);
+  if (st != FR_OK) return st;
   const bool ok = get(&c->d_p, E) && get(&c->d_nbr_face, ef) && get(&c->d_orient, ef) &&
-                  get(&c->d_recs, sizeof(FaceRec) * (inner / 2)) && get(&c->d_brecs, sizeof(BndRec) * bnd) &&
                   get(&c->d_lay, sizeof(LayoutMeta) + sizeof(int64_t) * nb + sizeof(int) * 2 * nb * kND) &&
                   get(&c->d_face_hist, sizeof(int) * (size_t)kFaceKeys * nfb) &&
                   cudaMallocHost(&c->h_lay, sizeof(LayoutMeta) + E) == cudaSuccess;
@@ -345,9 +375,10 @@ fr_status layout_alloc(fr_ctx* c) {
     set_error("layout tables: allocation failed");
     return FR_ERR_NOMEM;
   }
-  if (bnd == 0 && !get(&c->d_fnbr, sizeof(FusedNbr) * ef)) {   // the fused JVP is then not offered
+  const bool closed = std::all_of(c->nbr.begin(), c->nbr.end(), [](int32_t n) { return n >= 0; });
+  if (closed && !get(&c->lt.fnbr, sizeof(FusedNbr) * ef)) {    // the fused JVP is then not offered
     cudaGetLastError();
-    c->d_fnbr = nullptr;
+    c->lt.fnbr = nullptr;
   }
   if (!get(&c->d_work, sizeof(WorkItem) * (E + 2 * kND))) {    // launches then go per bucket
     cudaGetLastError();
@@ -359,11 +390,23 @@ fr_status layout_alloc(fr_ctx* c) {
   return cuda_check(cudaGetLastError(), "layout tables");
 }
 
+// The second set of tables, on the first change of degrees.
+fr_status layout_spare(fr_ctx* c) {
+  if (c->lt_spare.slot_elem) return FR_OK;
+  const fr_status st = tables_alloc(c, c->lt_spare);
+  if (st != FR_OK || !c->lt.fnbr) return st;
+  if (get(&c->lt_spare.fnbr, sizeof(FusedNbr) * (size_t)c->E * c->nf)) return FR_OK;
+  cudaGetLastError();
+  layout_free(c->lt_spare);
+  set_error("layout tables: allocation failed");
+  return FR_ERR_NOMEM;
+}
+
 const int64_t* layout_n_dof(const fr_ctx* c) { return &static_cast<const LayoutMeta*>(c->d_lay)->n_dof; }
 
-// Every device table of the layout of the degrees d_p (element order), queued
-// on s, and the copies the host needs (the degrees too when p_changed).
-fr_status layout_device(fr_ctx* c, const int8_t* d_p, cudaStream_t s) {
+// Every device table of the layout of the degrees d_p (element order) into t,
+// queued on s, and the copies the host needs.
+fr_status layout_device(fr_ctx* c, const int8_t* d_p, const LayoutTables& t, cudaStream_t s) {
   const int E = c->E, nf = c->nf;
   const int64_t ef = (int64_t)E * nf;
   const int nb = (E + kSortBlock - 1) / kSortBlock, nfb = (int)((ef + kFaceBlock - 1) / kFaceBlock);
@@ -376,16 +419,15 @@ fr_status layout_device(fr_ctx* c, const int8_t* d_p, cudaStream_t s) {
   FR_LAUNCH(c, "rebucket", s,
             k_sort_scan<<<1, 32 * (kND + 1), 0, s>>>(blk_counts, nb, c->nd, c->nv, blk_off, blk_canon, meta));
   FR_LAUNCH(c, "rebucket", s,
-            k_sort_scatter<<<nb, kSortBlock, 0, s>>>(d_p, E, c->nd, c->nv, blk_off, blk_canon, meta, c->d_slot_elem,
-                                                     c->d_elem_slot, c->d_slot_p, c->d_state_off, c->d_canon_off));
+            k_sort_scatter<<<nb, kSortBlock, 0, s>>>(d_p, E, c->nd, c->nv, blk_off, blk_canon, meta, t.slot_elem,
+                                                     t.elem_slot, t.slot_p, t.state_off, t.canon_off));
   FR_LAUNCH(c, "rebucket", s, k_face_count<<<nfb, kFaceBlock, 0, s>>>(m, nfb, c->d_face_hist));
   FR_LAUNCH(c, "rebucket", s, k_face_scan<<<kFaceKeys, 32, 0, s>>>(c->d_face_hist, nfb, meta));
   FR_LAUNCH(c, "rebucket", s,
-            k_face_scatter<<<nfb, kFaceBlock, 0, s>>>(m, nfb, c->d_face_hist, meta, c->d_elem_slot, c->d_recs, c->d_brecs));
-  if (c->d_fnbr)
+            k_face_scatter<<<nfb, kFaceBlock, 0, s>>>(m, nfb, c->d_face_hist, meta, t.elem_slot, t.recs, t.brecs));
+  if (t.fnbr)
     FR_LAUNCH(c, "rebucket", s,
-              k_fused_table<<<(unsigned)((ef + 255) / 256), 256, 0, s>>>(m, meta, c->d_slot_elem, c->d_elem_slot,
-                                                                         (FusedNbr*)c->d_fnbr));
+              k_fused_table<<<(unsigned)((ef + 255) / 256), 256, 0, s>>>(m, meta, t.slot_elem, t.elem_slot, t.fnbr));
   cudaMemcpyAsync(c->h_lay, meta, sizeof(LayoutMeta), cudaMemcpyDeviceToHost, s);
   cudaMemcpyAsync(static_cast<char*>(c->h_lay) + sizeof(LayoutMeta), d_p, E, cudaMemcpyDeviceToHost, s);
   return cuda_check(cudaGetLastError(), "layout");
@@ -433,7 +475,7 @@ fr_status layout_host(fr_ctx* c, cudaStream_t s) {
     g.pm = k / 3 / kMaxDeg + 1;
     g.ps = k / 3 % kMaxDeg + 1;
     g.n = n;
-    g.d_recs = c->d_recs + at;
+    g.d_recs = c->lt.recs + at;
     at += n;
     conforming = conforming && g.pm == g.ps;
     c->fgroups.push_back(g);
@@ -446,13 +488,13 @@ fr_status layout_host(fr_ctx* c, cudaStream_t s) {
     g.p = k / 2 + 1;
     g.kind = k % 2 == 0 ? FR_BC_FARFIELD : FR_BC_WALL;
     g.n = n;
-    g.d_recs = c->d_brecs + at;
+    g.d_recs = c->lt.brecs + at;
     at += n;
     c->bgroups.push_back(g);
   }
   // the compact face kernel finds a block at the trace-gradient offset scaled
   // by ct / nvt: true when every bucket's compact base is its trace base so scaled
-  c->fused_ok = c->d_fnbr && c->bgroups.empty() && conforming && cb <= c->trace_cap;
+  c->fused_ok = c->lt.fnbr && c->bgroups.empty() && conforming && cb <= c->trace_cap;
   for (const auto& b : c->buckets)
     if (b.trace_base % c->nvt != 0 || b.trace_base / c->nvt * ct != b.ctrace_base) c->fused_ok = false;
   rebuild_work_table(c, s);   // a failure leaves no table: launches go per bucket
@@ -461,7 +503,7 @@ fr_status layout_host(fr_ctx* c, cudaStream_t s) {
 
 // The layout of the degrees in d_p, complete on return (context creation).
 fr_status build_layout(fr_ctx* c) {
-  fr_status st = layout_device(c, c->d_p, nullptr);
+  fr_status st = layout_device(c, c->d_p, c->lt, nullptr);
   if (st == FR_OK) st = cuda_check(cudaStreamSynchronize(nullptr), "layout");
   if (st == FR_OK) st = layout_host(c, nullptr);
   if (st == FR_OK) st = cuda_check(cudaStreamSynchronize(nullptr), "layout");

@@ -555,7 +555,7 @@ fr_status fr_precond_build(fr_ctx* c, const double* q64_dev, double sigma, void*
   for (int col = 0; col < c->n_colors && kmax > 0 && e == FR_OK; ++col) {
     auto probe = [&](const PcLane& ln, int k, int next) {
       FR_LAUNCH(c, "precond_build", ln.s,
-                k_pc_probe<<<pg, 256, 0, ln.s>>>(pb, c->d_pc, c->d_pc_off, ln.J, ln.v, c->d_state_off, c->d_slot_color,
+                k_pc_probe<<<pg, 256, 0, ln.s>>>(pb, c->d_pc, c->d_pc_off, ln.J, ln.v, c->lt.state_off, c->d_slot_color,
                                                  col, k, next, sg));
     };
     for (int l = 0; l < nl && l < kmax; ++l) {
@@ -650,7 +650,7 @@ static fr_status precond_apply_t(fr_ctx* c, double a, const VT* w, double b, con
   }
   FR_LAUNCH_B(c, "precond_apply", s, bytes,
               k_pc_apply<VT><<<(unsigned)pb.first[pb.n], threads, smem, s>>>(
-                  pb, c->d_pc, c->d_pc_off, c->d_state_off, a, w, b, u, z, 1.0 / c->pc_sigma, gate, bscale));
+                  pb, c->d_pc, c->d_pc_off, c->lt.state_off, a, w, b, u, z, 1.0 / c->pc_sigma, gate, bscale));
   return cuda_check(cudaGetLastError(), "precond_apply");
 }
 
