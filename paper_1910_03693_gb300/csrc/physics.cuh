@@ -104,13 +104,15 @@ __device__ __forceinline__ Dual<T> dsqrt(Dual<T> x) {
   return {r, x.d / (T(2) * r)};
 }
 // 1 / x; the tangent -x.d / x^2 from the reciprocal, not by a second division
-// (a division is the longest operation here, of the FP64 pipe above all)
+// (a division is the longest operation here, of the FP64 pipe above all), and
+// not from 1 / x^2, which leaves FP32's range where x.d / x and 1 / x do not
+// (|x| < 5.4e-20 or > 1e19: densities and squared sound speeds in other units)
 template <typename S>
 __device__ __forceinline__ S recip(S x) { return S(1) / x; }
 template <typename T>
 __device__ __forceinline__ Dual<T> recip(Dual<T> x) {
   const T r = T(1) / x.v;
-  return {r, -(r * r) * x.d};
+  return {r, -(r * x.d) * r};
 }
 // sqrt(x) given its value c
 template <typename T>
