@@ -424,7 +424,11 @@ fr_status esdirk_step(fr_ctx* ctx, const fr_tableau* tab, double dt, double* q_i
 #define FR_TUNE_GRAPHS 2        /* host-driven GMRES: the Arnoldi products
                                    replayed from a CUDA graph               */
 #define FR_TUNE_DIAG_METRICS 4  /* 3D meshes of axis-aligned affine elements:
-                                   kernels that skip the zero metric terms   */
+                                   kernels that skip the zero metric terms
+                                   (viscous: where both sides of every
+                                   interior face have the same axis and
+                                   tangential extents, as fr_create checks;
+                                   elsewhere the general ones)              */
 #define FR_TUNE_FUSED_JVP 8     /* meshes whose faces are all interior and
                                    conforming (same degree both sides, no
                                    boundary): the exact JVP from compact

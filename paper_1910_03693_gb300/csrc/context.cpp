@@ -151,6 +151,37 @@ static bool element_is_affine(const fr_ctx* c, int e) {
   return twist <= 1e-13 * scale;
 }
 
+// Whether both sides of every interior face have the same axis and the same
+// tangential metric (axis-aligned elements, metrics g as below).  The viscous
+// diagonal-metric face kernels rely on it: they take the tangential part of the
+// common gradient from q^com with the master's metric, and the slave's normal
+// metric on the master's axis.  The connectivity alone does not ensure it
+// (layers of different extent glued together, axes exchanged or reflected
+// across a face).  Extents are compared to the rounding of the nodes they are
+// differences of.
+static bool faces_match(const fr_ctx* c, const std::vector<double>& g, int nk) {
+  const int nd = c->nd, nf = c->nf;
+  double xmax = 0.0;
+  for (double x : c->nodes) xmax = std::max(xmax, std::fabs(x));
+  auto extent = [&](int e, int j) {   // |J| / S_jj
+    const double* m = g.data() + (size_t)e * nk;
+    return m[nd * nd] / m[j * nd + j];
+  };
+  for (int e = 0; e < c->E; ++e)
+    for (int f = 0; f < nf; ++f) {
+      const int n = c->nbr[(size_t)e * nf + f], o = c->orient[(size_t)e * nf + f];
+      if (n < 0) continue;
+      const int d = f >> 1;
+      if ((c->nbr_face[(size_t)e * nf + f] >> 1) != d || (o & 1)) return false;
+      for (int j = 0, k = 0; j < nd; ++j) {
+        if (j == d) continue;
+        const double a = extent(e, j), b = extent(n, j), flip = (o >> ++k) & 1 ? -1.0 : 1.0;
+        if (std::fabs(a - flip * b) > 1e-12 * std::fabs(a) + 64.0 * 2.2e-16 * xmax) return false;
+      }
+    }
+  return true;
+}
+
 void collect_graph_timers(fr_ctx* c) {
   for (int k = 0; k < 2; ++k)
     if (c->graph_timers_live[k]) {
@@ -352,7 +383,7 @@ static fr_status create_impl(const fr_mesh_desc* m, const fr_physics* ph, const 
       }
       derive(v1.data(), ipow(2, nd), g.data() + (size_t)e * NKF, 1, true);
     }
-    c->diag_mesh = diag;
+    c->diag_mesh = diag && (!c->visc || faces_match(c, g, NKF));
     c->diag = c->diag_mesh && c->use_diag;
     FR_TRY(upload_cast(g, &c->d_gaff64));
     FR_TRY(upload_cast(g, &c->d_gaff32));

@@ -176,7 +176,7 @@ struct PhysParams {
 struct fr_ctx {
   int nd = 0, nv = 0, nf = 0, E = 0, geom_order = 1, p_min = 1, p_max = 1;
   bool affine = false, visc = false;
-  bool diag_mesh = false;   // 3D, affine, every metric diagonal (axis-aligned boxes)
+  bool diag_mesh = false;   // 3D, affine, every metric diagonal (axis-aligned boxes), faces that match (viscous)
   bool diag = false;        // diag_mesh and the diagonal-metric kernels enabled
   frgb::PhysParams phys{};
   int device = 0;

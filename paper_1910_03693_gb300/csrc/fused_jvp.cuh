@@ -627,8 +627,9 @@ __device__ __forceinline__ void cface_geo(const CFaceArgs<T>& a, const FaceRec& 
   }
 }
 
-// Diagonal metrics (axis-aligned elements; both sides of a conforming face then
-// have the same tangential metric): the tangential part of the common gradient
+// Diagonal metrics (axis-aligned elements; both sides of a conforming face
+// have the same tangential metric, which context creation checks before it
+// chooses these kernels): the tangential part of the common gradient
 // is the tangential derivative of q^com itself, taken once from q^com of the
 // whole face in shared memory instead of from both sides' traces.  kCommonTang
 // faces need that memory (cface_scratch values a face) and a barrier among the
