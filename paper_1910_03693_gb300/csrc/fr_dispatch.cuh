@@ -962,8 +962,10 @@ static void vjp_impl(fr_ctx* c, const T* q, const T* w, T* out, cudaStream_t s) 
 
 // ---------------------------------------------------------------------------
 // Autotuner: elements per CTA of the trace and volume kernels for every
-// degree present, then one launch per bucket vs the multi-bucket launch.
-// Candidates are timed with CUDA events (best of `reps`) on the caller's state.
+// degree present, then one launch per bucket vs the multi-bucket launch.  The
+// default rule's value is a candidate beside the powers of two and a full CTA,
+// and where it wins the slot stays 0: the rule then also follows a change of
+// degrees.  Candidates are timed with CUDA events (best of `reps`) on the caller's state.
 // ---------------------------------------------------------------------------
 template <typename F>
 static float time_best(int reps, cudaStream_t s, F&& f) {
@@ -999,10 +1001,13 @@ static void autotune_impl(fr_ctx* c, const T* q, T* scratch, int reps, cudaStrea
     if (kind == 2) jvp_impl<T, ND, VISC, DIAG>(c, q, q, scratch, s);
     for (const auto& b : c->buckets) {
       const int P = b.p + 1, nsp = nsp_of(ND, P);
-      std::vector<int> cand;
-      for (int e = 1; e * nsp <= 256; e *= 2) cand.push_back(e);
-      const int dflt = nsp >= 256 ? 1 : 256 / nsp;
-      if (std::find(cand.begin(), cand.end(), dflt) == cand.end()) cand.push_back(dflt);
+      const int dflt = epb_by_rule(epb_rule<T>(), nsp, mesh_threads(c));
+      std::vector<int> cand{dflt};
+      auto add = [&](int e) {
+        if (std::find(cand.begin(), cand.end(), e) == cand.end()) cand.push_back(e);
+      };
+      for (int e = 1; e * nsp <= 256; e *= 2) add(e);
+      add(std::max(1, 256 / nsp));
       float best = 1e30f;
       int best_e = dflt;
       for (int e : cand) {
@@ -1045,15 +1050,13 @@ static void autotune_impl(fr_ctx* c, const T* q, T* scratch, int reps, cudaStrea
           best_e = e;
         }
       }
-      c->epb_tab[prec][kind][P] = best_e;
+      c->epb_tab[prec][kind][P] = best_e == dflt ? 0 : best_e;
     }
   }
   (void)trv;
   clear_work_cache(c);
   // per kernel kind: one launch per bucket against one multi-bucket launch,
-  // with the tuned elements per CTA (the multi kernel carries the register
-  // footprint of its largest degree, so large meshes usually prefer separate
-  // launches and small batches of buckets the single one)
+  // with the tuned elements per CTA (see use_multi for both sides' times)
   c->multi_launch = true;
   if (c->buckets.size() > 1) {
     residual_impl<T, ND, VISC, DIAG>(c, q, scratch, s);
