@@ -265,8 +265,8 @@ typedef struct {
                               and rounding may be why: FR_F32, at the first
                               such iterate; FR_DF, once ||F|| is within ten
                               times the double-float residual's noise, which
-                              one FP64 evaluation measures at the first such
-                              iterate (of a stage, or of the step in
+                              the first such iterate has measured against an
+                              FP64 residual (of F; once a step, of q^n, in
                               esdirk_step).  Convergence is only declared
                               on an FP64 F, and the last F of the stage is
                               always FP64.                                    */

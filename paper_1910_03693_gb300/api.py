@@ -371,7 +371,7 @@ class FRContext:
         ``low_precision`` ("df" double-float, or "f32") while ||F||/||F0|| is
         above it, FP64 below, and also once iterates that reduce ||F|| by less
         than 10 % may be bound by rounding ("df": ||F|| within ten times the
-        noise, measured by one FP64 evaluation); convergence is decided in FP64."""
+        noise, measured against an FP64 evaluation); convergence is decided in FP64."""
         S = len(A)
         tab = _lib.Tableau()
         tab.s = S

@@ -1566,11 +1566,17 @@ fr_status gmres_solve(fr_ctx* c, const fr_shifted_op* op, const double* b_dev, d
   return gmres_impl(c, op, R0, b_dev, x_dev, opts, stats, s);
 }
 
-// esdirk_stage; *noise: the rounding noise of the double-float residual,
-// ||F_df - F_64||, negative while it has not been measured.
+// What is known of the rounding noise of the double-float residual: its norm,
+// negative while it has not been measured, and (esdirk_step) the FP64 residual
+// of q^n to measure it against.
+struct DfNoise {
+  double norm = -1.0;
+  const double* Rn = nullptr;
+};
+
 static fr_status stage_impl(fr_ctx* c, const fr_tableau* tab, int32_t stage, double dt, const double* qn_dev,
                             double* const* Rstages_dev, double* qi_dev, const fr_newton_opts* o,
-                            fr_stage_stats* st, void* stream, double* noise) {
+                            fr_stage_stats* st, void* stream, DfNoise* noise) {
   if (!c || !tab || !qn_dev || !qi_dev || !o || !st || tab->s < 2 || tab->s > 6 || stage < 2 ||
       stage > tab->s || !(dt > 0.0) || !(o->tol > 0.0) || !(o->dtau_init > 0.0) || !(o->dtau_max > 0.0) ||
       !(o->low_above >= 0.0) || (o->low_above > 0.0 && o->low_prec != FR_F32 && o->low_prec != FR_DF) ||
@@ -1658,25 +1664,37 @@ static fr_status stage_impl(fr_ctx* c, const fr_tableau* tab, int32_t stage, dou
     // FP64 from here on, starting with this F, once ||F|| is below the
     // threshold, or once an iteration reduced it by less than 10 % and the
     // noise of the low-precision residual may be why.  FP32: at the first such
-    // iterate.  Double-float: at the first one F is evaluated in FP64 too, which
-    // measures the noise; while ||F|| is more than ten times that, slow
-    // iterates are the pseudo-time ramp and the iteration stays in double-float.
-    // On a perturbed Taylor-Green flow the first four to six iterates reduce
-    // ||F|| by less than 10 % each with the noise ten orders below; in FP64 from
-    // the first of them on, 22 of 25 F a stage ran at 3.1 times the cost.
+    // iterate.  Double-float: the first one has the noise measured, by one
+    // more residual; while ||F|| is more than ten times that, slow iterates are
+    // the pseudo-time ramp and the iteration stays in double-float.  On a
+    // perturbed Taylor-Green flow the first four to six iterates reduce ||F|| by
+    // less than 10 % each with the noise ten orders below; in FP64 from the
+    // first of them on, 22 of 25 F a stage ran at 3.1 times the cost.
     const bool slow = norm_prev > 0.0 && norm > 0.9 * norm_prev;
-    if (low && (norm <= o->low_above * st->norm0 || (slow && (low32 || *noise < 0.0 || norm <= 10.0 * *noise)))) {
-      const bool measure = !low32 && norm > o->low_above * st->norm0 && *noise < 0.0;
-      if (measure) cudaMemcpyAsync(dq, F, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);   // dq: idle until the solve
-      low = false;
-      if ((e = evalF(&norm)) != FR_OK) return e;
-      if (measure) {
-        vaxpby(c, 1.0, F, -1.0, dq, n, s);
-        if ((e = norm2(c, dq, n, noise, s)) != FR_OK) return e;
-        low = norm > 10.0 * *noise && norm > o->tol * st->norm0;
+    bool exact = !low;   // F is the FP64 one
+    if (low && !low32 && slow && norm > o->low_above * st->norm0 && noise->norm < 0.0) {
+      // dq is idle until the solve
+      if (noise->Rn) {
+        if ((e = launch_residual(c, qn_dev, dq, FR_DF, s)) != FR_OK) return e;
+        vaxpby(c, -1.0, noise->Rn, 1.0, dq, n, s);
+      } else {
+        cudaMemcpyAsync(dq, F, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
+        low = false;
+        e = evalF(&norm);
+        low = true;
+        if (e != FR_OK) return e;
+        exact = true;
+        vaxpby(c, -1.0, F, 1.0, dq, n, s);
       }
+      if ((e = norm2(c, dq, n, &noise->norm, s)) != FR_OK) return e;
     }
-    if (!low && norm <= o->tol * st->norm0) {
+    if (low && (norm <= o->low_above * st->norm0 || (slow && (low32 || norm <= 10.0 * noise->norm)))) {
+      low = false;
+      if (!exact && (e = evalF(&norm)) != FR_OK) return e;
+      exact = true;
+    }
+    if (exact && norm <= o->tol * st->norm0) {
+      low = false;
       st->converged = 1;
       break;
     }
@@ -1712,7 +1730,7 @@ static fr_status stage_impl(fr_ctx* c, const fr_tableau* tab, int32_t stage, dou
 fr_status esdirk_stage(fr_ctx* c, const fr_tableau* tab, int32_t stage, double dt, const double* qn_dev,
                        double* const* Rstages_dev, double* qi_dev, const fr_newton_opts* o,
                        fr_stage_stats* st, void* stream) {
-  double noise = -1.0;
+  DfNoise noise;
   return stage_impl(c, tab, stage, dt, qn_dev, Rstages_dev, qi_dev, o, st, stream, &noise);
 }
 
@@ -1761,7 +1779,8 @@ fr_status esdirk_step(fr_ctx* c, const fr_tableau* tab, double dt, double* q, co
   cudaMemcpyAsync(qi, qn, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
   // stage i starts from the value of stage i-1; the fluxes whose rounding makes
   // the double-float noise are those of one step, so it is measured once
-  double noise = -1.0;
+  DfNoise noise;
+  noise.Rn = Rst[0];
   for (int i = 2; i <= S; ++i) {
     fr_stage_stats st;
     std::memset(&st, 0, sizeof(st));
