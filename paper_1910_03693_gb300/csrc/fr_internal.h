@@ -132,7 +132,7 @@ inline int epb_multi(int nd, int P, int threads = 256) {
 // Element weight of the multi-bucket work table (tuning slot [0][0][P = 1]):
 // 0 n_sp (p+1) (the default), 1 n_sp, 2 n_sp^2, 3 n_sp^3 -- the paper's
 // candidate element weights for repartitioning (Sec. 3.2), reused as CTA
-// work weights for the order in which the persistent launch takes tiles.
+// work weights for the order of the multi-bucket launch's tiles.
 inline double element_weight(int model, int nsp, int P) {
   switch (model) {
     case 1: return (double)nsp;
@@ -155,6 +155,7 @@ struct PcLane {
 
 // The device tables of one layout (layout.cu).
 struct LayoutTables {
+  void* block = nullptr;          // the allocation that holds them
   int32_t* slot_elem = nullptr;   // [E]
   int32_t* elem_slot = nullptr;   // [E] slot of each element
   int64_t* canon_off = nullptr;   // [E] canonical offset of the element at each slot
@@ -259,8 +260,7 @@ struct fr_ctx {
   double* h_red = nullptr;               // pinned host mirror
   frgb::Timing timing;                   // launch counter and optional per-kernel events
   // launch configuration: elements per CTA by [precision][kind][P] (kind 0
-  // trace, 1 volume residual, 2 volume JVP), 0 = default; cost-ordered work
-  // tables of the multi-bucket launch by (precision, kind)
+  // trace, 1 volume residual, 2 volume JVP), 0 = default
   int epb_tab[2][3][frgb::kPM + 1] = {};
   bool multi_launch = true;
   // tile table of the multi-bucket launch (the same for every precision and

@@ -11,7 +11,7 @@
 // nothing is allocated when the degrees change.  Built on the host, with the
 // records' vectors, uploads and one allocation and free a group, one adaptation
 // of 8,000 hexahedra with its way back (two changes of degrees) took 2.96 ms;
-// it takes 0.45 ms, 0.33 ms of it in kernels.
+// it takes 0.43 ms, 0.33 ms of it in kernels.
 #include <algorithm>
 #include <cstring>
 #include <vector>
@@ -334,39 +334,48 @@ static bool get(T** p, size_t bytes) {
 }
 
 void layout_free(LayoutTables& t) {
-  cudaFree(t.slot_elem);
-  cudaFree(t.elem_slot);
-  cudaFree(t.canon_off);
-  cudaFree(t.state_off);
-  cudaFree(t.slot_p);
-  cudaFree(t.recs);
-  cudaFree(t.brecs);
-  cudaFree(t.fnbr);
+  cudaFree(t.block);
   t = LayoutTables{};
 }
 
-// One set of tables but fnbr; all of it or nothing.
-static fr_status tables_alloc(fr_ctx* c, LayoutTables& t) {
-  const int64_t E = c->E;
-  int64_t inner = 0, bnd = 0;
+// One set of tables in one allocation.
+static bool tables_alloc(fr_ctx* c, LayoutTables& t, bool fnbr) {
+  const size_t E = c->E;
+  size_t inner = 0, bnd = 0;
   for (int32_t n : c->nbr) (n >= 0 ? inner : bnd) += 1;
-  if (get(&t.slot_elem, sizeof(int32_t) * E) && get(&t.elem_slot, sizeof(int32_t) * E) &&
-      get(&t.canon_off, sizeof(int64_t) * E) && get(&t.state_off, sizeof(int64_t) * E) && get(&t.slot_p, E) &&
-      get(&t.recs, sizeof(FaceRec) * (inner / 2)) && get(&t.brecs, sizeof(BndRec) * bnd))
-    return FR_OK;
-  cudaGetLastError();
-  layout_free(t);
-  set_error("layout tables: allocation failed");
-  return FR_ERR_NOMEM;
+  const size_t size[8] = {sizeof(int32_t) * E, sizeof(int32_t) * E, sizeof(int64_t) * E, sizeof(int64_t) * E, E,
+                          sizeof(FaceRec) * (inner / 2), sizeof(BndRec) * bnd, fnbr ? sizeof(FusedNbr) * E * c->nf : 0};
+  size_t at[8], end = 0;
+  for (int i = 0; i < 8; ++i) {
+    at[i] = end;
+    end += (size[i] + 255) / 256 * 256;
+  }
+  if (!get(&t.block, end)) {
+    cudaGetLastError();
+    t.block = nullptr;
+    return false;
+  }
+  char* p = static_cast<char*>(t.block);
+  t.slot_elem = reinterpret_cast<int32_t*>(p + at[0]);
+  t.elem_slot = reinterpret_cast<int32_t*>(p + at[1]);
+  t.canon_off = reinterpret_cast<int64_t*>(p + at[2]);
+  t.state_off = reinterpret_cast<int64_t*>(p + at[3]);
+  t.slot_p = reinterpret_cast<int8_t*>(p + at[4]);
+  t.recs = reinterpret_cast<FaceRec*>(p + at[5]);
+  t.brecs = reinterpret_cast<BndRec*>(p + at[6]);
+  t.fnbr = fnbr ? reinterpret_cast<FusedNbr*>(p + at[7]) : nullptr;
+  return true;
 }
 
 // Buffers whose size the mesh decides, and the pinned mirror of what the host reads.
 fr_status layout_alloc(fr_ctx* c) {
   const int64_t E = c->E, ef = E * c->nf;
   const int nb = (int)((E + kSortBlock - 1) / kSortBlock), nfb = (int)((ef + kFaceBlock - 1) / kFaceBlock);
-  const fr_status st = tables_alloc(c, c->lt);
-  if (st != FR_OK) return st;
-  const bool ok = get(&c->d_p, E) && get(&c->d_nbr_face, ef) && get(&c->d_orient, ef) &&
+  // a mesh without boundary faces gets the neighbour table too; without the
+  // memory for it the fused JVP is not offered
+  const bool closed = std::all_of(c->nbr.begin(), c->nbr.end(), [](int32_t n) { return n >= 0; });
+  const bool ok = ((closed && tables_alloc(c, c->lt, true)) || tables_alloc(c, c->lt, false)) && get(&c->d_p, E) &&
+                  get(&c->d_nbr_face, ef) && get(&c->d_orient, ef) &&
                   get(&c->d_lay, sizeof(LayoutMeta) + sizeof(int64_t) * nb + sizeof(int) * 2 * nb * kND) &&
                   get(&c->d_face_hist, sizeof(int) * (size_t)kFaceKeys * nfb) &&
                   cudaMallocHost(&c->h_lay, sizeof(LayoutMeta) + E) == cudaSuccess;
@@ -374,11 +383,6 @@ fr_status layout_alloc(fr_ctx* c) {
     cudaGetLastError();
     set_error("layout tables: allocation failed");
     return FR_ERR_NOMEM;
-  }
-  const bool closed = std::all_of(c->nbr.begin(), c->nbr.end(), [](int32_t n) { return n >= 0; });
-  if (closed && !get(&c->lt.fnbr, sizeof(FusedNbr) * ef)) {    // the fused JVP is then not offered
-    cudaGetLastError();
-    c->lt.fnbr = nullptr;
   }
   if (!get(&c->d_work, sizeof(WorkItem) * (E + 2 * kND))) {    // launches then go per bucket
     cudaGetLastError();
@@ -392,12 +396,7 @@ fr_status layout_alloc(fr_ctx* c) {
 
 // The second set of tables, on the first change of degrees.
 fr_status layout_spare(fr_ctx* c) {
-  if (c->lt_spare.slot_elem) return FR_OK;
-  const fr_status st = tables_alloc(c, c->lt_spare);
-  if (st != FR_OK || !c->lt.fnbr) return st;
-  if (get(&c->lt_spare.fnbr, sizeof(FusedNbr) * (size_t)c->E * c->nf)) return FR_OK;
-  cudaGetLastError();
-  layout_free(c->lt_spare);
+  if (c->lt_spare.block || tables_alloc(c, c->lt_spare, c->lt.fnbr != nullptr)) return FR_OK;
   set_error("layout tables: allocation failed");
   return FR_ERR_NOMEM;
 }
