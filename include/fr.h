@@ -358,10 +358,14 @@ fr_status fr_dfloat_eval(int32_t op, const double* a, const double* b, const dou
  * 625 or 1080 DOFs, by a blocked elimination on the block in global memory:
  * panels of 32 pivots, then one rank-32 update of the other columns); it
  * synchronises `stream`.  Storage: the sum of the squared block sizes in
- * floats (32^3 elements at p = 3: 13.4 GB).  FR_ERR_NONFINITE on a singular block.
+ * floats (32^3 elements at p = 3: 13.4 GB).  Contexts of up to two
+ * full-occupancy waves of solution points (at p_max) probe on four streams and
+ * keep three more FP32 sets of v, J v, traces and face outputs (at most 0.85 GB;
+ * without the memory for them the build runs on one stream).
+ * FR_ERR_NONFINITE on a singular block.
  * Rebucketing or retuning invalidates the blocks.  fr_precond_apply: z =
  * M^-1 w (FP64 state layout, z may alias w).  fr_precond_release frees the
- * block storage. */
+ * block storage and those sets. */
 fr_status fr_precond_build(fr_ctx* ctx, const double* q64_dev, double sigma, void* stream);
 fr_status fr_precond_apply(fr_ctx* ctx, const double* w_dev, double* z_dev, void* stream);
 fr_status fr_precond_release(fr_ctx* ctx);

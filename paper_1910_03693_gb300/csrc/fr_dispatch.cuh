@@ -153,9 +153,7 @@ static inline bool use_multi(fr_ctx* c, int prec, int kind, bool df = false) {
 // Work table of the multi-bucket launch, built when the layout or the tuning
 // changed (rebuild_work_table); never allocated here.  Null when it could not
 // be built: the caller then launches per bucket.
-static const WorkItem* work_items(fr_ctx* c, int prec, int kind, int* n_items) {
-  (void)prec;
-  (void)kind;
+static const WorkItem* work_items(fr_ctx* c, int* n_items) {
   *n_items = c->n_work;
   return c->n_work > 0 ? c->d_work : nullptr;
 }
@@ -240,7 +238,7 @@ static void launch_traces(fr_ctx* c, const T* q, T* trace, cudaStream_t s) {
   }
   const char* name = kname<T>("trace_f64", "trace_f32", "trace_df");
   int n_items = 0;
-  const WorkItem* items = use_multi(c, prec, 0, is_dfloat<T>::value) ? work_items(c, prec, 0, &n_items) : nullptr;
+  const WorkItem* items = use_multi(c, prec, 0, is_dfloat<T>::value) ? work_items(c, &n_items) : nullptr;
   if (items) {
     TraceMulti<T> m;
     size_t smem = 0;
@@ -329,7 +327,7 @@ static void launch_vols(fr_ctx* c, const T* q, const T* v, T* out, cudaStream_t 
     nfl += MODE == 1 ? 0.0 : (double)b.count * nsp_of(ND, P) * flops_volume(ND, P, VISC, DIAG);
   }
   int n_items = 0;
-  const WorkItem* items = use_multi(c, prec, kind, is_dfloat<T>::value) ? work_items(c, prec, kind, &n_items) : nullptr;
+  const WorkItem* items = use_multi(c, prec, kind, is_dfloat<T>::value) ? work_items(c, &n_items) : nullptr;
   if (items) {
     VolMulti<T> m;
     size_t smem = 0;
@@ -638,6 +636,26 @@ static void launch_cface_vt_p(fr_ctx* c, const CFaceArgs<T>& a, cudaStream_t s) 
   }
 }
 
+// arguments of the compact face kernels for one group, traces of q at trq
+template <typename T>
+static CFaceArgs<T> compact_face_args(fr_ctx* c, const FaceGroup& g, const T* trq) {
+  CFaceArgs<T> a;
+  a.gate = c->gate;
+  a.recs = g.d_recs;
+  a.trq = trq;
+  a.trv = nullptr;
+  a.fout = (T*)c->d_fout;
+  a.basis = basis_ptr<T>(c);
+  a.geo = geo_view<T>(c, g.pm);
+  a.gamma = (T)c->phys.gamma;
+  a.mu = (T)c->phys.mu;
+  a.kappa = (T)c->phys.kappa;
+  a.flux = c->phys.flux;
+  a.n = g.n;
+  a.nvt = c->nvt;
+  return a;
+}
+
 template <typename T, int ND, bool VISC, bool DIAG>
 static void jvp_compact_impl(fr_ctx* c, const T* q, const T* v, T* Jv, cudaStream_t s, bool q_traces_ready,
                              double* neg64) {
@@ -651,19 +669,7 @@ static void jvp_compact_impl(fr_ctx* c, const T* q, const T* v, T* Jv, cudaStrea
       const Bucket* bk = nullptr;
       for (const auto& b : c->buckets)
         if (b.p == g.pm) bk = &b;
-      CFaceArgs<T> a;
-      a.gate = c->gate;
-      a.recs = g.d_recs;
-      a.trq = trq;
-      a.fout = (T*)c->d_fout;
-      a.basis = basis_ptr<T>(c);
-      a.geo = geo_view<T>(c, g.pm);
-      a.gamma = (T)c->phys.gamma;
-      a.mu = (T)c->phys.mu;
-      a.kappa = (T)c->phys.kappa;
-      a.flux = c->phys.flux;
-      a.n = g.n;
-      a.nvt = c->nvt;
+      CFaceArgs<T> a = compact_face_args<T>(c, g, trq);
       a.v = v;
       a.state_base = bk->state_base;
       a.trace_base = bk->trace_base;
@@ -687,20 +693,8 @@ static void jvp_compact_impl(fr_ctx* c, const T* q, const T* v, T* Jv, cudaStrea
   }
   launch_ctraces<T, ND, VISC>(c, v, trv, s);
   auto face_args = [&](const FaceGroup& g) {
-    CFaceArgs<T> a;
-    a.gate = c->gate;
-    a.recs = g.d_recs;
-    a.trq = trq;
+    CFaceArgs<T> a = compact_face_args<T>(c, g, trq);
     a.trv = trv;
-    a.fout = (T*)c->d_fout;
-    a.basis = basis_ptr<T>(c);
-    a.geo = geo_view<T>(c, g.pm);
-    a.gamma = (T)c->phys.gamma;
-    a.mu = (T)c->phys.mu;
-    a.kappa = (T)c->phys.kappa;
-    a.flux = c->phys.flux;
-    a.n = g.n;
-    a.nvt = c->nvt;
     return a;
   };
   // both sides' compact traces of q and v in; both sides' face outputs out
@@ -747,26 +741,6 @@ static void jvp_compact_impl(fr_ctx* c, const T* q, const T* v, T* Jv, cudaStrea
     });
   }
   launch_vols<T, ND, VISC, 1, DIAG>(c, q, v, Jv, s, neg64);
-}
-
-// arguments of the compact face kernels for one group, traces of q at trq
-template <typename T>
-static CFaceArgs<T> compact_face_args(fr_ctx* c, const FaceGroup& g, const T* trq) {
-  CFaceArgs<T> a;
-  a.gate = c->gate;
-  a.recs = g.d_recs;
-  a.trq = trq;
-  a.trv = nullptr;
-  a.fout = (T*)c->d_fout;
-  a.basis = basis_ptr<T>(c);
-  a.geo = geo_view<T>(c, g.pm);
-  a.gamma = (T)c->phys.gamma;
-  a.mu = (T)c->phys.mu;
-  a.kappa = (T)c->phys.kappa;
-  a.flux = c->phys.flux;
-  a.n = g.n;
-  a.nvt = c->nvt;
-  return a;
 }
 
 // Traces and faces of the residual: on viscous meshes of axis-aligned elements

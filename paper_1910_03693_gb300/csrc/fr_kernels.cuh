@@ -69,21 +69,6 @@ __device__ __forceinline__ int orient_map(int code, int t, int P, int nd) {
   if ((code & 4) && nd == 3) v = P - 1 - v;
   return u + P * v;
 }
-__device__ __forceinline__ int orient_inv(int code, int uu, int P, int nd) {
-  int u = uu % P, v = uu / P;
-  if (nd == 2) v = 0;
-  if (code & 2) u = P - 1 - u;
-  if ((code & 4) && nd == 3) v = P - 1 - v;
-  int ia, ib;
-  if (nd == 3 && (code & 1)) {
-    ia = v;
-    ib = u;
-  } else {
-    ia = u;
-    ib = v;
-  }
-  return ia + P * ib;
-}
 
 // State value i: for the double-float kernels the state pointer holds the FP64
 // state, converted on load (the FP64 pipe is otherwise idle in those kernels).

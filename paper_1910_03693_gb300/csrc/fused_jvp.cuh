@@ -575,9 +575,10 @@ namespace frgb {
 // compact traces, then this face kernel, then the ordinary volume kernel.  A
 // CTA takes FB faces of one group; both sides' compact traces of q and of v
 // (4 blocks of CT x NFP values a face) are staged in shared memory, each
-// thread forms both sides' physical gradients at its face point from them
-// (face_grad: the stored normal derivative, the tangential ones differentiate
-// the face trace) and evaluates the common flux, the BR2 gradient and the
+// thread forms the common gradient at its face point (general metrics: both
+// sides' physical gradients, face_grad, the stored normal derivative and the
+// tangential ones from the face trace; diagonal metrics: common_gradient, the
+// tangential part from q^com once a face) and evaluates the common flux and the
 // lifting once per face, writing the face outputs of both sides as the
 // trace-gradient face kernel does.  Against that kernel the traces move 2 NV
 // instead of NV (1 + ND) values a face point.
@@ -898,7 +899,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 4 : 2) cface_kernel(CFac
 // 232 -> 218; FP64 traces 613 -> 221, faces 831 -> 829 (the FP64 pipe and, double-
 // float, the FP32 pipe bound both).
 template <typename T, int ND, int P>
-__global__ void __launch_bounds__(128, is_dfloat<T>::value || sizeof(T) == 4 ? 4 : 3) cres_kernel(CFaceArgs<T> a) {
+__global__ void __launch_bounds__(128, is_dfloat<T>::value ? 4 : 3) cres_kernel(CFaceArgs<T> a) {
   constexpr int NV = ND + 2, NFP = ND == 2 ? P : P * P, CT = 2 * NV;
   constexpr int FB = NFP >= 128 ? 1 : 128 / NFP, SC = cface_scratch<ND, P, true, true, 0>();
   __shared__ __align__(16) T sqc[FB * SC];
@@ -1128,7 +1129,8 @@ __global__ void __launch_bounds__(128, 4) cface_tma_kernel(CFaceArgs<T> a, int* 
 // flux step.  Both land on the next tile's barrier, which expects all of its
 // bytes from the start.  One CTA barrier a tile frees the q-trace buffer and
 // the tangent traces; the bounded waits and the error path are those of
-// cface_tma_kernel.  Shared memory: 50 KB for 3D p = 3 (four CTAs an SM).
+// cface_tma_kernel.  Shared memory: 55 KB for 3D p = 3 (four CTAs an SM), 5 KB of
+// it the q^com scratch, which is reserved for general metrics too.
 // ---------------------------------------------------------------------------
 template <typename T, int ND, int P, bool VISC>
 struct CFaceVt {
