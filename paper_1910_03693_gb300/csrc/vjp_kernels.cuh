@@ -454,10 +454,11 @@ __device__ __forceinline__ void face_line_sums(F src, const BasisTab<T>& B, T* f
 }
 
 // DIAG: every metric S is diagonal (see trace_body).
-// FP32: bound by latency between barriers.  Three CTAs an SM for diagonal
-// metrics from p = 2 (box, p = 2 / 3 / 5, 8.6-10.5M DOF: 119 / 124 / 145 us, with
-// two 129 / 135 / 158); two at p = 1 (190, with three 195) and for full metrics,
-// which need the registers (O-grid, p = 1..4: 81 us in all, with three 86).
+// FP32: bound by the L1 data pipe (84 % of it at 20^3, p = 4, a third of the
+// warps, which wait on their loads).  Three CTAs an SM for diagonal metrics from
+// p = 2 (box, p = 2 / 3 / 5, 8.6-10.5M DOF: 119 / 124 / 145 us, with two 129 / 135 /
+// 158); two at p = 1 (190, with three 195) and for full metrics, which need the
+// registers (O-grid, p = 1..4: 81 us in all, with three 86).
 template <typename T, int ND, int P, bool VISC, bool DIAG>
 __global__ void __launch_bounds__(256, sizeof(T) != 4 ? 1 : (DIAG && P > 2 ? 3 : 2)) vol_adj_kernel(VolAdjArgs<T> a, int epb) {
   using Sh = Shape<ND, P>;
